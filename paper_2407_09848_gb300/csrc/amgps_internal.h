@@ -100,6 +100,11 @@ struct StepArgs {
   int split = 1;  // > 1: one block of `split` warps per slice, entries split among them
   // host hint for the scaled form: rin is still unscaled (b)
   bool rin_raw = false;
+  // TMA-fed kernel: whether the next kernel's blocks may start while this one
+  // runs.  Only another TMA-fed step gains by it: a kernel that works through
+  // L1 would start under this kernel's shared-memory carve-out, which an SM
+  // that is never idle keeps.
+  bool go = true;
 };
 
 // Most warps per slice in the split form of the step and transfer kernels

@@ -689,6 +689,7 @@ struct Engine {
         a.xin = U[q & 1];  // u_{j+2}
         a.c1 = XT(st[q].g);
       }
+      a.go = j > 1 || xzero;  // after the pre-smoother comes the residual step
       const int nvec = 2 + (a.rin ? 1 : 0) + (a.xin ? 1 : 0);
       const bool s0 = a.rin != nullptr, s1 = a.xin != nullptr;
       ProfScope ps(c, profl, 0, step_bytes<VT, XT>(L, nvec),
@@ -738,6 +739,7 @@ struct Engine {
         a.dinv = md;
         a.fam = FAM_JAC;
         a.init = true;
+        a.go = j < k - 1 || xzero;
         ProfScope ps(c, profl, 0, step_bytes<VT, XT>(L, 4), step_flops(L, FAM_JAC, false, false),
                      step_inst(L, FAM_JAC, false, false));
         run_step(c, L, a, s);
@@ -775,6 +777,7 @@ struct Engine {
       a.rhoinv = XT(cf.rhoinv);
       a.fam = cf.fam;
       a.init = true;
+      a.go = k > 1;
       ProfScope ps(c, profl, 0, step_bytes<VT, XT>(L, a.write_r ? 6 : 5),
                    step_flops(L, cf.fam, false, true), step_inst(L, cf.fam, false, true));
       run_step(c, L, a, s);
@@ -806,6 +809,7 @@ struct Engine {
       a.fam = cf.fam;
       a.init = false;
       a.rin_raw = (rin_next == b);  // first step after k_first: r_0 = b
+      a.go = j < k - 1 || xzero;
       // streams: z_j, r in(/out), z_{j+1}, x in/out, and 1/M unless scaled
       const bool no_dinv = L.sval && ((cf.fam == FAM_CHEB4 && !a.rin_raw) || cf.fam == FAM_CHEB1);
       const bool raw = a.rin_raw && cf.fam == FAM_CHEB4;
@@ -871,6 +875,7 @@ struct Engine {
       a.zout = (XT*)L.r;
       a.fam = FAM_RES;
       a.init = true;
+      a.go = false;
       run_step(c, L, a, s);
       if (L.xfer_general) launch_xfer<XT>(L.Rm, (const XT*)L.r, (XT*)C.b, 0, L.rsplit, s);
       else do_aggregate(L, (const XT*)L.r, (XT*)C.b, s);
@@ -935,6 +940,7 @@ struct Engine {
       a.beta = XT(0);
       a.fam = FAM_CHEB4;
       a.init = true;
+      a.go = false;
       run_step(c, L, a, s);
       rin_next = r;
     }
@@ -955,6 +961,7 @@ struct Engine {
       a.c2 = XT(cf.c2[j + 1]);
       a.beta = XT(0);
       a.fam = FAM_CHEB4;
+      a.go = false;
       a.rin_raw = (rin_next == b);
       run_step(c, L, a, s);
       launch_dot(n, (const double*)gx, (const double*)zn, rw, c->ddots, slot0 + j, 0, s);
@@ -977,6 +984,7 @@ struct Engine {
       a.zout = gx0;
       a.fam = FAM_RES;
       a.init = true;
+      a.go = false;
       run_step(c, L, a, c->stream);
     }
     if (slot0 >= 0 && cf.fam == FAM_CHEB4) zdots(c, l, cf, b, x0, gx, slot0);
@@ -1015,6 +1023,7 @@ struct Engine {
       a.zout = t1;
       a.fam = FAM_RES;
       a.init = true;
+      a.go = false;
       run_step(c, L, a, s);
     }
     // pre-smoother x1 = S(b, 0)

@@ -1,6 +1,8 @@
 // Device helpers shared by the kernel translation units.
 #pragma once
 
+#include <utility>
+
 #include "amgps_internal.h"
 
 namespace amgps {
@@ -18,88 +20,136 @@ __device__ __forceinline__ float ldval(const __nv_bfloat16* p) {
 template <class T>
 __device__ __forceinline__ T absv(T v) { return v < T(0) ? -v : v; }
 
-// Load of a vector entry.  CG = false: a plain load, or for the gathered
-// operand of a product the read-only path (__ldg), which is valid in kernels
-// whose launch does not write that vector.  CG = true: an L2 (coherent) load,
-// for the persistent kernel that reads in one phase what other blocks wrote in
-// an earlier phase of the same launch.
+// ---- programmatic dependent launch ----
+// The kernels of a V-cycle and of the outer solver are launched so that their
+// blocks may start while the previous kernel of the stream still runs
+// (launch_dep below).  pdl_wait() returns when that kernel has finished and
+// its writes are visible; before it a kernel may only read what no kernel of
+// the chain writes -- the matrix arrays, the aggregate maps, 1/M -- and may
+// write nothing.  pdl_go() lets the next kernel's blocks start; it comes
+// after the wait, so at most two kernels of a chain overlap.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_go() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Load of a vector entry.  CG = false: a plain cached load, issued where it
+// stands (volatile: neither the compiler nor the read-only path may move it
+// before pdl_wait).  CG = true: an L2 (coherent) load, for the persistent
+// kernel that reads in one phase what other blocks wrote in an earlier phase
+// of the same launch.
+__device__ __forceinline__ double ldg_ca(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ float ldg_ca(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
 template <bool CG, class T>
 __device__ __forceinline__ T ldv(const T* p) {
   if constexpr (CG) return __ldcg(p);
-  else return *p;
-}
-template <bool CG, class T>
-__device__ __forceinline__ T ldu(const T* p) {
-  if constexpr (CG) return __ldcg(p);
-  else return __ldg(p);
+  else return ldg_ca(p);
 }
 
-// init + SIGN * (A u)_row from one pass over the row (SIGN = +1 or -1, so a
-// residual b - A u comes out of the same multiply-adds).  `lane` is the row's
-// position in slice `s`.  Rows past n (tail of the last slice) see only zero
-// padding and clamped, in-range columns.  FP64 arithmetic is the scarce
-// resource on this GPU (its FP64 pipe issues about 2 FMAs per clock per SM),
-// so the row costs exactly one multiply-add per stored entry and nothing else.
-// Entries k in [k0, k1) of row `row` of slice s: init + SIGN * sum a_k u_{c_k}.
-template <int SIGN, class VT, class XT, bool CG = false>
-__device__ __forceinline__ XT row_spmv_range(const DevMat<VT>& A, int64_t s, int lane, int64_t row,
-                                             const XT* __restrict__ u, XT init, int k0, int k1) {
-  const SliceDesc d = A.sd[s];
+// Slice descriptor (constant while any kernel runs): one 16-byte load.
+__device__ __forceinline__ SliceDesc ld_desc(const SliceDesc* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  SliceDesc d;
+  d.vbase = (int64_t)(uint32_t)v.x | ((int64_t)v.y << 32);
+  d.w = v.z;
+  d.cref = v.w;
+  return d;
+}
+
+// init() + SIGN * (A u)_row over the entries k in [k0, k1) of row `row`
+// (position `lane` in slice `s`), in storage order (SIGN = +1 or -1, so a
+// residual b - A u comes out of the same multiply-adds).  Rows past n (tail
+// of the last slice) see only zero padding and clamped, in-range columns.
+// FP64 arithmetic is the scarce resource on this GPU (its FP64 pipe issues
+// about 2 FMAs per clock per SM), so the row costs exactly one multiply-add
+// per stored entry and nothing else.
+// WAIT: the kernel's pdl_wait() / pdl_go() happen here, after the first
+// entries of the row (values and columns) are on their way and before
+// init(), which loads the row's own vector entries: what a dependent launch
+// still has to wait for is then one round of vector loads.  On the levels of a
+// few thousand rows, where a kernel is three dependent loads long, that is
+// most of its time.  Rows of other lengths go NB entries at a time; PIPE (the
+// kernels of wide rows): the next NB values and columns are fetched while the
+// current products are formed.
+template <int SIGN, class VT, class XT, bool CG, bool WAIT, int NB, bool PIPE, class Init>
+__device__ __forceinline__ XT row_accumulate(const DevMat<VT>& A, const SliceDesc d, int lane,
+                                             int64_t row, const XT* u, Init init, int k0, int k1) {
   const int64_t nm1 = A.n - 1;
-  XT t = init;
+  auto fetch = [&](int k, XT& av, int32_t& cv) {
+    const int64_t e = d.vbase + (int64_t)k * kSlice + lane;
+    av = XT(ldval(A.val + e));
+    if (d.cref >= 0) {
+      const int64_t cc = row + (int64_t)__ldg(A.off + d.cref + k);
+      cv = (int32_t)(cc < 0 ? 0 : (cc > nm1 ? nm1 : cc));
+    } else {
+      cv = __ldg(A.col + e);
+    }
+  };
   if (k1 - k0 == 7) {
     // the seven entries of a 7-point row without guards: on GB300's narrow
     // FP64 pipe a predicated-off multiply-add still takes an issue slot
     // (same operations in the same order as the general loop below)
-    XT a[7];
-    int64_t c[7];
+    XT a[7], uv[7];
+    int32_t c[7];
 #pragma unroll
-    for (int kk = 0; kk < 7; ++kk) {
-      const int k = k0 + kk;
-      const int64_t e = d.vbase + (int64_t)k * kSlice + lane;
-      a[kk] = XT(ldval(A.val + e));
-      if (d.cref >= 0) {
-        const int64_t cc = row + (int64_t)A.off[d.cref + k];
-        c[kk] = cc < 0 ? 0 : (cc > nm1 ? nm1 : cc);
-      } else {
-        c[kk] = A.col[e];
-      }
+    for (int kk = 0; kk < 7; ++kk) fetch(k0 + kk, a[kk], c[kk]);
+    if constexpr (WAIT) {
+      pdl_wait();
+      pdl_go();
     }
+    XT t = init();
 #pragma unroll
-    for (int kk = 0; kk < 7; ++kk) t = fma(SIGN > 0 ? a[kk] : -a[kk], ldu<CG>(u + c[kk]), t);
+    for (int kk = 0; kk < 7; ++kk) uv[kk] = ldv<CG>(u + c[kk]);
+#pragma unroll
+    for (int kk = 0; kk < 7; ++kk) t = fma(SIGN > 0 ? a[kk] : -a[kk], uv[kk], t);
     return t;
   }
-  for (int kb = k0; kb < k1; kb += 8) {
-    XT a[8];
-    int64_t c[8];
+  XT a[NB];
+  int32_t c[NB];
+  auto fetch_batch = [&](int kb) {
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      const int k = kb + kk;
-      a[kk] = XT(0);
-      c[kk] = 0;
-      if (k < k1) {
-        const int64_t e = d.vbase + (int64_t)k * kSlice + lane;
-        a[kk] = XT(ldval(A.val + e));
-        if (d.cref >= 0) {
-          int64_t cc = row + (int64_t)A.off[d.cref + k];
-          c[kk] = cc < 0 ? 0 : (cc > nm1 ? nm1 : cc);
-        } else {
-          c[kk] = A.col[e];
-        }
-      }
+    for (int kk = 0; kk < NB; ++kk)
+      if (kb + kk < k1) fetch(kb + kk, a[kk], c[kk]);
+  };
+  fetch_batch(k0);
+  if constexpr (WAIT) {
+    pdl_wait();
+    pdl_go();
+  }
+  XT t = init();
+  for (int kb = k0; kb < k1; kb += NB) {
+    XT av[NB], uv[NB];
+#pragma unroll
+    for (int kk = 0; kk < NB; ++kk) {
+      if (kb + kk < k1) uv[kk] = ldv<CG>(u + c[kk]);
+      av[kk] = a[kk];
     }
+    if (PIPE && kb + NB < k1) fetch_batch(kb + NB);
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk)
-      if (kb + kk < k1) t = fma(SIGN > 0 ? a[kk] : -a[kk], ldu<CG>(u + c[kk]), t);
+    for (int kk = 0; kk < NB; ++kk)
+      if (kb + kk < k1) t = fma(SIGN > 0 ? av[kk] : -av[kk], uv[kk], t);
+    if (!PIPE && kb + NB < k1) fetch_batch(kb + NB);
   }
   return t;
 }
 
 // The whole row: entries 0 .. w-1 of the slice.
-template <int SIGN, class VT, class XT, bool CG = false>
+template <int SIGN, class VT, class XT>
 __device__ __forceinline__ XT row_spmv(const DevMat<VT>& A, int64_t s, int lane, int64_t row,
-                                       const XT* __restrict__ u, XT init) {
-  return row_spmv_range<SIGN, VT, XT, CG>(A, s, lane, row, u, init, 0, A.sd[s].w);
+                                       const XT* u, XT init) {
+  const SliceDesc d = ld_desc(A.sd + s);
+  return row_accumulate<SIGN, VT, XT, false, false, 4, false>(
+      A, d, lane, row, u, [&] { return init; }, 0, d.w);
 }
 
 // The SpMV of one smoother step is accumulated as init + SIGN * (A u):
@@ -187,34 +237,45 @@ __device__ __forceinline__ void step_finish(const StepArgs<VT, XT>& a, int64_t r
 }
 
 // One smoother step on the 32 rows of slice s, one row per lane, operands
-// read from global memory (the direct form of the step).
-template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN, bool CG = false>
+// read from global memory (the direct form of the step).  WAIT: see
+// row_accumulate (1/M is fetched before the wait as well).
+template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN, bool CG = false,
+          bool WAIT = false>
 __device__ __forceinline__ void step_slice(const StepArgs<VT, XT>& a, int64_t s, int lane) {
   const int64_t row = s * kSlice + lane;
   const bool live = row < a.A.n;
+  const SliceDesc d = ld_desc(a.A.sd + s);
+  constexpr int kSign = StepForm<FAM, INIT>::kSign;
   if constexpr (is_op(FAM)) {
-    XT s0 = XT(0), s1 = XT(0), uc = XT(0);
-    if (live) {
-      if (reads_slot0<FAM, INIT>()) s0 = ldv<CG>(a.rin + row);
-      if (reads_slot1<FAM, ZOWN>()) s1 = ldv<CG>(a.xin + row);
-      if (FAM == FAM_OPT && WR) uc = ldv<CG>(a.u + row);
-    }
-    constexpr int kSign = StepForm<FAM, INIT>::kSign;
-    const XT acc = row_spmv<kSign, VT, XT, CG>(a.A, s, lane, row, a.u,
-                                               op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, s0, s1));
+    XT uc = XT(0);
+    const XT acc = row_accumulate<kSign, VT, XT, CG, WAIT, sizeof(XT) == 8 ? 4 : 8, false>(
+        a.A, d, lane, row, a.u,
+        [&] {
+          XT s0 = XT(0), s1 = XT(0);
+          if (live) {
+            if (reads_slot0<FAM, INIT>()) s0 = ldv<CG>(a.rin + row);
+            if (reads_slot1<FAM, ZOWN>()) s1 = ldv<CG>(a.xin + row);
+            if (FAM == FAM_OPT && WR) uc = ldv<CG>(a.u + row);
+          }
+          return op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, s0, s1);
+        },
+        0, d.w);
     if (live) op_finish<VT, XT, FAM, WR>(a, row, acc, uc);
     return;
   }
   XT rin = XT(0), xin = XT(0), zo = XT(0), di = XT(0);
-  if (live) {
-    rin = ldv<CG>(a.rin + row);
-    if (FAM != FAM_RES) xin = ldv<CG>(a.xin + row);
-    if (step_needs_dinv<FAM>()) di = a.dinv[row];  // formed at set-up, never written here
-    if (ZOWN) zo = ldv<CG>(a.zown + row);
-  }
-  using F = StepForm<FAM, INIT>;
-  const XT acc = row_spmv<F::kSign, VT, XT, CG>(a.A, s, lane, row, a.u,
-                                                 step_init<FAM, F::kResidual>(rin, di));
+  if (live && step_needs_dinv<FAM>()) di = __ldg(a.dinv + row);  // formed at set-up
+  const XT acc = row_accumulate<kSign, VT, XT, CG, WAIT, sizeof(XT) == 8 ? 4 : 8, false>(
+      a.A, d, lane, row, a.u,
+      [&] {
+        if (live) {
+          rin = ldv<CG>(a.rin + row);
+          if (FAM != FAM_RES) xin = ldv<CG>(a.xin + row);
+          if (ZOWN) zo = ldv<CG>(a.zown + row);
+        }
+        return step_init<FAM, StepForm<FAM, INIT>::kResidual>(rin, di);
+      },
+      0, d.w);
   if (!live) return;
   step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, row, acc, rin, xin, di, zo);
 }
@@ -223,14 +284,14 @@ __device__ __forceinline__ void step_slice(const StepArgs<VT, XT>& a, int64_t s,
 // launches (kernels_smooth.cu, kernels_krylov.cu) and by the persistent
 // coarse-level kernel (kernels_cycle.cu), so both give the same bits.
 
-// First step from x = 0 (no product with A), row i:
+// First step from x = 0 (no product with A), row i, with di = 1/M_i:
 //   4th kind: z_1 = c2 M^{-1} b, x = beta_1 z_1 (r_0 = b is not copied)
 //   1st kind: r^(0) = (1/rho) M^{-1} b, d^(0) = r^(0)/theta, x = d^(0)
 //   Jacobi:   x = M^{-1} b
 template <class XT, int FAM, bool CG = false>
-__device__ __forceinline__ void first_row(int64_t i, const XT* b, const XT* dinv, XT* rout,
-                                          XT* zout, XT* xout, XT c2, XT beta, XT rhoinv) {
-  const XT bm = ldv<CG>(b + i) * dinv[i];
+__device__ __forceinline__ void first_row(int64_t i, const XT* b, XT di, XT* rout, XT* zout,
+                                          XT* xout, XT c2, XT beta, XT rhoinv) {
+  const XT bm = ldv<CG>(b + i) * di;
   if constexpr (FAM == FAM_CHEB4) {
     const XT z = c2 * bm;
     zout[i] = z;
@@ -246,30 +307,69 @@ __device__ __forceinline__ void first_row(int64_t i, const XT* b, const XT* dinv
   }
 }
 
-// b_c[I] = sum of res over the children of coarse row I, in list order
-template <class XT, bool CG = false>
+// b_c[I] = sum of res over the children of coarse row I, in list order.  The
+// first eight children (all of a 2x2x2 block) are looked up before the wait
+// and loaded together.
+template <class XT, bool CG = false, bool WAIT = false>
 __device__ __forceinline__ void aggregate_row(int64_t I, const int32_t* cptr, const int32_t* cidx,
                                               const XT* res, XT* bc) {
+  const int q0 = __ldg(cptr + I), q1 = __ldg(cptr + I + 1);
+  int32_t c[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (q0 + k < q1) c[k] = __ldg(cidx + q0 + k);
+  if constexpr (WAIT) {
+    pdl_wait();
+    pdl_go();
+  }
+  XT v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (q0 + k < q1) v[k] = ldv<CG>(res + c[k]);
   XT acc = XT(0);
-  const int q1 = cptr[I + 1];
-  for (int q = cptr[I]; q < q1; ++q) acc += ldv<CG>(res + cidx[q]);
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (q0 + k < q1) acc += v[k];
+  for (int q = q0 + 8; q < q1; ++q) acc += ldv<CG>(res + __ldg(cidx + q));
   bc[I] = acc;
 }
 
 // x_i += e_c[agg_i]
-template <class XT, bool CG = false>
+template <class XT, bool CG = false, bool WAIT = false>
 __device__ __forceinline__ void prolong_row(int64_t i, const int32_t* agg, const XT* ec, XT* x) {
-  x[i] = ldv<CG>(x + i) + ldv<CG>(ec + agg[i]);
+  const int32_t c = __ldg(agg + i);
+  if constexpr (WAIT) {
+    pdl_wait();
+    pdl_go();
+  }
+  const XT xi = ldv<CG>(x + i);
+  x[i] = xi + ldv<CG>(ec + c);
 }
 
 // x_i = (A_c^{-1} b)_i for the coarsest level, one warp per row: lane l sums
-// columns l, l + 32, ... in order, then a fixed butterfly adds the lanes
-template <class XT, bool CG = false>
+// columns l, l + 32, ... in order, then a fixed butterfly adds the lanes.  The
+// first 16 entries of a lane (512 columns) are loaded together, before the wait.
+template <class XT, bool CG = false, bool WAIT = false>
 __device__ __forceinline__ void coarse_gemv_row(int i, int nc, const double* ainv, const XT* b,
                                                 XT* x, int lane) {
   const double* row = ainv + (size_t)i * nc;
+  double av[16];
+  XT bv[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    if (lane + 32 * k < nc) av[k] = __ldg(row + lane + 32 * k);
+  if constexpr (WAIT) {
+    pdl_wait();
+    pdl_go();
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    if (lane + 32 * k < nc) bv[k] = ldv<CG>(b + lane + 32 * k);
   double acc = 0.0;
-  for (int j = lane; j < nc; j += 32) acc = fma(row[j], (double)ldv<CG>(b + j), acc);
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    if (lane + 32 * k < nc) acc = fma(av[k], (double)bv[k], acc);
+  for (int j = lane + 512; j < nc; j += 32) acc = fma(__ldg(row + j), (double)ldv<CG>(b + j), acc);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) x[i] = XT(acc);
@@ -318,6 +418,27 @@ __device__ __forceinline__ void grid_sum(double v, const RedWork& w, Fin fin) {
       *w.counter = 0u;
     }
   }
+}
+
+// Launch of a kernel that calls pdl_wait() as the programmatic dependent of
+// the kernel before it on stream s (in a captured graph: a programmatic
+// edge).  Behind anything but a kernel (a copy, a memset, an event) it is an
+// ordinary launch.
+template <class... P, class... A>
+void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  count_launch();
 }
 
 }  // namespace amgps

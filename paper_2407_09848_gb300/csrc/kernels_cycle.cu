@@ -130,13 +130,13 @@ __global__ void __launch_bounds__(kCycleThreads, kCycleMaxBlocksPerSm)
       case CY_FIRST:
         for (int64_t i = gt; i < P.n; i += nt) {
           if (P.fam == FAM_CHEB4)
-            first_row<XT, FAM_CHEB4, true>(i, P.in0, P.in1, P.out0, P.out1, P.out2, P.c2, P.beta,
+            first_row<XT, FAM_CHEB4, true>(i, P.in0, __ldg(P.in1 + i), P.out0, P.out1, P.out2, P.c2, P.beta,
                                            P.rhoinv);
           else if (P.fam == FAM_CHEB1)
-            first_row<XT, FAM_CHEB1, true>(i, P.in0, P.in1, P.out0, P.out1, P.out2, P.c2, P.beta,
+            first_row<XT, FAM_CHEB1, true>(i, P.in0, __ldg(P.in1 + i), P.out0, P.out1, P.out2, P.c2, P.beta,
                                            P.rhoinv);
           else
-            first_row<XT, FAM_JAC, true>(i, P.in0, P.in1, P.out0, P.out1, P.out2, P.c2, P.beta,
+            first_row<XT, FAM_JAC, true>(i, P.in0, __ldg(P.in1 + i), P.out0, P.out1, P.out2, P.c2, P.beta,
                                          P.rhoinv);
         }
         break;

@@ -23,11 +23,15 @@ int reduction_grid(int64_t work_items, int nsm, int per_sm) {
   return (int)g;
 }
 
+// Entries a thread of the streaming reductions loads before it uses any.
+constexpr int kLoads = 4;
+
 // q = A p and p.q (S_PQ).  One warp per slice, grid-stride over slices.
-__global__ void __launch_bounds__(kBlock) k_spmv_dot(const DevMat<double> A,
-                                                     const double* __restrict__ p,
-                                                     double* __restrict__ q, const RedWork w,
+__global__ void __launch_bounds__(kBlock, 4) k_spmv_dot(const DevMat<double> A,
+                                                     const double* p, double* q, const RedWork w,
                                                      double* scal) {
+  pdl_wait();
+  pdl_go();
   const int lane = threadIdx.x & 31;
   const int64_t nw = (int64_t)gridDim.x * kWarpsPerBlock;
   double acc = 0.0;
@@ -37,7 +41,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_dot(const DevMat<double> A,
     const double t = row_spmv<1, double, double>(A, s, lane, row, p, 0.0);
     if (row < A.n) {
       q[row] = t;
-      acc = fma(p[row], t, acc);
+      acc = fma(ldv<false>(p + row), t, acc);
     }
   }
   grid_sum(acc, w, [&](double tot) {
@@ -48,8 +52,7 @@ __global__ void __launch_bounds__(kBlock) k_spmv_dot(const DevMat<double> A,
 
 void launch_spmv_dot(const DevMat<double>& A, const double* p, double* q, const RedWork& w,
                      double* scal, cudaStream_t s) {
-  k_spmv_dot<<<w.grid, kBlock, 0, s>>>(A, p, q, w, scal);
-  count_launch();
+  launch_dep(k_spmv_dot, w.grid, kBlock, 0, s, A, p, q, w, scal);
 }
 
 // Three sums in one pass (the one-reduction flexible CG): partials are laid
@@ -94,12 +97,12 @@ __device__ __forceinline__ void grid_sum3(double v0, double v1, double v2, const
 // grid reduction.  The last block forms beta = gamma / eta_old (the
 // A-orthogonalisation of z against p_old), eta = p.A p = delta - beta gamma
 // (by symmetry of A, with q = A p), and alpha = rho / eta.
-__global__ void __launch_bounds__(kBlock) k_spmv_dot3(const DevMat<double> A,
-                                                      const double* __restrict__ z,
-                                                      double* __restrict__ w,
-                                                      const double* __restrict__ r,
-                                                      const double* __restrict__ q, int first,
-                                                      const RedWork rw, double* scal) {
+__global__ void __launch_bounds__(kBlock, 4) k_spmv_dot3(const DevMat<double> A,
+                                                      const double* z, double* w, const double* r,
+                                                      const double* q, int first, const RedWork rw,
+                                                      double* scal) {
+  pdl_wait();
+  pdl_go();
   const int lane = threadIdx.x & 31;
   const int64_t nw = (int64_t)gridDim.x * kWarpsPerBlock;
   double zr = 0.0, zq = 0.0, zw = 0.0;
@@ -109,10 +112,10 @@ __global__ void __launch_bounds__(kBlock) k_spmv_dot3(const DevMat<double> A,
     const double t = row_spmv<1, double, double>(A, s, lane, row, z, 0.0);
     if (row < A.n) {
       w[row] = t;
-      const double zi = z[row];
+      const double zi = ldv<false>(z + row);
       zw = fma(zi, t, zw);
-      zr = fma(zi, r[row], zr);
-      if (!first) zq = fma(zi, q[row], zq);
+      zr = fma(zi, ldv<false>(r + row), zr);
+      if (!first) zq = fma(zi, ldv<false>(q + row), zq);
     }
   }
   grid_sum3(zr, zq, zw, rw, [&](double rho, double gam, double del) {
@@ -130,20 +133,20 @@ __global__ void __launch_bounds__(kBlock) k_spmv_dot3(const DevMat<double> A,
 void launch_spmv_dot3(const DevMat<double>& A, const double* z, double* w, const double* r,
                       const double* q, int first, const RedWork& rw, double* scal,
                       cudaStream_t s) {
-  k_spmv_dot3<<<rw.grid, kBlock, 0, s>>>(A, z, w, r, q, first, rw, scal);
-  count_launch();
+  launch_dep(k_spmv_dot3, rw.grid, kBlock, 0, s, A, z, w, r, q, first, rw, scal);
 }
 
 // p = z - beta p, q = w - beta q (first: p = z, q = w), x += alpha p,
 // r -= alpha q, r.r (S_RR)
-__global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* __restrict__ z,
-                                                       const double* __restrict__ w,
-                                                       double* __restrict__ p,
+__global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* z,
+                                                       const double* w, double* __restrict__ p,
                                                        double* __restrict__ q,
                                                        double* __restrict__ x,
                                                        double* __restrict__ r, int first,
                                                        const RedWork rw, double* scal) {
-  const double alpha = scal[S_ALPHA], beta = scal[S_BETA];
+  pdl_wait();
+  pdl_go();
+  const double alpha = ldv<false>(scal + S_ALPHA), beta = ldv<false>(scal + S_BETA);
   double acc = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * kBlock) {
@@ -162,8 +165,7 @@ __global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* 
 void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, double* q,
                        double* x, double* r, int first, const RedWork& rw, double* scal,
                        cudaStream_t s) {
-  k_fcg_update<<<rw.grid, kBlock, 0, s>>>(n, z, w, p, q, x, r, first, rw, scal);
-  count_launch();
+  launch_dep(k_fcg_update, rw.grid, kBlock, 0, s, n, z, w, p, q, x, r, first, rw, scal);
 }
 
 // r -= alpha q ; r.r (S_RR).  The x update of the same iteration is deferred
@@ -171,58 +173,81 @@ void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, d
 // stored-operator smoother of the next V-cycle starts from, same operation
 // as its own c pass).
 template <bool WC>
-__global__ void __launch_bounds__(kBlock) k_r_update(int64_t n, const double* __restrict__ q,
-                                                     double* __restrict__ r, const RedWork w,
-                                                     double* scal, const double* __restrict__ dinv,
-                                                     double* __restrict__ cout) {
-  const double alpha = scal[S_ALPHA];
+__global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n, const double* q, double* r,
+                                                     const RedWork w, double* scal,
+                                                     const double* __restrict__ dinv,
+                                                     double* cout) {
+  pdl_wait();
+  pdl_go();
+  const double alpha = ldv<false>(scal + S_ALPHA);
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * kBlock) {
-    const double ri = fma(-alpha, q[i], r[i]);
+  const uint32_t m = (uint32_t)n, step = gridDim.x * kBlock;  // n < 2^31: i + 2 step fits
+  auto one = [&](uint32_t i, double qi, double ri) {
+    ri = fma(-alpha, qi, ri);
     r[i] = ri;
-    if constexpr (WC) cout[i] = ri * dinv[i];
+    if constexpr (WC) cout[i] = ri * __ldg(dinv + i);
     acc = fma(ri, ri, acc);
+  };
+  uint32_t i = blockIdx.x * kBlock + threadIdx.x;
+  for (; i + step < m; i += 2 * step) {
+    const double q0 = ldv<false>(q + i), r0 = ldv<false>(r + i);
+    const double q1 = ldv<false>(q + i + step), r1 = ldv<false>(r + i + step);
+    one(i, q0, r0);
+    one(i + step, q1, r1);
   }
+  if (i < m) one(i, ldv<false>(q + i), ldv<false>(r + i));
   grid_sum(acc, w, [&](double tot) { scal[S_RR] = tot; });
 }
 
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
                      cudaStream_t s, const double* dinv, double* cout) {
-  if (cout)
-    k_r_update<true><<<w.grid, kBlock, 0, s>>>(n, q, r, w, scal, dinv, cout);
-  else
-    k_r_update<false><<<w.grid, kBlock, 0, s>>>(n, q, r, w, scal, nullptr, nullptr);
-  count_launch();
+  launch_dep(cout ? k_r_update<true> : k_r_update<false>, w.grid, kBlock, 0, s, n, q, r, w, scal,
+             dinv, cout);
 }
 
 // x += alpha p with the previous alpha, then p = z + beta p (x_beta = 1), or
 // only x += alpha p (x_beta = 0: the last iteration)
-__global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const double* __restrict__ z,
-                                                   double* __restrict__ p, double* __restrict__ x,
-                                                   const double* __restrict__ scal, int with_p) {
-  const double alpha = scal[S_ALPHA], beta = scal[S_BETA];
+__global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const double* z, double* p,
+                                                   double* x, const double* scal, int with_p) {
+  pdl_wait();
+  pdl_go();
+  const double alpha = ldv<false>(scal + S_ALPHA), beta = ldv<false>(scal + S_BETA);
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (i >= n) return;
-  const double pi = p[i];
-  x[i] = fma(alpha, pi, x[i]);
-  if (with_p) p[i] = fma(beta, pi, z[i]);
+  const double pi = ldv<false>(p + i), xi = ldv<false>(x + i);
+  const double zi = with_p ? ldv<false>(z + i) : 0.0;
+  x[i] = fma(alpha, pi, xi);
+  if (with_p) p[i] = fma(beta, pi, zi);
 }
 
 void launch_xpay_x(int64_t n, const double* z, double* p, double* x, const double* scal,
                    int with_p, cudaStream_t s) {
   if (n == 0) return;
-  k_xpay_x<<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, z, p, x, scal, with_p);
-  count_launch();
+  launch_dep(k_xpay_x, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, z, p, x, scal,
+             with_p);
 }
 
-__global__ void __launch_bounds__(kBlock) k_dot(int64_t n, const double* __restrict__ a,
-                                                const double* __restrict__ b, const RedWork w,
-                                                double* scal, int slot, int rz_shift) {
+__global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, const double* a, const double* b,
+                                                const RedWork w, double* scal, int slot,
+                                                int rz_shift) {
+  pdl_wait();
+  pdl_go();
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * kBlock)
-    acc = fma(a[i], b[i], acc);
+  const int64_t step = (int64_t)gridDim.x * kBlock;
+  for (int64_t i0 = (int64_t)blockIdx.x * kBlock + threadIdx.x; i0 < n; i0 += kLoads * step) {
+    double av[kLoads], bv[kLoads];
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+      const int64_t i = i0 + k * step;
+      if (i < n) {
+        av[k] = ldv<false>(a + i);
+        bv[k] = ldv<false>(b + i);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k)
+      if (i0 + k * step < n) acc = fma(av[k], bv[k], acc);
+  }
   grid_sum(acc, w, [&](double tot) {
     if (rz_shift) {
       scal[S_RZOLD] = scal[S_RZ];
@@ -236,56 +261,54 @@ __global__ void __launch_bounds__(kBlock) k_dot(int64_t n, const double* __restr
 
 void launch_dot(int64_t n, const double* a, const double* b, const RedWork& w, double* scal,
                 int out_slot, int rz_mode, cudaStream_t s) {
-  k_dot<<<w.grid, kBlock, 0, s>>>(n, a, b, w, scal, out_slot, rz_mode);
-  count_launch();
+  launch_dep(k_dot, w.grid, kBlock, 0, s, n, a, b, w, scal, out_slot, rz_mode);
 }
 
-__global__ void __launch_bounds__(kBlock) k_sub(int64_t n, const double* __restrict__ x,
-                                                const double* __restrict__ y,
-                                                double* __restrict__ out) {
+__global__ void __launch_bounds__(kBlock) k_sub(int64_t n, const double* x, const double* y,
+                                                double* out) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (i < n) out[i] = x[i] - y[i];
+  pdl_wait();
+  pdl_go();
+  if (i < n) out[i] = ldv<false>(x + i) - ldv<false>(y + i);
 }
 
 void launch_sub(int64_t n, const double* x, const double* y, double* out, cudaStream_t s) {
   if (n == 0) return;
-  k_sub<<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, x, y, out);
-  count_launch();
+  launch_dep(k_sub, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, x, y, out);
 }
 
-__global__ void __launch_bounds__(kBlock) k_scale_dev(int64_t n, const double* __restrict__ x,
-                                                      double* __restrict__ out,
-                                                      const double* __restrict__ sd,
-                                                      double factor) {
-  const double f = factor / sd[0];
+__global__ void __launch_bounds__(kBlock) k_scale_dev(int64_t n, const double* x, double* out,
+                                                      const double* sd, double factor) {
+  pdl_wait();
+  pdl_go();
+  const double f = factor / ldv<false>(sd);
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (i < n) out[i] = f * x[i];
+  if (i < n) out[i] = f * ldv<false>(x + i);
 }
 
 void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, double factor,
                       cudaStream_t s) {
   if (n == 0) return;
-  k_scale_dev<<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, x, out, s_dev, factor);
-  count_launch();
+  launch_dep(k_scale_dev, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, x, out, s_dev,
+             factor);
 }
 
 // Coarsest level: x = A_c^{-1} b with the inverse formed at load time from the
 // Cholesky factor (FP64).  One warp per row, lanes stride the columns.
 template <class XT>
 __global__ void __launch_bounds__(kBlock) k_coarse_gemv(int nc, const double* __restrict__ ainv,
-                                                        const XT* __restrict__ b,
-                                                        XT* __restrict__ x) {
+                                                        const XT* b, XT* x) {
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (i >= nc) return;
-  coarse_gemv_row<XT>(i, nc, ainv, b, x, lane);
+  coarse_gemv_row<XT, false, true>(i, nc, ainv, b, x, lane);
 }
 
 template <class XT>
 void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, cudaStream_t s) {
   if (nc == 0) return;
-  k_coarse_gemv<XT><<<(nc + kWarpsPerBlock - 1) / kWarpsPerBlock, kBlock, 0, s>>>(nc, ainv, b, x);
-  count_launch();
+  launch_dep(k_coarse_gemv<XT>, (nc + kWarpsPerBlock - 1) / kWarpsPerBlock, kBlock, 0, s, nc, ainv,
+             b, x);
 }
 
 // Dense Cholesky A = L L^T (right-looking, one block, in place in `work`,
@@ -348,7 +371,7 @@ void launch_chol_inverse(int n, double* work, double* ainv, int* status, cudaStr
 
 // w = M^{-1} A v and ||w||^2 into scal[S_NRM] (one power-iteration product).
 template <class VT, class XT>
-__global__ void __launch_bounds__(kBlock) k_power_step(const DevMat<VT> A,
+__global__ void __launch_bounds__(kBlock, 4) k_power_step(const DevMat<VT> A,
                                                        const XT* __restrict__ v,
                                                        const XT* __restrict__ dinv,
                                                        XT* __restrict__ w, const RedWork rw,

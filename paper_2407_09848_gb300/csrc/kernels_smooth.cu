@@ -31,16 +31,16 @@
 namespace amgps {
 
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
-__global__ void __launch_bounds__(kBlock) k_step(const StepArgs<VT, XT> a) {
+__global__ void __launch_bounds__(kBlock, 4) k_step(const StepArgs<VT, XT> a) {
   const int lane = threadIdx.x & 31;
   int64_t s = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (a.slices) {
     if (s >= a.nlist) return;
-    s = a.slices[s];
+    s = __ldg(a.slices + s);
   } else if (s >= a.A.nslices) {
     return;
   }
-  step_slice<VT, XT, FAM, INIT, WR, ZOWN>(a, s, lane);
+  step_slice<VT, XT, FAM, INIT, WR, ZOWN, false, true>(a, s, lane);
 }
 
 // Split form for levels with wide rows: one block per slice, a.split warps;
@@ -53,37 +53,42 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
   int64_t s = blockIdx.x;
   if (a.slices) {
     if (s >= a.nlist) return;
-    s = a.slices[s];
+    s = __ldg(a.slices + s);
   } else if (s >= a.A.nslices) {
     return;
   }
   const int64_t row = s * kSlice + lane;
   const bool live = row < a.A.n;
   using F = StepForm<FAM, INIT>;
-  const XT rin = (live && g == 0) ? a.rin[row] : XT(0);
-  const XT di = (live && g == 0 && step_needs_dinv<FAM>()) ? a.dinv[row] : XT(0);
-  const int w = a.A.sd[s].w;
-  const int k0 = (int)((int64_t)w * g / G), k1 = (int)((int64_t)w * (g + 1) / G);
-  part[g][lane] = row_spmv_range<F::kSign, VT, XT>(
-      a.A, s, lane, row, a.u, g == 0 ? step_init<FAM, F::kResidual>(rin, di) : XT(0), k0, k1);
+  const bool own = live && g == 0;
+  XT rin = XT(0), xin = XT(0), zo = XT(0);
+  const XT di = (own && step_needs_dinv<FAM>()) ? __ldg(a.dinv + row) : XT(0);
+  const SliceDesc d = ld_desc(a.A.sd + s);
+  const int k0 = (int)((int64_t)d.w * g / G), k1 = (int)((int64_t)d.w * (g + 1) / G);
+  part[g][lane] = row_accumulate<F::kSign, VT, XT, false, true, 4, true>(
+      a.A, d, lane, row, a.u,
+      [&] {
+        if (!own) return XT(0);
+        rin = ldv<false>(a.rin + row);
+        if (FAM != FAM_RES) xin = ldv<false>(a.xin + row);
+        if (ZOWN) zo = ldv<false>(a.zown + row);
+        return step_init<FAM, F::kResidual>(rin, di);
+      },
+      k0, k1);
   __syncthreads();
-  if (g != 0 || !live) return;
+  if (!own) return;
   XT acc = part[0][lane];
   for (int q = 1; q < G; ++q) acc += part[q][lane];
-  XT xin = XT(0), zo = XT(0);
-  if (FAM != FAM_RES) xin = a.xin[row];
-  if (ZOWN) zo = a.zown[row];
   step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, row, acc, rin, xin, di, zo);
 }
 
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
 static void go(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
   if (a.split > 1)
-    k_step_split<VT, XT, FAM, INIT, WR, ZOWN><<<(unsigned)work, 32 * a.split, 0, s>>>(a);
+    launch_dep(k_step_split<VT, XT, FAM, INIT, WR, ZOWN>, (unsigned)work, 32 * a.split, 0, s, a);
   else
-    k_step<VT, XT, FAM, INIT, WR, ZOWN>
-        <<<(unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock), kBlock, 0, s>>>(a);
-  count_launch();
+    launch_dep(k_step<VT, XT, FAM, INIT, WR, ZOWN>,
+               (unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock), kBlock, 0, s, a);
 }
 
 template <class VT, class XT, int FAM, bool INIT>
@@ -106,18 +111,17 @@ static void dispatch_op(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s)
     const unsigned g = (unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock);
     const bool s0 = a.rin != nullptr, s1 = a.xin != nullptr, wr = a.write_r;
     if (a.fam == FAM_OPT) {
-      if (wr) k_step<VT, XT, FAM_OPT, true, true, false><<<g, kBlock, 0, s>>>(a);
-      else k_step<VT, XT, FAM_OPT, true, false, false><<<g, kBlock, 0, s>>>(a);
+      if (wr) launch_dep(k_step<VT, XT, FAM_OPT, true, true, false>, g, kBlock, 0, s, a);
+      else launch_dep(k_step<VT, XT, FAM_OPT, true, false, false>, g, kBlock, 0, s, a);
     } else if (!s0) {
-      k_step<VT, XT, FAM_OP, false, false, false><<<g, kBlock, 0, s>>>(a);
+      launch_dep(k_step<VT, XT, FAM_OP, false, false, false>, g, kBlock, 0, s, a);
     } else if (!s1) {
-      if (wr) k_step<VT, XT, FAM_OP, true, true, false><<<g, kBlock, 0, s>>>(a);
-      else k_step<VT, XT, FAM_OP, true, false, false><<<g, kBlock, 0, s>>>(a);
+      if (wr) launch_dep(k_step<VT, XT, FAM_OP, true, true, false>, g, kBlock, 0, s, a);
+      else launch_dep(k_step<VT, XT, FAM_OP, true, false, false>, g, kBlock, 0, s, a);
     } else {
-      if (wr) k_step<VT, XT, FAM_OP, true, true, true><<<g, kBlock, 0, s>>>(a);
-      else k_step<VT, XT, FAM_OP, true, false, true><<<g, kBlock, 0, s>>>(a);
+      if (wr) launch_dep(k_step<VT, XT, FAM_OP, true, true, true>, g, kBlock, 0, s, a);
+      else launch_dep(k_step<VT, XT, FAM_OP, true, false, true>, g, kBlock, 0, s, a);
     }
-    count_launch();
   }
 }
 
@@ -161,28 +165,26 @@ void launch_step(const StepArgs<VT, XT>& a, cudaStream_t s) {
 
 // First step from x = 0 (no product with A): first_row (kernels_common.cuh).
 template <class XT, int FAM>
-__global__ void __launch_bounds__(kBlock) k_first(int64_t n, const XT* __restrict__ b,
-                                                  const XT* __restrict__ dinv,
-                                                  XT* __restrict__ rout, XT* __restrict__ zout,
-                                                  XT* __restrict__ xout, XT c2, XT beta,
-                                                  XT rhoinv) {
+__global__ void __launch_bounds__(kBlock) k_first(int64_t n, const XT* b,
+                                                  const XT* __restrict__ dinv, XT* rout, XT* zout,
+                                                  XT* xout, XT c2, XT beta, XT rhoinv) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (i >= n) return;
-  first_row<XT, FAM>(i, b, dinv, rout, zout, xout, c2, beta, rhoinv);
+  const XT di = dinv[i];
+  pdl_wait();
+  pdl_go();
+  first_row<XT, FAM>(i, b, di, rout, zout, xout, c2, beta, rhoinv);
 }
 
 template <class XT>
 void launch_first(int fam, int64_t n, const XT* b, const XT* dinv, XT* rout, XT* zout, XT* xout,
                   XT c2, XT beta, XT rhoinv, cudaStream_t s) {
   if (n == 0) return;
-  dim3 g((unsigned)((n + kBlock - 1) / kBlock));
-  if (fam == FAM_CHEB4)
-    k_first<XT, FAM_CHEB4><<<g, kBlock, 0, s>>>(n, b, dinv, rout, zout, xout, c2, beta, rhoinv);
-  else if (fam == FAM_CHEB1)
-    k_first<XT, FAM_CHEB1><<<g, kBlock, 0, s>>>(n, b, dinv, rout, zout, xout, c2, beta, rhoinv);
-  else
-    k_first<XT, FAM_JAC><<<g, kBlock, 0, s>>>(n, b, dinv, rout, zout, xout, c2, beta, rhoinv);
-  count_launch();
+  const unsigned g = (unsigned)((n + kBlock - 1) / kBlock);
+  auto* k = fam == FAM_CHEB4   ? k_first<XT, FAM_CHEB4>
+            : fam == FAM_CHEB1 ? k_first<XT, FAM_CHEB1>
+                               : k_first<XT, FAM_JAC>;
+  launch_dep(k, g, kBlock, 0, s, n, b, dinv, rout, zout, xout, c2, beta, rhoinv);
 }
 
 // b_c = P^T res for an unsmoothed aggregation P (Sec. 2): one thread per coarse
@@ -190,13 +192,12 @@ void launch_first(int fam, int64_t n, const XT* b, const XT* dinv, XT* rout, XT*
 // order, so the sum does not depend on scheduling.  The residual itself comes
 // from the FAM_RES step (pipelined and coalesced like the smoother steps).
 template <class XT>
-__global__ void __launch_bounds__(kBlock) k_aggregate(const int32_t* __restrict__ cptr,
+__global__ void __launch_bounds__(kBlock, 6) k_aggregate(const int32_t* __restrict__ cptr,
                                                       const int32_t* __restrict__ cidx, int64_t nc,
-                                                      const XT* __restrict__ res,
-                                                      XT* __restrict__ bc) {
+                                                      const XT* res, XT* bc) {
   const int64_t I = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (I >= nc) return;
-  aggregate_row<XT>(I, cptr, cidx, res, bc);
+  aggregate_row<XT, false, true>(I, cptr, cidx, res, bc);
 }
 
 template <class XT>
@@ -204,37 +205,36 @@ void launch_aggregate(const int32_t* cptr, const int32_t* cidx, int64_t nc, cons
                       cudaStream_t s) {
   if (nc == 0) return;
   const unsigned g = (unsigned)((nc + kBlock - 1) / kBlock);
-  k_aggregate<XT><<<g, kBlock, 0, s>>>(cptr, cidx, nc, res, bc);
-  count_launch();
+  launch_dep(k_aggregate<XT>, g, kBlock, 0, s, cptr, cidx, nc, res, bc);
 }
 
 // x += P e_c (gather through the aggregate map).
 template <class XT>
 __global__ void __launch_bounds__(kBlock) k_prolong(int64_t n, const int32_t* __restrict__ agg,
-                                                    const XT* __restrict__ ec, XT* x) {
+                                                    const XT* ec, XT* x) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (i < n) prolong_row<XT>(i, agg, ec, x);
+  if (i < n) prolong_row<XT, false, true>(i, agg, ec, x);
 }
 
 template <class XT>
 void launch_prolong(int64_t n, const int32_t* agg, const XT* ec, XT* x, cudaStream_t s) {
   if (n == 0) return;
-  k_prolong<XT><<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, agg, ec, x);
-  count_launch();
+  launch_dep(k_prolong<XT>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, agg, ec, x);
 }
 
 template <class XT>
-__global__ void __launch_bounds__(kBlock) k_add(int64_t n, const XT* __restrict__ x,
-                                                const XT* __restrict__ y, XT* out) {
+__global__ void __launch_bounds__(kBlock) k_add(int64_t n, const XT* x, const XT* y,
+                                                XT* out) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+  pdl_wait();
+  pdl_go();
   if (i < n) out[i] = x[i] + y[i];
 }
 
 template <class XT>
 void launch_add(int64_t n, const XT* x, const XT* y, XT* out, cudaStream_t s) {
   if (n == 0) return;
-  k_add<XT><<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, x, y, out);
-  count_launch();
+  launch_dep(k_add<XT>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, x, y, out);
 }
 
 // 1/M_i with M_i of Eq. l1smooth (a_ii + sum_{j != i} |a_ij|), formed once per level.
@@ -305,17 +305,17 @@ void launch_build_op(const DevMat<double>& B, double tau, double sigma, double* 
 }
 
 template <class A, class B>
-__global__ void __launch_bounds__(kBlock) k_convert(int64_t n, const A* __restrict__ in,
-                                                    B* __restrict__ out) {
+__global__ void __launch_bounds__(kBlock) k_convert(int64_t n, const A* in, B* out) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+  pdl_wait();
+  pdl_go();
   if (i < n) out[i] = B(in[i]);
 }
 
 template <class A, class B>
 void launch_convert(int64_t n, const A* in, B* out, cudaStream_t s) {
   if (n == 0) return;
-  k_convert<A, B><<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s>>>(n, in, out);
-  count_launch();
+  launch_dep(k_convert<A, B>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, in, out);
 }
 
 #define AMGPS_INST(VT, XT)                                                                   \
@@ -347,31 +347,32 @@ template void launch_convert<double, double>(int64_t, const double*, double*, cu
 // split > 1 one block per slice whose warps share the row's entries (partials
 // added in warp order).
 template <class XT>
-__global__ void __launch_bounds__(kBlock) k_xfer(const DevMat<double> M, const XT* __restrict__ u,
-                                                 XT* __restrict__ y, int add) {
+__global__ void __launch_bounds__(kBlock, 4) k_xfer(const DevMat<double> M, const XT* u, XT* y,
+                                                 int add) {
   const int lane = threadIdx.x & 31;
   const int64_t s = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (s >= M.nslices) return;
   const int64_t row = s * kSlice + lane;
-  const XT init = (add && row < M.n) ? y[row] : XT(0);
-  const XT t = row_spmv<1, double, XT>(M, s, lane, row, u, init);
+  const SliceDesc d = ld_desc(M.sd + s);
+  const XT t = row_accumulate<1, double, XT, false, true, 8, false>(
+      M, d, lane, row, u, [&] { return (add && row < M.n) ? ldv<false>(y + row) : XT(0); }, 0, d.w);
   if (row < M.n) y[row] = t;
 }
 
 template <class XT>
-__global__ void __launch_bounds__(32 * kMaxSplit) k_xfer_split(const DevMat<double> M,
-                                                               const XT* __restrict__ u,
-                                                               XT* __restrict__ y, int add) {
+__global__ void __launch_bounds__(32 * kMaxSplit) k_xfer_split(const DevMat<double> M, const XT* u,
+                                                               XT* y, int add) {
   __shared__ XT part[kMaxSplit][32];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, G = blockDim.x >> 5;
   const int64_t s = blockIdx.x;
   if (s >= M.nslices) return;
   const int64_t row = s * kSlice + lane;
   const bool live = row < M.n;
-  const XT init = (add && live && g == 0) ? y[row] : XT(0);
-  const int w = M.sd[s].w;
-  const int k0 = (int)((int64_t)w * g / G), k1 = (int)((int64_t)w * (g + 1) / G);
-  part[g][lane] = row_spmv_range<1, double, XT>(M, s, lane, row, u, init, k0, k1);
+  const SliceDesc d = ld_desc(M.sd + s);
+  const int k0 = (int)((int64_t)d.w * g / G), k1 = (int)((int64_t)d.w * (g + 1) / G);
+  part[g][lane] = row_accumulate<1, double, XT, false, true, 4, true>(
+      M, d, lane, row, u,
+      [&] { return (add && live && g == 0) ? ldv<false>(y + row) : XT(0); }, k0, k1);
   __syncthreads();
   if (g != 0 || !live) return;
   XT t = part[0][lane];
@@ -382,13 +383,11 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_xfer_split(const DevMat<doub
 template <class XT>
 void launch_xfer(const DevMat<double>& M, const XT* u, XT* y, int add, int split, cudaStream_t s) {
   if (M.nslices == 0) return;
-  if (split > 1) {
-    k_xfer_split<XT><<<(unsigned)M.nslices, 32 * split, 0, s>>>(M, u, y, add);
-  } else {
-    const unsigned grid = (unsigned)((M.nslices + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    k_xfer<XT><<<grid, kBlock, 0, s>>>(M, u, y, add);
-  }
-  count_launch();
+  if (split > 1)
+    launch_dep(k_xfer_split<XT>, (unsigned)M.nslices, 32 * split, 0, s, M, u, y, add);
+  else
+    launch_dep(k_xfer<XT>, (unsigned)((M.nslices + kWarpsPerBlock - 1) / kWarpsPerBlock), kBlock, 0,
+               s, M, u, y, add);
 }
 template void launch_xfer<double>(const DevMat<double>&, const double*, double*, int, int,
                                   cudaStream_t);

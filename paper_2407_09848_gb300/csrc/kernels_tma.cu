@@ -131,6 +131,31 @@ __global__ void __launch_bounds__((tma_warps<XT>() + 1) * 32, TmaShape<XT>::kCta
   __syncthreads();
 
   if (warp == 0) {
+    // the residual needs no x_in or 1/M; a scaled step with scaled rin no
+    // 1/M; FP64 stages hold no 1/M slot (read from global memory)
+    // (a stored-operator step copies the slots it reads)
+    constexpr bool wdi = step_needs_dinv<FAM>() && TmaShape<XT>::kVecSlots == 3;
+    constexpr bool c0 = reads_slot0<FAM, INIT>(), c1 = reads_slot1<FAM, ZOWN>();
+    constexpr int nvec = (c0 ? 1 : 0) + (c1 ? 1 : 0) + (wdi ? 1 : 0);
+    const uint32_t stage_tx = (uint32_t)(p.vals_bytes + nvec * p.vec_bytes + p.win_bytes);
+    // a tile's values (no kernel of the chain writes them) ...
+    auto copy_vals = [&](int st, long long r0, long long vb) {
+      stage_r0[st] = r0;
+      mbar_expect_tx(&full[st], stage_tx);
+      bulk_g2s(stages + (size_t)st * p.stage_bytes, a.A.val + vb, (uint32_t)p.vals_bytes,
+               &full[st]);
+    };
+    // ... and its vectors, which the previous kernel may have written
+    auto copy_vecs = [&](int st, long long r0) {
+      XT* sv = reinterpret_cast<XT*>(stages + (size_t)st * p.stage_bytes + p.vals_bytes);
+      if (c0) bulk_g2s(sv, a.rin + r0, (uint32_t)p.vec_bytes, &full[st]);
+      if (c1) bulk_g2s(sv + p.rows, a.xin + r0, (uint32_t)p.vec_bytes, &full[st]);
+      if (wdi) bulk_g2s(sv + 2 * p.rows, a.dinv + r0, (uint32_t)p.vec_bytes, &full[st]);
+      XT* sw = sv + TmaShape<XT>::kVecSlots * p.rows;
+      for (int g = 0; g < p.ngroups; ++g)
+        bulk_g2s(sw + p.g_smem[g], a.u + r0 + p.g_start[g],
+                 (uint32_t)(p.g_elems[g] * (int)sizeof(XT)), &full[st]);
+    };
     // The whole warp fetches the descriptors of this CTA's next 32 tiles in one
     // load; lane 0 then issues their copies without a global round trip per tile.
     int it = 0;
@@ -140,7 +165,25 @@ __global__ void __launch_bounds__((tma_warps<XT>() + 1) * 32, TmaShape<XT>::kCta
       TmaTile mine{0, 0};
       if (jl < ntiles) mine = tiles[jl];
       const int cnt = min(32, (ntiles - j0 + (int)gridDim.x - 1) / (int)gridDim.x);
-      for (int q = 0; q < cnt; ++q) {
+      int q0 = 0;
+      if (j0 == (int)blockIdx.x) {
+        // the first fill of the (empty) stages: the values before the wait for
+        // the previous kernel, while that kernel's last CTAs still run
+        q0 = min(cnt, ns);
+        for (int q = 0; q < q0; ++q) {
+          const long long rq = __shfl_sync(0xffffffffu, (long long)mine.r0, q);
+          const long long vq = __shfl_sync(0xffffffffu, (long long)mine.vbase, q);
+          if (lane == 0) copy_vals(q, rq, vq);
+        }
+        pdl_wait();
+        if (a.go) pdl_go();
+        for (int q = 0; q < q0; ++q) {
+          const long long rq = __shfl_sync(0xffffffffu, (long long)mine.r0, q);
+          if (lane == 0) copy_vecs(q, rq);
+        }
+        it = q0;
+      }
+      for (int q = q0; q < cnt; ++q) {
         const long long rq = __shfl_sync(0xffffffffu, (long long)mine.r0, q);
         const long long vq = __shfl_sync(0xffffffffu, (long long)mine.vbase, q);
         if (lane == 0) {
@@ -149,25 +192,8 @@ __global__ void __launch_bounds__((tma_warps<XT>() + 1) * 32, TmaShape<XT>::kCta
           if (abort_flag || !mbar_wait(&empty[st], ph ^ 1u)) {
             abort_flag = 1;
           } else {
-            unsigned char* base = stages + (size_t)st * p.stage_bytes;
-            const int64_t r0 = rq;
-            stage_r0[st] = rq;
-            // the residual needs no x_in or 1/M; a scaled step with scaled rin no
-            // 1/M; FP64 stages hold no 1/M slot (read from global memory)
-            // (a stored-operator step copies the slots it reads)
-            constexpr bool wdi = step_needs_dinv<FAM>() && TmaShape<XT>::kVecSlots == 3;
-            constexpr bool c0 = reads_slot0<FAM, INIT>(), c1 = reads_slot1<FAM, ZOWN>();
-            constexpr int nvec = (c0 ? 1 : 0) + (c1 ? 1 : 0) + (wdi ? 1 : 0);
-            mbar_expect_tx(&full[st], (uint32_t)(p.vals_bytes + nvec * p.vec_bytes + p.win_bytes));
-            bulk_g2s(base, a.A.val + vq, (uint32_t)p.vals_bytes, &full[st]);
-            XT* sv = reinterpret_cast<XT*>(base + p.vals_bytes);
-            if (c0) bulk_g2s(sv, a.rin + r0, (uint32_t)p.vec_bytes, &full[st]);
-            if (c1) bulk_g2s(sv + p.rows, a.xin + r0, (uint32_t)p.vec_bytes, &full[st]);
-            if (wdi) bulk_g2s(sv + 2 * p.rows, a.dinv + r0, (uint32_t)p.vec_bytes, &full[st]);
-            XT* sw = sv + TmaShape<XT>::kVecSlots * p.rows;
-            for (int g = 0; g < p.ngroups; ++g)
-              bulk_g2s(sw + p.g_smem[g], a.u + r0 + p.g_start[g],
-                       (uint32_t)(p.g_elems[g] * (int)sizeof(XT)), &full[st]);
+            copy_vals(st, rq, vq);
+            copy_vecs(st, rq);
             ++it;  // lane 0 counts issued tiles only: the drain waits for these
           }
         }
@@ -187,6 +213,7 @@ __global__ void __launch_bounds__((tma_warps<XT>() + 1) * 32, TmaShape<XT>::kCta
     return;
   }
 
+  pdl_wait();
   const int c = warp - 1;
   constexpr int kGroups = TmaShape<XT>::kGroups, kCons = TmaShape<XT>::kConsumers;
   const int grp = c / kCons, cw = c % kCons;
@@ -337,9 +364,8 @@ template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN, int W>
 void launch_inst(const StepArgs<VT, XT>& a, const TmaPlan& p, const TmaTile* tiles, int ntiles,
                  int grid, double* err, cudaStream_t s) {
   const int smem = kBarrierBytes + p.nstages * p.stage_bytes;
-  k_step_tma<VT, XT, FAM, INIT, WR, ZOWN, W><<<grid, (tma_warps<XT>() + 1) * 32, smem, s>>>(
-      a, p, tiles, ntiles, a.slices, a.slices ? a.nlist : 0, err);
-  count_launch();
+  launch_dep(k_step_tma<VT, XT, FAM, INIT, WR, ZOWN, W>, grid, (tma_warps<XT>() + 1) * 32, smem, s,
+             a, p, tiles, ntiles, a.slices, a.slices ? a.nlist : 0, err);
 }
 
 template <class VT, class XT, int FAM, bool INIT, int W>
