@@ -105,6 +105,9 @@ struct StepArgs {
   // L1 would start under this kernel's shared-memory carve-out, which an SM
   // that is never idle keeps.
   bool go = true;
+  // direct step on FP64 levels: this many vectors, vector v at u + v n, rin + v n
+  // and so on (one A); the values of a 7-point row are loaded once for four
+  int nvec = 1;
 };
 
 // Most warps per slice in the split form of the step and transfer kernels
@@ -197,13 +200,15 @@ bool launch_step_tma(const StepArgs<VT, XT>& a, const TmaPlan& p, const TmaTile*
                      int ntiles, int grid, double* err_slot, cudaStream_t s);
 template <class XT>
 void launch_first(int fam, int64_t n, const XT* b, const XT* dinv, XT* rout, XT* zout, XT* xout,
-                  XT c2, XT beta, XT rhoinv, cudaStream_t s);
+                  XT c2, XT beta, XT rhoinv, int nvec, cudaStream_t s);
 // b_c[I] = sum of res over the children of coarse row I (children lists)
+// (nvec vectors of n fine and nc coarse entries, one after another)
 template <class XT>
-void launch_aggregate(const int32_t* cptr, const int32_t* cidx, int64_t nc, const XT* res, XT* bc,
-                      cudaStream_t s);
+void launch_aggregate(const int32_t* cptr, const int32_t* cidx, int64_t n, int64_t nc,
+                      const XT* res, XT* bc, int nvec, cudaStream_t s);
 template <class XT>
-void launch_prolong(int64_t n, const int32_t* agg, const XT* ec, XT* x, cudaStream_t s);
+void launch_prolong(int64_t n, int64_t nc, const int32_t* agg, const XT* ec, XT* x, int nvec,
+                    cudaStream_t s);
 // general prolongator transfers: y = M u (add = 0) or y += M u (add = 1);
 // split > 1: one block of `split` warps per slice
 template <class XT>
@@ -212,8 +217,9 @@ void launch_xfer(const DevMat<double>& M, const XT* u, XT* y, int add, int split
 template <class XT>
 void launch_add(int64_t n, const XT* x, const XT* y, XT* out, cudaStream_t s);
 void launch_sub(int64_t n, const double* x, const double* y, double* out, cudaStream_t s);
-void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, double factor,
-                      cudaStream_t s);
+// (vector v of nvec: out + v n = (factor / s_dev[v stride]) (x + v n))
+void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, int stride,
+                      double factor, int nvec, cudaStream_t s);
 
 // ---- persistent kernel for the coarse levels of a V-cycle (kernels_cycle.cu) ----
 // The levels below the TMA-fed ones are launch-latency-bound: their kernels

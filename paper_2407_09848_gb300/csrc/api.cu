@@ -249,6 +249,7 @@ struct amgps_ctx {
   double* dloss = nullptr;      // per error vector: <e0, A e0>, <e1, A e1>
   double* hdots = nullptr;
   bool bwd_ready = false;
+  int nvec = 1;                 // vectors the engine's kernels work on (> 1 inside a Batch)
   double* part = nullptr;
   unsigned* counters = nullptr;
   int red_grid = 0;
@@ -351,6 +352,7 @@ void free_hierarchy(amgps_ctx* c) {
   c->loaded = false;
   c->bwd_ready = false;
   c->pr = c->pp = c->pq = c->pz = c->pz2 = c->stage_b = c->stage_x = nullptr;
+  c->dacc = c->dloss = nullptr;
 }
 
 void enter(amgps_ctx* c) {
@@ -508,7 +510,7 @@ struct Engine {
   }
 
   static void do_first(int fam, int64_t n, const XT* b, const XT* dinv, XT* r, XT* z, XT* x,
-                       XT c2, XT beta, XT rhoinv, cudaStream_t s) {
+                       XT c2, XT beta, XT rhoinv, int nvec, cudaStream_t s) {
     if (auto* R = rec()) {
       CyclePhase<VT, XT> p;
       p.op = CY_FIRST;
@@ -525,7 +527,7 @@ struct Engine {
       R->push_back(p);
       return;
     }
-    launch_first<XT>(fam, n, b, dinv, r, z, x, c2, beta, rhoinv, s);
+    launch_first<XT>(fam, n, b, dinv, r, z, x, c2, beta, rhoinv, nvec, s);
   }
 
   static void do_copy(XT* dst, const XT* src, int64_t n, cudaStream_t s) {
@@ -541,7 +543,7 @@ struct Engine {
     CK(cudaMemcpyAsync(dst, src, n * sizeof(XT), cudaMemcpyDeviceToDevice, s));
   }
 
-  static void do_aggregate(const Level& L, const XT* res, XT* bc, cudaStream_t s) {
+  static void do_aggregate(const Level& L, const XT* res, XT* bc, int nvec, cudaStream_t s) {
     if (auto* R = rec()) {
       CyclePhase<VT, XT> p;
       p.op = CY_AGG;
@@ -553,10 +555,10 @@ struct Engine {
       R->push_back(p);
       return;
     }
-    launch_aggregate<XT>(L.cptr, L.cidx, L.nc, res, bc, s);
+    launch_aggregate<XT>(L.cptr, L.cidx, L.n, L.nc, res, bc, nvec, s);
   }
 
-  static void do_prolong(const Level& L, const XT* ec, XT* x, cudaStream_t s) {
+  static void do_prolong(const Level& L, const XT* ec, XT* x, int nvec, cudaStream_t s) {
     if (auto* R = rec()) {
       CyclePhase<VT, XT> p;
       p.op = CY_PROLONG;
@@ -567,10 +569,10 @@ struct Engine {
       R->push_back(p);
       return;
     }
-    launch_prolong<XT>(L.n, L.agg, ec, x, s);
+    launch_prolong<XT>(L.n, L.nc, L.agg, ec, x, nvec, s);
   }
 
-  static void do_gemv(const Level& L, const XT* b, XT* x, cudaStream_t s) {
+  static void do_gemv(const Level& L, const XT* b, XT* x, int nvec, cudaStream_t s) {
     if (auto* R = rec()) {
       CyclePhase<VT, XT> p;
       p.op = CY_GEMV;
@@ -581,13 +583,14 @@ struct Engine {
       R->push_back(p);
       return;
     }
-    launch_coarse_gemv<XT>((int)L.n, L.ainv, b, x, s);
+    launch_coarse_gemv<XT>((int)L.n, L.ainv, b, x, nvec, s);
   }
 
   // One fused step on level L: the TMA-fed kernel over its tiles plus the
   // direct kernel over the remaining slices, or the direct kernel alone.
   static void run_step(amgps_ctx* c, const Level& L, StepArgs<VT, XT> a, cudaStream_t s) {
     a.split = L.split;
+    a.nvec = c->nvec;
     if (L.sval && a.fam == FAM_CHEB4) {
       a.A.val = (const VT*)L.sval;
       a.fam = (a.rin_raw || a.init) ? FAM_CHEB4SR : FAM_CHEB4S;  // an initial step's rin is b
@@ -610,7 +613,7 @@ struct Engine {
       R->push_back(p);
       return;
     }
-    if (level_uses_tma(c, L)) {
+    if (c->nvec == 1 && level_uses_tma(c, L)) {
       // the TMA kernel also runs the slices outside its plan (slice list)
       StepArgs<VT, XT> t = a;
       t.slices = L.ngen > 0 ? L.gen_slices : nullptr;
@@ -651,7 +654,8 @@ struct Engine {
     XT* t = (XT*)L.r;
     const bool profl = (l == 0);
     if (!c_ready)
-      do_first(FAM_JAC, L.n, b, (const XT*)L.dinv, nullptr, nullptr, cv, XT(0), XT(0), XT(1), s);
+      do_first(FAM_JAC, L.n, b, (const XT*)L.dinv, nullptr, nullptr, cv, XT(0), XT(0), XT(1),
+               c->nvec, s);
     const DevMat<VT> A = devmat<VT>(L);
     if (!xzero) {
       StepArgs<VT, XT> a;
@@ -726,7 +730,7 @@ struct Engine {
       XT* oth = xb;
       int j0 = 0;
       if (xzero) {
-        do_first(FAM_JAC, L.n, b, md, nullptr, nullptr, cur, XT(0), XT(0), XT(1), s);
+        do_first(FAM_JAC, L.n, b, md, nullptr, nullptr, cur, XT(0), XT(0), XT(1), c->nvec, s);
         j0 = 1;
       }
       for (int j = j0; j < k; ++j) {
@@ -746,7 +750,7 @@ struct Engine {
         ps.done();
         std::swap(cur, oth);
       }
-      if (cur != x) do_copy(x, cur, L.n, s);
+      if (cur != x) do_copy(x, cur, L.n * c->nvec, s);
       check_launch();
       return false;
     }
@@ -759,7 +763,7 @@ struct Engine {
         c2 *= rhoinv;
         rhoinv = 1.0;
       }
-      do_first(cf.fam, L.n, b, md, r, zc, x, XT(c2), XT(cf.beta[1]), XT(rhoinv), s);
+      do_first(cf.fam, L.n, b, md, r, zc, x, XT(c2), XT(cf.beta[1]), XT(rhoinv), c->nvec, s);
       rin_next = (cf.fam == FAM_CHEB4) ? b : r;
     } else {
       StepArgs<VT, XT> a;
@@ -821,7 +825,7 @@ struct Engine {
       rin_next = r;
       std::swap(zc, zn);
     }
-    if (xcur != x) do_copy(x, xcur, L.n, s);
+    if (xcur != x) do_copy(x, xcur, L.n * c->nvec, s);
     check_launch();
     return false;
   }
@@ -837,7 +841,7 @@ struct Engine {
       cf.k = c->coarse_sweeps;
       smooth(c, l, cf, b, x, true);
     } else {
-      do_gemv(L, b, x, c->stream);
+      do_gemv(L, b, x, c->nvec, c->stream);
       check_launch();
     }
   }
@@ -848,7 +852,7 @@ struct Engine {
                            bool c_ready = false) {
     Level& L = c->lv[l];
     cudaStream_t s = c->stream;
-    if (!record && !rec() && c->tail_ok && l == c->tail_level && b == (const XT*)L.b &&
+    if (!record && !rec() && c->nvec == 1 && c->tail_ok && l == c->tail_level && b == (const XT*)L.b &&
         x == (XT*)L.x) {
       launch_tail(c);
       return;
@@ -878,13 +882,13 @@ struct Engine {
       a.go = false;
       run_step(c, L, a, s);
       if (L.xfer_general) launch_xfer<XT>(L.Rm, (const XT*)L.r, (XT*)C.b, 0, L.rsplit, s);
-      else do_aggregate(L, (const XT*)L.r, (XT*)C.b, s);
+      else do_aggregate(L, (const XT*)L.r, (XT*)C.b, c->nvec, s);
       ps.done();
     }
     {
       // levels >= 1 of the cycle, timed as one class-4 interval from level 0
       ProfScope ps(c, l == 0, 4, 0.0);
-      if (l + 1 == 1 && c->graph_ok && !record && !capturing(c)) {
+      if (l + 1 == 1 && c->nvec == 1 && c->graph_ok && !record && !capturing(c)) {
         CK(cudaGraphLaunch(c->gexec, s));
         c->launch_adjust += c->graph_kernels;
       } else {
@@ -893,8 +897,9 @@ struct Engine {
       ps.done();
     }
     if (L.xfer_general) launch_xfer<XT>(L.Pm, (const XT*)C.x, x, 1, L.psplit, s);
-    else do_prolong(L, (const XT*)C.x, x, s);
-    if (record) CK(cudaMemcpyAsync(L.bx2, x, L.n * sizeof(XT), cudaMemcpyDeviceToDevice, s));
+    else do_prolong(L, (const XT*)C.x, x, c->nvec, s);
+    if (record)
+      CK(cudaMemcpyAsync(L.bx2, x, c->nvec * L.n * sizeof(XT), cudaMemcpyDeviceToDevice, s));
     smooth(c, l, cf, b, x, false, c_kept);
     check_launch();
   }
@@ -918,12 +923,12 @@ struct Engine {
     XT* zc = (XT*)L.za;
     XT* zn = (XT*)L.zb;
     XT* xs = (XT*)L.xb;
-    const int64_t n = L.n;
+    const int64_t n = L.n * c->nvec;  // <gx, z_j> summed over the vectors of a batch
     const int k = cf.k;
     RedWork rw = redwork(c, 5, n);
     const XT* rin_next;
     if (!x0) {
-      launch_first<XT>(FAM_CHEB4, n, b, md, r, zc, xs, XT(cf.c2[1]), XT(0), XT(1), s);
+      launch_first<XT>(FAM_CHEB4, L.n, b, md, r, zc, xs, XT(cf.c2[1]), XT(0), XT(1), c->nvec, s);
       rin_next = b;
     } else {
       StepArgs<VT, XT> a;
@@ -1008,13 +1013,13 @@ struct Engine {
     smooth_bwd(c, l, cf, bl, (const XT*)L.bx2, xbar, t1, t2, l * 32);
     // x2 = x1 + P xc ; xc = V_{l+1}(P^T (b - A x1))
     if (L.xfer_general) launch_xfer<XT>(L.Rm, (const XT*)t2, (XT*)C.bgx, 0, L.rsplit, s);
-    else launch_aggregate<XT>(L.cptr, L.cidx, L.nc, t2, (XT*)C.bgx, s);
+    else launch_aggregate<XT>(L.cptr, L.cidx, L.n, L.nc, t2, (XT*)C.bgx, c->nvec, s);
     vcycle_bwd(c, l + 1, (const XT*)C.b, (const XT*)C.bgx, (XT*)C.bgb);
-    CK(cudaMemsetAsync(t3, 0, L.n * sizeof(XT), s));
+    CK(cudaMemsetAsync(t3, 0, c->nvec * L.n * sizeof(XT), s));
     // dL/dres = P dL/db_c
     if (L.xfer_general) launch_xfer<XT>(L.Pm, (const XT*)C.bgb, t3, 1, L.psplit, s);
-    else launch_prolong<XT>(L.n, L.agg, (const XT*)C.bgb, t3, s);
-    launch_add<XT>(L.n, t1, t3, gbout, s);
+    else launch_prolong<XT>(L.n, L.nc, L.agg, (const XT*)C.bgb, t3, c->nvec, s);
+    launch_add<XT>(c->nvec * L.n, t1, t3, gbout, s);
     {
       StepArgs<VT, XT> a;  // dL/dx1 = dL/dx2 - A dL/dres  -> t1
       a.A = devmat<VT>(L);
@@ -1028,14 +1033,17 @@ struct Engine {
     }
     // pre-smoother x1 = S(b, 0)
     smooth_bwd(c, l, cf, bl, nullptr, t1, t2, nullptr, l * 32 + 16);
-    launch_add<XT>(L.n, gbout, t2, gbout, s);
+    launch_add<XT>(c->nvec * L.n, gbout, t2, gbout, s);
     check_launch();
+  }
+
+  static void ensure_loss(amgps_ctx* c) {
+    if (!c->dacc) c->dacc = (double*)dalloc(c, kDotSlots * sizeof(double));
+    if (!c->dloss) c->dloss = (double*)dalloc(c, 2 * kMaxLossVectors * sizeof(double));
   }
 
   static void ensure_bwd(amgps_ctx* c) {
     if (c->bwd_ready) return;
-    c->dacc = (double*)dalloc(c, kDotSlots * sizeof(double));
-    c->dloss = (double*)dalloc(c, 2 * kMaxLossVectors * sizeof(double));
     for (auto& L : c->lv) {
       const size_t bytes = L.n * sizeof(XT);
       L.bgx = dalloc(c, bytes);
@@ -1453,6 +1461,183 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
 }  // namespace
 
 // ---------------------------------------------------------------------------
+// Batches: the loss gradient and the error cycles take m independent vectors
+// through the same V-cycles.  One vector of a 64^3 training grid leaves a
+// kernel of 2 to 8 us that is mostly latency; a batch runs every kernel on B
+// vectors at once (vector v at + v n of each buffer), so there are B times
+// fewer launches and a 7-point row's values are read once for four vectors.
+// B x n_0 is kept near kBatchRows: measured on the 32 vectors of a 64^3
+// problem, one pass (6 pre-cycles, loss and gradient) takes 43.2 ms one by one
+// and 17.8 ms in two batches of 16 (its FP64 multiply-adds alone: 10.6 ms).
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr int64_t kBatchRows = int64_t(1) << 22;
+
+// The batch buffers come from one stream-ordered pool per device, shared by
+// the contexts of the process (a training run holds hundreds of contexts and
+// uses one at a time).  Between calls the pool keeps at most kPoolKeep bytes;
+// the last context of a device to be destroyed gives them back.
+constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
+constexpr int kPoolDevices = 64;
+struct BatchPools {
+  std::mutex mu;
+  cudaMemPool_t pool[kPoolDevices] = {};
+  int users[kPoolDevices] = {};
+};
+BatchPools& batch_pools() {
+  static BatchPools* p = new BatchPools();  // outlives every context
+  return *p;
+}
+
+void pool_enter(int device) {
+  if (device >= kPoolDevices) return;
+  BatchPools& P = batch_pools();
+  std::lock_guard<std::mutex> lk(P.mu);
+  ++P.users[device];
+}
+
+void pool_leave(int device) {
+  if (device >= kPoolDevices) return;
+  BatchPools& P = batch_pools();
+  std::lock_guard<std::mutex> lk(P.mu);
+  if (--P.users[device] == 0 && P.pool[device]) {
+    cudaMemPoolTrimTo(P.pool[device], 0);
+    cudaGetLastError();
+  }
+}
+
+// null when the device has no pool (the calls then go one vector at a time)
+cudaMemPool_t pool_of(int device) {
+  if (device >= kPoolDevices) return nullptr;
+  BatchPools& P = batch_pools();
+  std::lock_guard<std::mutex> lk(P.mu);
+  if (!P.pool[device]) {
+    cudaMemPoolProps pr = {};
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    pr.location.id = device;
+    cudaMemPool_t p = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&p, &pr) != cudaSuccess ||
+        cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      if (p) cudaMemPoolDestroy(p);
+      return nullptr;
+    }
+    P.pool[device] = p;
+  }
+  return P.pool[device];
+}
+
+// Puts B-vector buffers in the place of every level's own for its lifetime
+// (FP64 hierarchies); ok() is false, and nothing changed, when they cannot be
+// had.
+class Batch {
+ public:
+  Batch(amgps_ctx* c, int B, bool bwd) : c_(c), n0_(c->lv[0].n) {
+    bytes_ = layout(c, B, bwd, nullptr);
+    cudaMemPool_t pool = pool_of(c->device);
+    if (!pool || cudaMallocFromPoolAsync(&base_, bytes_, pool, c->stream) != cudaSuccess) {
+      cudaGetLastError();
+      base_ = nullptr;
+      return;
+    }
+    saved_ = c->lv;
+    c->nvec = B;
+    layout(c, B, bwd, (char*)base_);
+  }
+  ~Batch() {
+    if (!base_) return;
+    for (size_t l = 0; l < saved_.size(); ++l) {
+      Level &L = c_->lv[l], &S = saved_[l];
+      L.b = S.b, L.x = S.x, L.r = S.r, L.za = S.za, L.zb = S.zb, L.xb = S.xb;
+      L.bx2 = S.bx2, L.bgx = S.bgx, L.bgb = S.bgb, L.bt1 = S.bt1, L.bt2 = S.bt2, L.bt3 = S.bt3;
+    }
+    c_->nvec = 1;
+    cudaFreeAsync(base_, c_->stream);
+  }
+  Batch(const Batch&) = delete;
+  Batch& operator=(const Batch&) = delete;
+  bool ok() const { return base_ != nullptr; }
+  // a smaller last batch: the buffers keep their places
+  void size(int B) { c_->nvec = B; }
+  double *r = nullptr, *z = nullptr, *e1 = nullptr, *dots = nullptr;
+  RedWork rw;
+
+  // the most bytes a batch of B may take
+  static size_t need(amgps_ctx* c, int B, bool bwd) {
+    return Batch(c).layout(c, B, bwd, nullptr);
+  }
+
+ private:
+  explicit Batch(amgps_ctx* c) : c_(c), n0_(c->lv[0].n) {}
+
+  // places every buffer from `base` on (null: only adds up); returns the bytes
+  size_t layout(amgps_ctx* c, int B, bool bwd, char* base) {
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+      void* p = base ? base + at : nullptr;
+      at += (bytes + 255) / 256 * 256;
+      return p;
+    };
+    const size_t vec0 = (size_t)B * n0_ * sizeof(double);
+    rw.grid = reduction_grid(c->lv[0].nslices * kSlice, c->nsm, std::max(1, 8 / B));
+    rw.counter = (unsigned*)take(B * sizeof(unsigned));
+    rw.part = (double*)take((size_t)B * rw.grid * sizeof(double));
+    dots = (double*)take(B * sizeof(double));
+    r = (double*)take(vec0);
+    z = (double*)take(vec0);
+    if (bwd) e1 = (double*)take(vec0);
+    for (size_t l = 0; l < c->lv.size(); ++l) {
+      Level& L = c->lv[l];
+      const size_t v = (size_t)B * L.n * sizeof(double);
+      auto put = [&](void*& p) {
+        void* q = take(v);
+        if (base) p = q;
+      };
+      if (l > 0) put(L.b), put(L.x);
+      put(L.r), put(L.za), put(L.zb), put(L.xb);
+      if (!bwd) continue;
+      if (l > 0) put(L.bgx);
+      put(L.bgb);
+      if (!L.coarsest) put(L.bx2), put(L.bt1), put(L.bt2), put(L.bt3);
+    }
+    return at;
+  }
+
+  amgps_ctx* c_;
+  int64_t n0_;
+  size_t bytes_ = 0;
+  void* base_ = nullptr;
+  std::vector<Level> saved_;
+};
+
+// Vectors per batch for m vectors: 1 (one by one, in the context's own
+// buffers) for FP32/BF16 hierarchies, levels that the batched kernels do not
+// take (several warps per slice, general prolongators), grids of more than
+// half of kBatchRows, while kernels are being timed, under stream capture, or
+// where the allocation limit leaves no room.
+int batch_size(amgps_ctx* c, int m, bool bwd) {
+  if (c->prec != AMGPS_F64 || c->prof || c->lv.size() < 2) return 1;
+  cudaStreamCaptureStatus cap;
+  CK(cudaStreamIsCapturing(c->stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return 1;
+  for (const Level& L : c->lv)
+    if (L.coarsest ? (c->coarse_sweeps > 0 && L.split > 1) : (L.split > 1 || L.xfer_general))
+      return 1;
+  int64_t B = std::min<int64_t>(m, kBatchRows / c->lv[0].n);
+  if (B < 2) return 1;
+  const int64_t parts = (m + B - 1) / B;  // of equal size
+  B = (m + parts - 1) / parts;
+  if (c->alloc_limit)
+    while (B > 1 && c->alloc_bytes + Batch::need(c, (int)B, bwd) > c->alloc_limit) B /= 2;
+  return (int)B;
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
 // Allocation-free smoother application (amgps_smooth_noalloc).
 //
 // Its work vectors (the recurrence residual r, the two z buffers, the second
@@ -1578,6 +1763,7 @@ amgps_status amgps_create(amgps_ctx** out, int device, void* user_stream) {
     CK(cudaMalloc(&u->counters, 8 * sizeof(unsigned)));
     CK(cudaMemset(u->counters, 0, 8 * sizeof(unsigned)));
     c = u.release();
+    pool_enter(device);
   });
   if (st == AMGPS_OK) *out = c;
   return st;
@@ -1605,6 +1791,7 @@ amgps_status amgps_destroy(amgps_ctx* c) {
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->ev_sync) cudaEventDestroy(c->ev_sync);
   if (c->stream) cudaStreamDestroy(c->stream);
+  pool_leave(c->device);
   delete c;
   return AMGPS_OK;
 }
@@ -1956,7 +2143,7 @@ amgps_status amgps_vcycle_backward(amgps_ctx* c, const double* r, const double* 
     E::ensure_bwd(c);
     Level& L0 = c->lv[0];
     if (L0.coarsest) {
-      launch_coarse_gemv<double>((int)L0.n, L0.ainv, gz, gr ? gr : (double*)L0.bgb, c->stream);
+      launch_coarse_gemv<double>((int)L0.n, L0.ainv, gz, gr ? gr : (double*)L0.bgb, 1, c->stream);
       check_launch();
     } else {
       E::vcycle_level(c, 0, r, (double*)L0.x, true);  // forward, recording each level's x2
@@ -1991,29 +2178,54 @@ amgps_status amgps_vcycle_loss_grad(amgps_ctx* c, const double* E0, int m, doubl
     REQ(c->lv.size() >= 2 && c->lv.size() <= 32, AMGPS_E_ARG, "needs 2..32 levels");
     using E = Engine<double, double>;
     enter(c);
-    E::ensure_bwd(c);
+    E::ensure_loss(c);
     cudaStream_t s = c->stream;
     Level& L0 = c->lv[0];
     const int64_t n = L0.n;
     const DevMat<double> A = devmat64(L0, c->prec);
-    RedWork rw = redwork(c, 1, n);
-    rw.grid = reduction_grid(L0.nslices * kSlice, c->nsm);
-    double *r = c->pp, *z = c->pz, *e1 = c->pr, *q1 = c->pq, *gz = c->stage_x;
     CK(cudaMemsetAsync(c->dacc, 0, kDotSlots * sizeof(double), s));
-    for (int i = 0; i < m; ++i) {
-      const double* e0 = E0 + (size_t)i * n;
-      launch_spmv_dot(A, e0, r, rw, c->dscal, s);  // r = A e0, <e0, A e0>
-      CK(cudaMemcpyAsync(c->dloss + 2 * i, c->dscal + S_PQ, sizeof(double),
-                         cudaMemcpyDeviceToDevice, s));
-      E::vcycle_level(c, 0, r, z, true);            // z = B r, recorded
-      launch_sub(n, e0, z, e1, s);                  // e1 = (I - B A) e0
-      launch_spmv_dot(A, e1, q1, rw, c->dscal, s);  // A e1, <e1, A e1>
-      CK(cudaMemcpyAsync(c->dloss + 2 * i + 1, c->dscal + S_PQ, sizeof(double),
-                         cudaMemcpyDeviceToDevice, s));
-      launch_scale_dev(n, q1, gz, c->dloss + 2 * i, -2.0 / m, s);  // dL/dz
-      E::vcycle_bwd(c, 0, r, gz, (double*)L0.bgb);
-      launch_add<double>(kDotSlots, c->dacc, c->ddots, c->dacc, s);
-      check_launch();
+    const int B = batch_size(c, m, true);
+    std::unique_ptr<Batch> bt;
+    if (B > 1) {
+      bt.reset(new Batch(c, B, true));
+      if (!bt->ok()) bt.reset();
+    }
+    if (bt) {
+      CK(cudaMemsetAsync(bt->rw.counter, 0, B * sizeof(unsigned), s));
+      for (int i = 0; i < m; i += B) {
+        const int nv = std::min(B, m - i);
+        bt->size(nv);
+        const double* e0 = E0 + (size_t)i * n;
+        launch_spmv_dot_mv(A, e0, bt->r, bt->rw, c->dloss + 2 * i, 2, nv, s);  // r = A e0
+        E::vcycle_level(c, 0, bt->r, bt->z, true);       // z = B r, recorded
+        launch_sub(n * nv, e0, bt->z, bt->e1, s);        // e1 = (I - B A) e0
+        launch_spmv_dot_mv(A, bt->e1, bt->z, bt->rw, c->dloss + 2 * i + 1, 2, nv, s);  // A e1
+        launch_scale_dev(n, bt->z, bt->z, c->dloss + 2 * i, 2, -2.0 / m, nv, s);       // dL/dz
+        E::vcycle_bwd(c, 0, bt->r, bt->z, (double*)L0.bgb);
+        launch_add<double>(kDotSlots, c->dacc, c->ddots, c->dacc, s);
+        check_launch();
+      }
+      bt.reset();
+    } else {
+      E::ensure_bwd(c);
+      RedWork rw = redwork(c, 1, n);
+      rw.grid = reduction_grid(L0.nslices * kSlice, c->nsm);
+      double *r = c->pp, *z = c->pz, *e1 = c->pr, *q1 = c->pq, *gz = c->stage_x;
+      for (int i = 0; i < m; ++i) {
+        const double* e0 = E0 + (size_t)i * n;
+        launch_spmv_dot(A, e0, r, rw, c->dscal, s);  // r = A e0, <e0, A e0>
+        CK(cudaMemcpyAsync(c->dloss + 2 * i, c->dscal + S_PQ, sizeof(double),
+                           cudaMemcpyDeviceToDevice, s));
+        E::vcycle_level(c, 0, r, z, true);            // z = B r, recorded
+        launch_sub(n, e0, z, e1, s);                  // e1 = (I - B A) e0
+        launch_spmv_dot(A, e1, q1, rw, c->dscal, s);  // A e1, <e1, A e1>
+        CK(cudaMemcpyAsync(c->dloss + 2 * i + 1, c->dscal + S_PQ, sizeof(double),
+                           cudaMemcpyDeviceToDevice, s));
+        launch_scale_dev(n, q1, gz, c->dloss + 2 * i, 0, -2.0 / m, 1, s);  // dL/dz
+        E::vcycle_bwd(c, 0, r, gz, (double*)L0.bgb);
+        launch_add<double>(kDotSlots, c->dacc, c->ddots, c->dacc, s);
+        check_launch();
+      }
     }
     std::vector<double> hl(2 * (size_t)m);
     CK(cudaMemcpyAsync(hl.data(), c->dloss, 2 * m * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2047,14 +2259,35 @@ amgps_status amgps_error_cycles(amgps_ctx* c, double* E, int m, int cycles) {
     Level& L0 = c->lv[0];
     const int64_t n = L0.n;
     const DevMat<double> A = devmat64(L0, c->prec);
-    RedWork rw = redwork(c, 1, n);
-    rw.grid = reduction_grid(L0.nslices * kSlice, c->nsm);
-    for (int i = 0; i < m; ++i) {
-      double* e = E + (size_t)i * n;
-      for (int q = 0; q < cycles; ++q) {
-        launch_spmv_dot(A, e, c->pp, rw, c->dscal, s);  // r = A e
-        with_engine(c, [&](auto eng) { decltype(eng)::vcycle(c, c->pp, c->pz); });
-        launch_sub(n, e, c->pz, e, s);                   // e <- (I - B A) e
+    const int B = cycles > 0 ? batch_size(c, m, false) : 1;
+    std::unique_ptr<Batch> bt;
+    if (B > 1) {
+      bt.reset(new Batch(c, B, false));
+      if (!bt->ok()) bt.reset();
+    }
+    if (bt) {
+      CK(cudaMemsetAsync(bt->rw.counter, 0, B * sizeof(unsigned), s));
+      for (int i = 0; i < m; i += B) {
+        const int nv = std::min(B, m - i);
+        bt->size(nv);
+        double* e = E + (size_t)i * n;
+        for (int q = 0; q < cycles; ++q) {
+          launch_spmv_dot_mv(A, e, bt->r, bt->rw, bt->dots, 1, nv, s);  // r = A e
+          Engine<double, double>::vcycle_level(c, 0, bt->r, bt->z);
+          launch_sub(n * nv, e, bt->z, e, s);                           // e <- (I - B A) e
+        }
+      }
+      bt.reset();
+    } else {
+      RedWork rw = redwork(c, 1, n);
+      rw.grid = reduction_grid(L0.nslices * kSlice, c->nsm);
+      for (int i = 0; i < m; ++i) {
+        double* e = E + (size_t)i * n;
+        for (int q = 0; q < cycles; ++q) {
+          launch_spmv_dot(A, e, c->pp, rw, c->dscal, s);  // r = A e
+          with_engine(c, [&](auto eng) { decltype(eng)::vcycle(c, c->pp, c->pz); });
+          launch_sub(n, e, c->pz, e, s);                   // e <- (I - B A) e
+        }
       }
     }
     check_launch();

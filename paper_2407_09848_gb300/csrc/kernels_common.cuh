@@ -280,6 +280,79 @@ __device__ __forceinline__ void step_slice(const StepArgs<VT, XT>& a, int64_t s,
   step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, row, acc, rin, xin, di, zo);
 }
 
+// The same step for vectors v0 .. v1-1 of a batch (vector v at +v n of every
+// vector argument): a 7-point slice loads its values, columns and 1/M once for
+// all of them.  Each vector's operations and their order are those of
+// step_slice.
+template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
+__device__ __forceinline__ void step_slice_mv(const StepArgs<VT, XT>& a, int64_t s, int lane,
+                                              int v0, int v1) {
+  const int64_t n = a.A.n, row = s * kSlice + lane;
+  const SliceDesc d = ld_desc(a.A.sd + s);
+  constexpr int kSign = StepForm<FAM, INIT>::kSign;
+  if (d.w == 7) {
+    // a lane past n works on row n - 1 and stores nothing
+    const bool live = row < n;
+    const int64_t lr = live ? row : n - 1;
+    XT av[7];
+    int32_t cv[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+      const int64_t e = d.vbase + (int64_t)k * kSlice + lane;
+      av[k] = XT(__ldg(a.A.val + e));
+      if (d.cref >= 0) {
+        const int64_t cc = row + (int64_t)__ldg(a.A.off + d.cref + k);
+        cv[k] = (int32_t)(cc < 0 ? 0 : (cc > n - 1 ? n - 1 : cc));
+      } else {
+        cv[k] = __ldg(a.A.col + e);
+      }
+    }
+    XT di = XT(0);
+    if (step_needs_dinv<FAM>()) di = __ldg(a.dinv + lr);
+    pdl_wait();
+    pdl_go();
+    for (int v = v0; v < v1; ++v) {
+      const int64_t o = v * n, ro = o + lr;
+      XT rin = XT(0), xin = XT(0), zo = XT(0), uc = XT(0), uv[7], t;
+      if constexpr (is_op(FAM)) {
+        if (reads_slot0<FAM, INIT>()) rin = ldv<false>(a.rin + ro);
+        if (reads_slot1<FAM, ZOWN>()) xin = ldv<false>(a.xin + ro);
+        if (FAM == FAM_OPT && WR) uc = ldv<false>(a.u + ro);
+      } else {
+        rin = ldv<false>(a.rin + ro);
+        if (FAM != FAM_RES) xin = ldv<false>(a.xin + ro);
+        if (ZOWN) zo = ldv<false>(a.zown + ro);
+      }
+      const XT* u = a.u + o;
+#pragma unroll
+      for (int k = 0; k < 7; ++k) uv[k] = ldv<false>(u + cv[k]);
+      if constexpr (is_op(FAM)) t = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, rin, xin);
+      else t = step_init<FAM, StepForm<FAM, INIT>::kResidual>(rin, di);
+#pragma unroll
+      for (int k = 0; k < 7; ++k) t = fma(kSign > 0 ? av[k] : -av[k], uv[k], t);
+      if (live) {
+        if constexpr (is_op(FAM)) op_finish<VT, XT, FAM, WR>(a, ro, t, uc);
+        else step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, ro, t, rin, xin, di, zo);
+      }
+    }
+    return;
+  }
+  pdl_wait();
+  pdl_go();
+  for (int v = v0; v < v1; ++v) {
+    StepArgs<VT, XT> b = a;
+    const int64_t o = v * n;
+    b.u += o;
+    if (b.rin) b.rin += o;
+    if (b.rout) b.rout += o;
+    if (b.zown) b.zown += o;
+    if (b.zout) b.zout += o;
+    if (b.xin) b.xin += o;
+    if (b.xout) b.xout += o;
+    step_slice<VT, XT, FAM, INIT, WR, ZOWN>(b, s, lane);
+  }
+}
+
 // Per-element bodies of the elementwise V-cycle kernels, shared by their own
 // launches (kernels_smooth.cu, kernels_krylov.cu) and by the persistent
 // coarse-level kernel (kernels_cycle.cu), so both give the same bits.
@@ -348,13 +421,13 @@ __device__ __forceinline__ void prolong_row(int64_t i, const int32_t* agg, const
 
 // x_i = (A_c^{-1} b)_i for the coarsest level, one warp per row: lane l sums
 // columns l, l + 32, ... in order, then a fixed butterfly adds the lanes.  The
-// first 16 entries of a lane (512 columns) are loaded together, before the wait.
+// first 16 entries of a lane (512 columns) are loaded together, before the
+// wait, and serve all nv vectors (vector v at b + v nc, x + v nc).
 template <class XT, bool CG = false, bool WAIT = false>
 __device__ __forceinline__ void coarse_gemv_row(int i, int nc, const double* ainv, const XT* b,
-                                                XT* x, int lane) {
+                                                XT* x, int lane, int nv = 1) {
   const double* row = ainv + (size_t)i * nc;
   double av[16];
-  XT bv[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k)
     if (lane + 32 * k < nc) av[k] = __ldg(row + lane + 32 * k);
@@ -362,17 +435,21 @@ __device__ __forceinline__ void coarse_gemv_row(int i, int nc, const double* ain
     pdl_wait();
     pdl_go();
   }
+  for (int v = 0; v < nv; ++v, b += nc, x += nc) {
+    XT bv[16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (lane + 32 * k < nc) bv[k] = ldv<CG>(b + lane + 32 * k);
-  double acc = 0.0;
+    for (int k = 0; k < 16; ++k)
+      if (lane + 32 * k < nc) bv[k] = ldv<CG>(b + lane + 32 * k);
+    double acc = 0.0;
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    if (lane + 32 * k < nc) acc = fma(av[k], (double)bv[k], acc);
-  for (int j = lane + 512; j < nc; j += 32) acc = fma(__ldg(row + j), (double)ldv<CG>(b + j), acc);
+    for (int k = 0; k < 16; ++k)
+      if (lane + 32 * k < nc) acc = fma(av[k], (double)bv[k], acc);
+    for (int j = lane + 512; j < nc; j += 32)
+      acc = fma(__ldg(row + j), (double)ldv<CG>(b + j), acc);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) x[i] = XT(acc);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) x[i] = XT(acc);
+  }
 }
 
 // Sum over a block (any blockDim multiple of 32, <= 1024); result valid in thread 0.

@@ -55,6 +55,37 @@ void launch_spmv_dot(const DevMat<double>& A, const double* p, double* q, const 
   launch_dep(k_spmv_dot, w.grid, kBlock, 0, s, A, p, q, w, scal);
 }
 
+// A batch of products: blockIdx.y is the vector, with its own row of partials
+// and its own counter.
+__global__ void __launch_bounds__(kBlock, 4) k_spmv_dot_mv(const DevMat<double> A, const double* p,
+                                                           double* q, RedWork w, double* out,
+                                                           int stride) {
+  pdl_wait();
+  pdl_go();
+  const int lane = threadIdx.x & 31, v = blockIdx.y;
+  p += v * A.n;
+  q += v * A.n;
+  w.part += (size_t)v * gridDim.x;
+  w.counter += v;
+  const int64_t nw = (int64_t)gridDim.x * kWarpsPerBlock;
+  double acc = 0.0;
+  for (int64_t s = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); s < A.nslices;
+       s += nw) {
+    const int64_t row = s * kSlice + lane;
+    const double t = row_spmv<1, double, double>(A, s, lane, row, p, 0.0);
+    if (row < A.n) {
+      q[row] = t;
+      acc = fma(ldv<false>(p + row), t, acc);
+    }
+  }
+  grid_sum(acc, w, [&](double tot) { out[v * stride] = tot; });
+}
+
+void launch_spmv_dot_mv(const DevMat<double>& A, const double* p, double* q, const RedWork& w,
+                        double* out, int stride, int nvec, cudaStream_t s) {
+  launch_dep(k_spmv_dot_mv, dim3(w.grid, nvec), kBlock, 0, s, A, p, q, w, out, stride);
+}
+
 // Three sums in one pass (the one-reduction flexible CG): partials are laid
 // out [v0 of every block | v1 ... | v2 ...] in w.part (3 x grid doubles); the
 // last block adds each column in index order and calls fin(t0, t1, t2).
@@ -278,37 +309,42 @@ void launch_sub(int64_t n, const double* x, const double* y, double* out, cudaSt
 }
 
 __global__ void __launch_bounds__(kBlock) k_scale_dev(int64_t n, const double* x, double* out,
-                                                      const double* sd, double factor) {
+                                                      const double* sd, int stride,
+                                                      double factor) {
   pdl_wait();
   pdl_go();
-  const double f = factor / ldv<false>(sd);
-  const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (i < n) out[i] = f * ldv<false>(x + i);
+  const double f = factor / ldv<false>(sd + blockIdx.y * stride);
+  const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x, o = blockIdx.y * n;
+  if (i < n) out[o + i] = f * ldv<false>(x + o + i);
 }
 
-void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, double factor,
-                      cudaStream_t s) {
+void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, int stride,
+                      double factor, int nvec, cudaStream_t s) {
   if (n == 0) return;
-  launch_dep(k_scale_dev, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, x, out, s_dev,
-             factor);
+  launch_dep(k_scale_dev, dim3((unsigned)((n + kBlock - 1) / kBlock), nvec), kBlock, 0, s, n, x,
+             out, s_dev, stride, factor);
 }
 
 // Coarsest level: x = A_c^{-1} b with the inverse formed at load time from the
 // Cholesky factor (FP64).  One warp per row, lanes stride the columns.
+constexpr int kGemvVecs = 4;  // vectors of a batch per warp (one read of the row)
 template <class XT>
 __global__ void __launch_bounds__(kBlock) k_coarse_gemv(int nc, const double* __restrict__ ainv,
-                                                        const XT* b, XT* x) {
+                                                        const XT* b, XT* x, int nvec) {
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   if (i >= nc) return;
-  coarse_gemv_row<XT, false, true>(i, nc, ainv, b, x, lane);
+  const int v0 = blockIdx.y * kGemvVecs;
+  const size_t o = (size_t)v0 * nc;
+  coarse_gemv_row<XT, false, true>(i, nc, ainv, b + o, x + o, lane, min(kGemvVecs, nvec - v0));
 }
 
 template <class XT>
-void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, cudaStream_t s) {
+void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, int nvec,
+                        cudaStream_t s) {
   if (nc == 0) return;
-  launch_dep(k_coarse_gemv<XT>, (nc + kWarpsPerBlock - 1) / kWarpsPerBlock, kBlock, 0, s, nc, ainv,
-             b, x);
+  const dim3 g((nc + kWarpsPerBlock - 1) / kWarpsPerBlock, (nvec + kGemvVecs - 1) / kGemvVecs);
+  launch_dep(k_coarse_gemv<XT>, g, kBlock, 0, s, nc, ainv, b, x, nvec);
 }
 
 // Dense Cholesky A = L L^T (right-looking, one block, in place in `work`,
@@ -435,8 +471,10 @@ void launch_norm2(int64_t n, const XT* v, const RedWork& rw, double* scal, int s
   count_launch();
 }
 
-template void launch_coarse_gemv<double>(int, const double*, const double*, double*, cudaStream_t);
-template void launch_coarse_gemv<float>(int, const double*, const float*, float*, cudaStream_t);
+template void launch_coarse_gemv<double>(int, const double*, const double*, double*, int,
+                                         cudaStream_t);
+template void launch_coarse_gemv<float>(int, const double*, const float*, float*, int,
+                                        cudaStream_t);
 template void launch_power_step<double, double>(const DevMat<double>&, const double*, const double*,
                                                 double*, const RedWork&, double*, cudaStream_t);
 template void launch_power_step<float, float>(const DevMat<float>&, const float*, const float*,

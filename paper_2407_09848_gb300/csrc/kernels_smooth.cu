@@ -43,6 +43,18 @@ __global__ void __launch_bounds__(kBlock, 4) k_step(const StepArgs<VT, XT> a) {
   step_slice<VT, XT, FAM, INIT, WR, ZOWN, false, true>(a, s, lane);
 }
 
+// Vectors of a batch that one warp takes through its slice: the 7-point values
+// (56 B a row, more than half of a step's bytes) are then read once for four
+// vectors, and the step is bound by FP64 issue alone.
+constexpr int kVecs = 4;
+template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
+__global__ void __launch_bounds__(kBlock, 3) k_step_mv(const StepArgs<VT, XT> a) {
+  const int64_t s = (int64_t)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+  if (s >= a.A.nslices) return;
+  const int v0 = blockIdx.y * kVecs;
+  step_slice_mv<VT, XT, FAM, INIT, WR, ZOWN>(a, s, threadIdx.x & 31, v0, min(v0 + kVecs, a.nvec));
+}
+
 // Split form for levels with wide rows: one block per slice, a.split warps;
 // warp g sums entries [g w / G, (g+1) w / G) of each row, warp 0 adds the
 // partials in warp order (deterministic) and finishes the rows.
@@ -84,6 +96,15 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
 
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
 static void go(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
+  if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
+    if (a.nvec > 1) {  // batches run on levels of one warp per slice, all slices
+      launch_dep(k_step_mv<VT, XT, FAM, INIT, WR, ZOWN>,
+                 dim3((unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock),
+                      (a.nvec + kVecs - 1) / kVecs),
+                 kBlock, 0, s, a);
+      return;
+    }
+  }
   if (a.split > 1)
     launch_dep(k_step_split<VT, XT, FAM, INIT, WR, ZOWN>, (unsigned)work, 32 * a.split, 0, s, a);
   else
@@ -108,19 +129,18 @@ static void dispatch_wr(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s)
 template <class VT, class XT>
 static void dispatch_op(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
   if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
-    const unsigned g = (unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock);
     const bool s0 = a.rin != nullptr, s1 = a.xin != nullptr, wr = a.write_r;
     if (a.fam == FAM_OPT) {
-      if (wr) launch_dep(k_step<VT, XT, FAM_OPT, true, true, false>, g, kBlock, 0, s, a);
-      else launch_dep(k_step<VT, XT, FAM_OPT, true, false, false>, g, kBlock, 0, s, a);
+      if (wr) go<VT, XT, FAM_OPT, true, true, false>(a, work, s);
+      else go<VT, XT, FAM_OPT, true, false, false>(a, work, s);
     } else if (!s0) {
-      launch_dep(k_step<VT, XT, FAM_OP, false, false, false>, g, kBlock, 0, s, a);
+      go<VT, XT, FAM_OP, false, false, false>(a, work, s);
     } else if (!s1) {
-      if (wr) launch_dep(k_step<VT, XT, FAM_OP, true, true, false>, g, kBlock, 0, s, a);
-      else launch_dep(k_step<VT, XT, FAM_OP, true, false, false>, g, kBlock, 0, s, a);
+      if (wr) go<VT, XT, FAM_OP, true, true, false>(a, work, s);
+      else go<VT, XT, FAM_OP, true, false, false>(a, work, s);
     } else {
-      if (wr) launch_dep(k_step<VT, XT, FAM_OP, true, true, true>, g, kBlock, 0, s, a);
-      else launch_dep(k_step<VT, XT, FAM_OP, true, false, true>, g, kBlock, 0, s, a);
+      if (wr) go<VT, XT, FAM_OP, true, true, true>(a, work, s);
+      else go<VT, XT, FAM_OP, true, false, true>(a, work, s);
     }
   }
 }
@@ -173,14 +193,15 @@ __global__ void __launch_bounds__(kBlock) k_first(int64_t n, const XT* b,
   const XT di = dinv[i];
   pdl_wait();
   pdl_go();
-  first_row<XT, FAM>(i, b, di, rout, zout, xout, c2, beta, rhoinv);
+  const int64_t o = (int64_t)blockIdx.y * n;  // vector of a batch
+  first_row<XT, FAM>(i, b + o, di, rout + o, zout + o, xout + o, c2, beta, rhoinv);
 }
 
 template <class XT>
 void launch_first(int fam, int64_t n, const XT* b, const XT* dinv, XT* rout, XT* zout, XT* xout,
-                  XT c2, XT beta, XT rhoinv, cudaStream_t s) {
+                  XT c2, XT beta, XT rhoinv, int nvec, cudaStream_t s) {
   if (n == 0) return;
-  const unsigned g = (unsigned)((n + kBlock - 1) / kBlock);
+  const dim3 g((unsigned)((n + kBlock - 1) / kBlock), nvec);
   auto* k = fam == FAM_CHEB4   ? k_first<XT, FAM_CHEB4>
             : fam == FAM_CHEB1 ? k_first<XT, FAM_CHEB1>
                                : k_first<XT, FAM_JAC>;
@@ -193,33 +214,36 @@ void launch_first(int fam, int64_t n, const XT* b, const XT* dinv, XT* rout, XT*
 // from the FAM_RES step (pipelined and coalesced like the smoother steps).
 template <class XT>
 __global__ void __launch_bounds__(kBlock, 6) k_aggregate(const int32_t* __restrict__ cptr,
-                                                      const int32_t* __restrict__ cidx, int64_t nc,
-                                                      const XT* res, XT* bc) {
+                                                      const int32_t* __restrict__ cidx, int64_t n,
+                                                      int64_t nc, const XT* res, XT* bc) {
   const int64_t I = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (I >= nc) return;
-  aggregate_row<XT, false, true>(I, cptr, cidx, res, bc);
+  aggregate_row<XT, false, true>(I, cptr, cidx, res + blockIdx.y * n, bc + blockIdx.y * nc);
 }
 
 template <class XT>
-void launch_aggregate(const int32_t* cptr, const int32_t* cidx, int64_t nc, const XT* res, XT* bc,
-                      cudaStream_t s) {
+void launch_aggregate(const int32_t* cptr, const int32_t* cidx, int64_t n, int64_t nc,
+                      const XT* res, XT* bc, int nvec, cudaStream_t s) {
   if (nc == 0) return;
-  const unsigned g = (unsigned)((nc + kBlock - 1) / kBlock);
-  launch_dep(k_aggregate<XT>, g, kBlock, 0, s, cptr, cidx, nc, res, bc);
+  const dim3 g((unsigned)((nc + kBlock - 1) / kBlock), nvec);
+  launch_dep(k_aggregate<XT>, g, kBlock, 0, s, cptr, cidx, n, nc, res, bc);
 }
 
 // x += P e_c (gather through the aggregate map).
 template <class XT>
-__global__ void __launch_bounds__(kBlock) k_prolong(int64_t n, const int32_t* __restrict__ agg,
-                                                    const XT* ec, XT* x) {
+__global__ void __launch_bounds__(kBlock) k_prolong(int64_t n, int64_t nc,
+                                                    const int32_t* __restrict__ agg, const XT* ec,
+                                                    XT* x) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
-  if (i < n) prolong_row<XT, false, true>(i, agg, ec, x);
+  if (i < n) prolong_row<XT, false, true>(i, agg, ec + blockIdx.y * nc, x + blockIdx.y * n);
 }
 
 template <class XT>
-void launch_prolong(int64_t n, const int32_t* agg, const XT* ec, XT* x, cudaStream_t s) {
+void launch_prolong(int64_t n, int64_t nc, const int32_t* agg, const XT* ec, XT* x, int nvec,
+                    cudaStream_t s) {
   if (n == 0) return;
-  launch_dep(k_prolong<XT>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, agg, ec, x);
+  const dim3 g((unsigned)((n + kBlock - 1) / kBlock), nvec);
+  launch_dep(k_prolong<XT>, g, kBlock, 0, s, n, nc, agg, ec, x);
 }
 
 template <class XT>
@@ -327,16 +351,18 @@ AMGPS_INST(__nv_bfloat16, float)
 #undef AMGPS_INST
 
 template void launch_first<double>(int, int64_t, const double*, const double*, double*, double*,
-                                   double*, double, double, double, cudaStream_t);
+                                   double*, double, double, double, int, cudaStream_t);
 template void launch_first<float>(int, int64_t, const float*, const float*, float*, float*,
-                                  float*, float, float, float, cudaStream_t);
-template void launch_aggregate<double>(const int32_t*, const int32_t*, int64_t, const double*,
-                                       double*, cudaStream_t);
-template void launch_aggregate<float>(const int32_t*, const int32_t*, int64_t, const float*, float*,
-                                      cudaStream_t);
-template void launch_prolong<double>(int64_t, const int32_t*, const double*, double*, cudaStream_t);
+                                  float*, float, float, float, int, cudaStream_t);
+template void launch_aggregate<double>(const int32_t*, const int32_t*, int64_t, int64_t, const double*,
+                                       double*, int, cudaStream_t);
+template void launch_aggregate<float>(const int32_t*, const int32_t*, int64_t, int64_t, const float*,
+                                       float*, int, cudaStream_t);
+template void launch_prolong<double>(int64_t, int64_t, const int32_t*, const double*, double*, int,
+                                     cudaStream_t);
 template void launch_add<double>(int64_t, const double*, const double*, double*, cudaStream_t);
-template void launch_prolong<float>(int64_t, const int32_t*, const float*, float*, cudaStream_t);
+template void launch_prolong<float>(int64_t, int64_t, const int32_t*, const float*, float*, int,
+                                     cudaStream_t);
 template void launch_convert<double, float>(int64_t, const double*, float*, cudaStream_t);
 template void launch_convert<float, double>(int64_t, const float*, double*, cudaStream_t);
 template void launch_convert<double, double>(int64_t, const double*, double*, cudaStream_t);

@@ -25,6 +25,10 @@ struct RedWork {
 // ---- launchers (kernels_krylov.cu) ----
 void launch_spmv_dot(const DevMat<double>& A, const double* p, double* q, const RedWork& w,
                      double* scal, cudaStream_t s);
+// nvec products: vector v has q + v n = A (p + v n), out[v stride] = p.q of it.
+// w.grid blocks a vector; w.part and w.counter hold nvec x grid and nvec entries
+void launch_spmv_dot_mv(const DevMat<double>& A, const double* p, double* q, const RedWork& w,
+                        double* out, int stride, int nvec, cudaStream_t s);
 // one-reduction flexible CG: w = A z with z.r, z.q, z.w in one reduction
 // (first = 1: no q yet), then p = z - beta p, q = w - beta q, x += alpha p,
 // r -= alpha q, r.r
@@ -47,7 +51,7 @@ void launch_xpay_x(int64_t n, const double* z, double* p, double* x, const doubl
 void launch_dot(int64_t n, const double* a, const double* b, const RedWork& w, double* scal,
                 int out_slot, int rz_mode, cudaStream_t s);
 template <class XT>
-void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, cudaStream_t s);
+void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, int nvec, cudaStream_t s);
 void launch_chol_inverse(int n, double* work, double* ainv, int* status, cudaStream_t s);
 template <class VT, class XT>
 void launch_power_step(const DevMat<VT>& A, const XT* v, const XT* dinv, XT* w, const RedWork& rw,
