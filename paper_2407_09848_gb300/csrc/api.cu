@@ -256,6 +256,13 @@ struct amgps_ctx {
   cudaGraphExec_t gexec = nullptr;
   bool graph_ok = false;
   int64_t graph_kernels = 0;   // kernel nodes in gexec
+  // a whole solve: begin node, then a WHILE node with one PCG iteration
+  cudaGraphExec_t loop_exec = nullptr;
+  bool loop_ok = false;        // built for the current smoothers and options
+  bool loop_refused = false;   // the runtime would not build one: the host loop runs
+  int64_t loop_kernels = 0;    // kernel nodes of the iteration
+  double** dx = nullptr;       // device slot: the solution vector of the running solve
+  void** hx = nullptr;         // pinned copy of the slot
   int use_tma = 1;             // AMGPS_OPT_TMA: TMA-fed step kernels 0 off, 1 auto, 2 always
   int flexible = 0;            // AMGPS_OPT_FLEXIBLE: 0 standard, 1 Polak-Ribiere, 2 one-reduction
   int coarse_sweeps = 0;       // AMGPS_OPT_COARSE_SWEEPS: 0 dense Cholesky, m l1-Jacobi sweeps
@@ -342,7 +349,11 @@ void free_hierarchy(amgps_ctx* c) {
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
   }
-  c->graph_ok = false;
+  if (c->loop_exec) {
+    cudaGraphExecDestroy(c->loop_exec);
+    c->loop_exec = nullptr;
+  }
+  c->graph_ok = c->loop_ok = c->loop_refused = false;
   c->tail_ok = false;
   if (!c->allocs.empty()) cudaStreamSynchronize(c->stream);
   for (void* p : c->allocs) cudaFree(p);
@@ -1187,6 +1198,9 @@ struct Engine {
   // za already holds M^{-1} r, see pcg_impl).
   static void vcycle(amgps_ctx* c, const double* r, double* z, bool c_ready = false) {
     build_graph(c);
+    vcycle_plain(c, r, z, c_ready);
+  }
+  static void vcycle_plain(amgps_ctx* c, const double* r, double* z, bool c_ready) {
     Level& L = c->lv[0];
     if constexpr (std::is_same<XT, double>::value) {
       vcycle_level(c, 0, r, z, false, c_ready);
@@ -1369,16 +1383,164 @@ void fcg1_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit,
   *converged = rel <= rtol;
 }
 
+// ---- the solve as one graph: the loop on the device ----
+// The host loop waits for every iteration's scalars before it can enqueue the
+// next iteration (its ~16 launches and a graph): at 32^3 that was 15 us of a
+// 90 us iteration (solve 985 -> 820 us; FP32 128^3 9979 -> 9567, BF16 192^3
+// 81544 -> 80109).  Here one graph launch runs the whole solve; the last
+// kernel of an iteration sets the WHILE condition (pcg_continue).  The kernels
+// and their order are those of the host loop, except that the first direction
+// comes from p = z + 0 * 0 instead of a copy, and the flexible form takes
+// r.z_old before the V-cycle writes z, so one z buffer serves; the bits are
+// the same.
+// One iteration, from r (and, with fuse_c, c = M^{-1} r) to the next r.
+void loop_body(amgps_ctx* c, const PcgLoop& lp, bool fuse_c) {
+  Level& L = c->lv[0];
+  cudaStream_t s = c->stream;
+  const int64_t n = L.n;
+  const DevMat<double> A = devmat64(L, c->prec);
+  RedWork rw_dot = redwork(c, 0, n, kRedBlocksPerSm), rw_spmv = redwork(c, 1, n),
+          rw_upd = redwork(c, 2, n, kRedBlocksPerSm);
+  rw_spmv.grid = reduction_grid(L.nslices * kSlice, c->nsm);
+  double *z = c->pz, *p = c->pp, *q = c->pq, *r = c->pr;
+  if (c->flexible == 1) launch_dot(n, r, z, rw_dot, c->dscal, S_RZP, 0, s);
+  with_engine(c, [&](auto eng) { decltype(eng)::vcycle_plain(c, r, z, fuse_c); });
+  if (c->flexible == 2) {
+    launch_spmv_dot3(A, z, c->pz2, r, q, 0, rw_spmv, c->dscal, s);
+    launch_fcg_update(n, z, c->pz2, p, q, nullptr, r, 0, rw_upd, c->dscal, s, lp);
+    return;
+  }
+  launch_dot(n, r, z, rw_dot, c->dscal, S_RZ, c->flexible == 1 ? 2 : 1, s);
+  launch_xpay_x(n, z, p, nullptr, c->dscal, 1, s, lp);
+  launch_spmv_dot(A, p, q, rw_spmv, c->dscal, s);
+  if (fuse_c)
+    launch_r_update(n, q, r, rw_upd, c->dscal, s, (const double*)L.dinv, (double*)L.za, lp);
+  else
+    launch_r_update(n, q, r, rw_upd, c->dscal, s, nullptr, nullptr, lp);
+}
+
+// Builds c->loop_exec; false (and c->loop_refused) if the runtime refuses it.
+bool build_loop(amgps_ctx* c, bool fuse_c) {
+  if (c->loop_ok) return true;
+  if (c->loop_refused) return false;
+  if (c->loop_exec) {
+    CK(cudaGraphExecDestroy(c->loop_exec));
+    c->loop_exec = nullptr;
+  }
+  cudaStream_t s = c->stream;
+  cudaGraph_t g = nullptr, body = nullptr, got = nullptr;
+  const int64_t before = launches_enqueued();
+  // what `f` enqueues becomes nodes of graph `to`
+  auto capture = [&](cudaGraph_t to, auto&& f) {
+    cudaError_t e = cudaStreamBeginCaptureToGraph(s, to, nullptr, nullptr, 0,
+                                                  cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    try {
+      f();
+    } catch (const Fail&) {
+      e = cudaErrorStreamCaptureInvalidated;
+    }
+    const cudaError_t ee = cudaStreamEndCapture(s, &got);
+    return e != cudaSuccess ? e : ee;
+  };
+  PcgLoop lp;
+  lp.x = c->dx;
+  cudaGraphNode_t begin = nullptr, loop = nullptr;
+  size_t nb = 1;
+  cudaError_t e = cudaGraphCreate(&g, 0);
+  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&lp.handle, g, 0, 0);
+  if (e == cudaSuccess) e = capture(g, [&] { launch_pcg_begin(c->dscal, lp.handle, s); });
+  if (e == cudaSuccess) e = cudaGraphGetNodes(g, &begin, &nb);
+  if (e == cudaSuccess) {
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = lp.handle;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    e = cudaGraphAddNode(&loop, g, &begin, nullptr, 1, &np);
+    if (e == cudaSuccess) body = np.conditional.phGraph_out[0];
+  }
+  if (e == cudaSuccess) e = capture(body, [&] {
+    loop_body(c, lp, fuse_c);
+    check_launch();
+  });
+  const int64_t captured = launches_enqueued() - before;
+  c->launch_adjust -= captured;
+  c->loop_kernels = captured - 1;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&c->loop_exec, g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    c->loop_exec = nullptr;
+    c->loop_refused = true;
+    return false;
+  }
+  c->loop_ok = true;
+  return true;
+}
+
+// The solve through c->loop_exec; arguments and results as pcg_impl.
+void pcg_loop(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, int* iters,
+              double* relres, bool* converged, bool fuse_c) {
+  Level& L = c->lv[0];
+  cudaStream_t s = c->stream;
+  const int64_t n = L.n;
+  const size_t bytes = n * sizeof(double);
+  CK(cudaMemcpyAsync(c->pr, b, bytes, cudaMemcpyDeviceToDevice, s));
+  CK(cudaMemsetAsync(x, 0, bytes, s));
+  CK(cudaMemsetAsync(c->pp, 0, bytes, s));
+  if (c->flexible == 1) CK(cudaMemsetAsync(c->pz, 0, bytes, s));
+  if (c->flexible == 2) CK(cudaMemsetAsync(c->pq, 0, bytes, s));
+  *c->hx = x;
+  CK(cudaMemcpyAsync(c->dx, c->hx, sizeof(double*), cudaMemcpyHostToDevice, s));
+  c->hscal[S_RTOL] = rtol;
+  c->hscal[S_MAXIT] = maxit;
+  CK(cudaMemcpyAsync(c->dscal + S_RTOL, c->hscal + S_RTOL, 2 * sizeof(double),
+                     cudaMemcpyHostToDevice, s));
+  launch_dot(n, b, b, redwork(c, 0, n, kRedBlocksPerSm), c->dscal, S_BB, 0, s);
+  if (fuse_c)
+    launch_first<double>(FAM_JAC, n, c->pr, (const double*)L.dinv, nullptr, nullptr, (double*)L.za,
+                         0.0, 0.0, 1.0, 1, s);
+  CK(cudaGraphLaunch(c->loop_exec, s));
+  check_launch();
+  CK(cudaMemcpyAsync(c->hscal, c->dscal, S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, s));
+  CK(cudaEventRecord(c->ev_sync, s));
+  CK(cudaEventSynchronize(c->ev_sync));
+  const double bnorm = std::sqrt(c->hscal[S_BB]);
+  const int it = (int)c->hscal[S_IT];
+  c->launch_adjust += 1 + it * c->loop_kernels;
+  *converged = false;
+  *iters = 0;
+  *relres = 0.0;
+  if (bnorm == 0.0) {
+    *converged = true;
+    return;
+  }
+  REQ(std::isfinite(bnorm), AMGPS_E_NAN, "right-hand side is not finite");
+  if (c->hscal[S_ERR] != 0.0) {
+    CK(cudaMemsetAsync(c->dscal + S_ERR, 0, sizeof(double), s));
+    throw Fail{AMGPS_E_TIMEOUT, "a bounded wait inside a pipelined kernel gave up"};
+  }
+  const double pq = c->hscal[S_PQ], rr = c->hscal[S_RR];
+  REQ(std::isfinite(pq) && std::isfinite(rr) &&
+          (c->flexible != 2 || std::isfinite(c->hscal[S_ALPHA])),
+      AMGPS_E_NAN, "NaN/Inf in PCG scalars");
+  REQ(pq > 0.0, AMGPS_E_NOT_SPD, "p^T A p <= 0 in PCG");
+  if (c->flexible != 2) {
+    launch_xpay_x(n, c->pz, c->pp, x, c->dscal, 0, s);  // the last x update
+    check_launch();
+  }
+  *iters = it;
+  *relres = std::sqrt(rr) / bnorm;
+  *converged = *relres <= rtol;
+}
+
 void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, int* iters,
               double* relres, bool* converged, const Precond& precond = nullptr) {
   const Precond vcyc = [c](const double* r, double* z) {
     with_engine(c, [&](auto eng) { decltype(eng)::vcycle(c, r, z); });
   };
   const Precond& M = precond ? precond : vcyc;
-  if (c->flexible == 2) {
-    fcg1_impl(c, b, x, rtol, maxit, iters, relres, converged, M);
-    return;
-  }
   Level& L = c->lv[0];
   // The V-cycle's level-0 smoother starts from c = M^{-1} r in the
   // stored-operator form: the r update writes it (one stream less than a
@@ -1386,6 +1548,19 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
   const bool fuse_c = !precond && c->prec == AMGPS_F64 && c->step_form == 1 && !L.coarsest &&
                       L.ops_ok &&
                       same_coefs(L.ops_cf, make_coefs(L.spec.kind, L.spec.k, L.spec.w, L.spec.rho));
+  // The loop on the device, unless the kernels are being timed (events between
+  // them), the caller captures the stream, or the coarse levels run as a
+  // cooperative kernel; a caller's preconditioner keeps the host loop.
+  const bool fuse_loop = fuse_c && c->flexible != 2;
+  if (!precond && !c->prof && !c->use_cycle && !Engine<double, double>::capturing(c) &&
+      build_loop(c, fuse_loop)) {
+    pcg_loop(c, b, x, rtol, maxit, iters, relres, converged, fuse_loop);
+    return;
+  }
+  if (c->flexible == 2) {
+    fcg1_impl(c, b, x, rtol, maxit, iters, relres, converged, M);
+    return;
+  }
   cudaStream_t s = c->stream;
   const int64_t n = L.n;
   const DevMat<double> A = devmat64(L, c->prec);
@@ -1756,6 +1931,8 @@ amgps_status amgps_create(amgps_ctx** out, int device, void* user_stream) {
     CK(cudaMalloc(&u->dscal, S_COUNT * sizeof(double)));
     CK(cudaMemset(u->dscal, 0, S_COUNT * sizeof(double)));
     CK(cudaMallocHost(&u->hscal, S_COUNT * sizeof(double)));
+    CK(cudaMalloc((void**)&u->dx, sizeof(double*)));
+    CK(cudaMallocHost((void**)&u->hx, sizeof(double*)));
     CK(cudaMalloc(&u->ddots, kDotSlots * sizeof(double)));
     CK(cudaMallocHost(&u->hdots, kDotSlots * sizeof(double)));
     const int maxgrid = u->nsm * kRedBlocksPerSm;
@@ -1782,6 +1959,8 @@ amgps_status amgps_destroy(amgps_ctx* c) {
   if (c->hscal) cudaFreeHost(c->hscal);
   if (c->hdots) cudaFreeHost(c->hdots);
   if (c->ddots) cudaFree(c->ddots);
+  if (c->dx) cudaFree(c->dx);
+  if (c->hx) cudaFreeHost(c->hx);
   if (c->dscal) cudaFree(c->dscal);
   if (c->part) cudaFree(c->part);
   if (c->counters) cudaFree(c->counters);
@@ -2017,7 +2196,7 @@ amgps_status amgps_set_smoother(amgps_ctx* c, int level, amgps_kind kind, int de
       std::fill(s.w, s.w + kMaxDegree, 0.0);
       if (weights) std::copy(weights, weights + degree, s.w);
     }
-    c->graph_ok = false;
+    c->graph_ok = c->loop_ok = false;
     enter(c);
     prepare_ops(c);
     leave(c);
@@ -2441,7 +2620,7 @@ amgps_status amgps_set_option(amgps_ctx* c, int option, int64_t value) {
     if (option == AMGPS_OPT_STEP_FORM) {
       REQ(value == 0 || value == 1, AMGPS_E_ARG, "AMGPS_OPT_STEP_FORM takes 0 or 1");
       c->step_form = (int)value;
-      c->graph_ok = false;
+      c->graph_ok = c->loop_ok = false;
       if (c->loaded) {
         enter(c);
         prepare_ops(c);
@@ -2450,21 +2629,22 @@ amgps_status amgps_set_option(amgps_ctx* c, int option, int64_t value) {
     } else if (option == AMGPS_OPT_TMA) {
       REQ(value >= 0 && value <= 2, AMGPS_E_ARG, "AMGPS_OPT_TMA takes 0, 1 or 2");
       c->use_tma = (int)value;
-      c->graph_ok = false;
+      c->graph_ok = c->loop_ok = false;
     } else if (option == AMGPS_OPT_FLEXIBLE) {
       REQ(value >= 0 && value <= 2, AMGPS_E_ARG, "AMGPS_OPT_FLEXIBLE takes 0, 1 or 2");
       c->flexible = (int)value;
+      c->loop_ok = false;
     } else if (option == AMGPS_OPT_ALLOC_LIMIT) {
       REQ(value >= 0, AMGPS_E_ARG, "AMGPS_OPT_ALLOC_LIMIT takes a byte count >= 0");
       c->alloc_limit = (size_t)value;
     } else if (option == AMGPS_OPT_COARSE_KERNEL) {
       REQ(value == 0 || value == 1, AMGPS_E_ARG, "AMGPS_OPT_COARSE_KERNEL takes 0 or 1");
       c->use_cycle = (int)value;
-      c->graph_ok = false;
+      c->graph_ok = c->loop_ok = false;
     } else {
       REQ(value >= 0 && value <= 1000, AMGPS_E_ARG, "AMGPS_OPT_COARSE_SWEEPS takes 0..1000");
       c->coarse_sweeps = (int)value;
-      c->graph_ok = false;  // the coarse-level graph holds the coarse solve
+      c->graph_ok = c->loop_ok = false;  // the coarse-level graph holds the coarse solve
     }
   });
 }

@@ -167,6 +167,34 @@ void launch_spmv_dot3(const DevMat<double>& A, const double* z, double* w, const
   launch_dep(k_spmv_dot3, rw.grid, kBlock, 0, s, A, z, w, r, q, first, rw, scal);
 }
 
+// Ends an iteration of a solve in a loop (thread 0 of the last block; rr is
+// its r.r): the tests of the host loop in api.cu, in the same order of
+// operations, so both take the same number of iterations.  The one-reduction
+// form (FCG) also needs a finite alpha.
+template <bool FCG>
+__device__ __forceinline__ void pcg_continue(cudaGraphConditionalHandle h, double* scal, double rr) {
+  if (!h) return;
+  const double it = scal[S_IT] + 1.0, pq = scal[S_PQ];
+  scal[S_IT] = it;
+  const bool ok = scal[S_ERR] == 0.0 && isfinite(pq) && isfinite(rr) && pq > 0.0 &&
+                  (!FCG || isfinite(scal[S_ALPHA]));
+  const bool more = !(sqrt(rr) / sqrt(scal[S_BB]) <= scal[S_RTOL]) && it < scal[S_MAXIT];
+  cudaGraphSetConditional(h, ok && more ? 1u : 0u);
+}
+
+__global__ void k_pcg_begin(double* scal, cudaGraphConditionalHandle h) {
+  scal[S_ALPHA] = scal[S_BETA] = scal[S_IT] = 0.0;
+  scal[S_PQ] = 1.0;
+  scal[S_RZ] = INFINITY;
+  const double bb = scal[S_BB];
+  cudaGraphSetConditional(h, bb > 0.0 && isfinite(bb) ? 1u : 0u);
+}
+
+void launch_pcg_begin(double* scal, cudaGraphConditionalHandle h, cudaStream_t s) {
+  k_pcg_begin<<<1, 1, 0, s>>>(scal, h);
+  count_launch();
+}
+
 // p = z - beta p, q = w - beta q (first: p = z, q = w), x += alpha p,
 // r -= alpha q, r.r (S_RR)
 __global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* z,
@@ -174,9 +202,11 @@ __global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* 
                                                        double* __restrict__ q,
                                                        double* __restrict__ x,
                                                        double* __restrict__ r, int first,
-                                                       const RedWork rw, double* scal) {
+                                                       const RedWork rw, double* scal,
+                                                       const PcgLoop loop) {
   pdl_wait();
   pdl_go();
+  if (loop.x) x = *loop.x;
   const double alpha = ldv<false>(scal + S_ALPHA), beta = ldv<false>(scal + S_BETA);
   double acc = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < n;
@@ -190,13 +220,16 @@ __global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* 
     r[i] = ri;
     acc = fma(ri, ri, acc);
   }
-  grid_sum(acc, rw, [&](double tot) { scal[S_RR] = tot; });
+  grid_sum(acc, rw, [&](double tot) {
+    scal[S_RR] = tot;
+    pcg_continue<true>(loop.handle, scal, tot);
+  });
 }
 
 void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, double* q,
                        double* x, double* r, int first, const RedWork& rw, double* scal,
-                       cudaStream_t s) {
-  launch_dep(k_fcg_update, rw.grid, kBlock, 0, s, n, z, w, p, q, x, r, first, rw, scal);
+                       cudaStream_t s, const PcgLoop& loop) {
+  launch_dep(k_fcg_update, rw.grid, kBlock, 0, s, n, z, w, p, q, x, r, first, rw, scal, loop);
 }
 
 // r -= alpha q ; r.r (S_RR).  The x update of the same iteration is deferred
@@ -206,8 +239,8 @@ void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, d
 template <bool WC>
 __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n, const double* q, double* r,
                                                      const RedWork w, double* scal,
-                                                     const double* __restrict__ dinv,
-                                                     double* cout) {
+                                                     const double* __restrict__ dinv, double* cout,
+                                                     cudaGraphConditionalHandle h) {
   pdl_wait();
   pdl_go();
   const double alpha = ldv<false>(scal + S_ALPHA);
@@ -227,21 +260,26 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n,
     one(i + step, q1, r1);
   }
   if (i < m) one(i, ldv<false>(q + i), ldv<false>(r + i));
-  grid_sum(acc, w, [&](double tot) { scal[S_RR] = tot; });
+  grid_sum(acc, w, [&](double tot) {
+    scal[S_RR] = tot;
+    pcg_continue<false>(h, scal, tot);
+  });
 }
 
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
-                     cudaStream_t s, const double* dinv, double* cout) {
+                     cudaStream_t s, const double* dinv, double* cout, const PcgLoop& loop) {
   launch_dep(cout ? k_r_update<true> : k_r_update<false>, w.grid, kBlock, 0, s, n, q, r, w, scal,
-             dinv, cout);
+             dinv, cout, loop.handle);
 }
 
 // x += alpha p with the previous alpha, then p = z + beta p (x_beta = 1), or
 // only x += alpha p (x_beta = 0: the last iteration)
 __global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const double* z, double* p,
-                                                   double* x, const double* scal, int with_p) {
+                                                   double* x, const double* scal, int with_p,
+                                                   double* const* xslot) {
   pdl_wait();
   pdl_go();
+  if (xslot) x = *xslot;
   const double alpha = ldv<false>(scal + S_ALPHA), beta = ldv<false>(scal + S_BETA);
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (i >= n) return;
@@ -252,10 +290,10 @@ __global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const double* z, d
 }
 
 void launch_xpay_x(int64_t n, const double* z, double* p, double* x, const double* scal,
-                   int with_p, cudaStream_t s) {
+                   int with_p, cudaStream_t s, const PcgLoop& loop) {
   if (n == 0) return;
   launch_dep(k_xpay_x, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, z, p, x, scal,
-             with_p);
+             with_p, loop.x);
 }
 
 __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, const double* a, const double* b,

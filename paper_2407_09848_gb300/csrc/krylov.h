@@ -13,7 +13,18 @@ enum Scalar {
   S_RZP = 9,  // r . z_old (flexible CG)
   S_GAMMA = 10,  // z . q_old (one-reduction flexible CG)
   S_DELTA = 11,  // z . A z (one-reduction flexible CG)
+  // the solve loop on the device (PcgLoop): iterations done, rtol, maxit
+  S_IT = 12, S_RTOL = 13, S_MAXIT = 14,
   S_COUNT = 16
+};
+
+// A solve whose iterations run as the body of a WHILE node of a CUDA graph:
+// the kernel that ends an iteration decides on the device, by the tests the
+// host makes, whether there is another one.  Without a loop (handle 0) the
+// host decides.
+struct PcgLoop {
+  cudaGraphConditionalHandle handle = 0;
+  double* const* x = nullptr;  // where the solve's solution vector stands
 };
 
 struct RedWork {
@@ -37,14 +48,18 @@ void launch_spmv_dot3(const DevMat<double>& A, const double* z, double* w, const
                       cudaStream_t s);
 void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, double* q,
                        double* x, double* r, int first, const RedWork& rw, double* scal,
-                       cudaStream_t s);
+                       cudaStream_t s, const PcgLoop& loop = {});
+// start of a solve in a loop: alpha = beta = 0 and r_old.z_old infinite (the
+// first direction is then z), no iterations done; the loop runs if b.b > 0
+void launch_pcg_begin(double* scal, cudaGraphConditionalHandle handle, cudaStream_t s);
 // standard PCG with the x update deferred: r -= alpha q and r.r (with cout:
 // also cout = dinv .* r); later x += alpha p together with p = z + beta p
 // (with_p = 0: x only)
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
-                     cudaStream_t s, const double* dinv = nullptr, double* cout = nullptr);
+                     cudaStream_t s, const double* dinv = nullptr, double* cout = nullptr,
+                     const PcgLoop& loop = {});
 void launch_xpay_x(int64_t n, const double* z, double* p, double* x, const double* scal,
-                   int with_p, cudaStream_t s);
+                   int with_p, cudaStream_t s, const PcgLoop& loop = {});
 // rz_mode 0: scal[out_slot] = a.b.  1: scal[S_RZOLD] <- scal[S_RZ], scal[S_RZ] = a.b,
 // scal[S_BETA] = S_RZ / S_RZOLD.  2: as 1 with the flexible (Polak-Ribiere)
 // beta = (S_RZ - S_RZP) / S_RZOLD.
