@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
   }
   const int64_t row = s * kSlice + lane;
   const bool live = row < a.A.n;
+  const int64_t o = (int64_t)blockIdx.y * a.A.n, ro = o + row;  // vector of a batch
   using F = StepForm<FAM, INIT>;
   const bool own = live && g == 0;
   XT rin = XT(0), xin = XT(0), zo = XT(0);
@@ -78,12 +79,12 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
   const SliceDesc d = ld_desc(a.A.sd + s);
   const int k0 = (int)((int64_t)d.w * g / G), k1 = (int)((int64_t)d.w * (g + 1) / G);
   part[g][lane] = row_accumulate<F::kSign, VT, XT, false, true, 4, true>(
-      a.A, d, lane, row, a.u,
+      a.A, d, lane, row, a.u + o,
       [&] {
         if (!own) return XT(0);
-        rin = ldv<false>(a.rin + row);
-        if (FAM != FAM_RES) xin = ldv<false>(a.xin + row);
-        if (ZOWN) zo = ldv<false>(a.zown + row);
+        rin = ldv<false>(a.rin + ro);
+        if (FAM != FAM_RES) xin = ldv<false>(a.xin + ro);
+        if (ZOWN) zo = ldv<false>(a.zown + ro);
         return step_init<FAM, F::kResidual>(rin, di);
       },
       k0, k1);
@@ -91,13 +92,13 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
   if (!own) return;
   XT acc = part[0][lane];
   for (int q = 1; q < G; ++q) acc += part[q][lane];
-  step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, row, acc, rin, xin, di, zo);
+  step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, ro, acc, rin, xin, di, zo);
 }
 
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
 static void go(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
   if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
-    if (a.nvec > 1) {  // batches run on levels of one warp per slice, all slices
+    if (a.nvec > 1 && a.split == 1) {  // batches run on all slices
       launch_dep(k_step_mv<VT, XT, FAM, INIT, WR, ZOWN>,
                  dim3((unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock),
                       (a.nvec + kVecs - 1) / kVecs),
@@ -106,7 +107,8 @@ static void go(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
     }
   }
   if (a.split > 1)
-    launch_dep(k_step_split<VT, XT, FAM, INIT, WR, ZOWN>, (unsigned)work, 32 * a.split, 0, s, a);
+    launch_dep(k_step_split<VT, XT, FAM, INIT, WR, ZOWN>, dim3((unsigned)work, a.nvec),
+               32 * a.split, 0, s, a);
   else
     launch_dep(k_step<VT, XT, FAM, INIT, WR, ZOWN>,
                (unsigned)((work + kWarpsPerBlock - 1) / kWarpsPerBlock), kBlock, 0, s, a);
