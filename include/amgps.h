@@ -432,15 +432,20 @@ amgps_status amgps_profile_read(amgps_ctx* ctx, int kernel_class, int reset,
 /* The algorithmic FP64 flops of the launches counted in class 0, 1 or 2
  * since its last reset (a multiply-add counts 2, a lone multiply or add 1;
  * the products of a step count 2 per nonzero of A): class 0 has them for
- * both step forms of AMGPS_OPT_STEP_FORM, classes 1 and 2 report 0.  Read it
+ * both step forms of AMGPS_OPT_STEP_FORM, classes 1 and 2 report 0.  They are
+ * the flops of the method's steps: a launch that needs fewer (the first
+ * post-smoothing step, which runs with the coarse correction, and the scaled
+ * steps of the stored-operator form) counts as the step it performs.  Read it
  * before the amgps_profile_read call that resets the class.  Synchronous. */
 amgps_status amgps_profile_flops(amgps_ctx* ctx, int kernel_class, double* flops);
 
 /* The FP64 thread instructions the same launches issue (class 0; others 0):
  * one multiply-add per stored matrix entry, zeros of the SELL padding
- * included, plus one per vector term of a row.  Against the FP64 issue rate
- * (2 per clock per SM on GB300) it gives the pipe's utilisation, which the
- * flop count understates where a lone multiply takes a whole issue slot.
+ * included, plus one per vector term of a row, counted like the flops for the
+ * method's plain steps (the launches issue up to a tenth fewer).  Against the
+ * FP64 issue rate (2 per clock per SM on GB300) it is the rate of plain steps,
+ * where the flop count understates a lone multiply, which takes a whole issue
+ * slot.
  * Read it before the resetting amgps_profile_read.  Synchronous. */
 amgps_status amgps_profile_fp64_inst(amgps_ctx* ctx, int kernel_class, double* inst);
 

@@ -221,13 +221,52 @@ void launch_sub(int64_t n, const double* x, const double* y, double* out, cudaSt
 void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, int stride,
                       double factor, int nvec, cudaStream_t s);
 
+// ---- coarse correction with the first post-smoothing step (kernels_smooth.cu) ----
+// After the coarse solve e, the post-smoother starts from x_0 = x + P e and
+// its residual.  With an aggregation P, M^{-1}(b - A x_0) = M^{-1} r - (M^{-1} A P) e
+// where r = b - A x is what the restriction has just formed, and a row of
+// M^{-1} A P has one entry per aggregate that the row touches: four for a
+// 7-point row (its own and one neighbour per axis).  So one kernel does the
+// prolongation and the first post-smoothing step with 4 products instead of 7:
+//   s = (1/M) r - sum_k w_k e_{c_k},  x_0 = x + e_{c_0},
+//   z = c2 s,  xout = x_0 + beta z
+constexpr int kCorrEntries = 4;
+constexpr int kCorrTable = 1024;  // distinct column offsets c_k - c_0 of a level
+struct CorrMat {
+  // entry k of row i at val[(i / 32) 128 + 32 k + i % 32]; k = 0: the row's own
+  // aggregate agg[i], k > 0: agg[i] + delta[bits 10(k-1) .. of code[i]]
+  const double* val = nullptr;
+  const uint32_t* code = nullptr;
+  const int32_t* delta = nullptr;
+  const int32_t* agg = nullptr;
+};
+struct CorrArgs {
+  CorrMat m;
+  int64_t n = 0, nc = 0;
+  const double *r = nullptr, *dinv = nullptr, *e = nullptr, *x = nullptr;
+  double* x0out = nullptr;  // also x_0 (null: not kept)
+  double* sout = nullptr;   // s (may equal r); null: not kept
+  double* zout = nullptr;   // z; null: not kept
+  double* xout = nullptr;   // may equal x or r
+  double c2 = 1, beta = 0;
+};
+void launch_correct(const CorrArgs& a, int nvec, cudaStream_t s);
+// Fills val and code of the level whose row-scaled matrix is B; delta holds
+// kCorrTable entries (kCorrEmpty, entry 0: 0).  *bad != 0 afterwards: a row
+// touches more than four aggregates, or there are too many distinct offsets.
+constexpr int32_t kCorrEmpty = INT32_MIN;
+void launch_build_correct(const DevMat<double>& B, const int32_t* agg, double* val, uint32_t* code,
+                          int32_t* delta, int* bad, cudaStream_t s);
+
 // ---- persistent kernel for the coarse levels of a V-cycle (kernels_cycle.cu) ----
 // The levels below the TMA-fed ones are launch-latency-bound: their kernels
 // last a few microseconds each.  The host records the kernel sequence of
 // those levels once (the same calls, same arguments, same order) as a list of
 // phases, and one co-resident grid runs the phases with a grid-wide barrier
 // between consecutive ones.
-enum CycleOp { CY_STEP = 0, CY_FIRST = 1, CY_AGG = 2, CY_PROLONG = 3, CY_GEMV = 4, CY_COPY = 5 };
+enum CycleOp {
+  CY_STEP = 0, CY_FIRST = 1, CY_AGG = 2, CY_PROLONG = 3, CY_GEMV = 4, CY_COPY = 5, CY_CORRECT = 6
+};
 
 template <class VT, class XT>
 struct CyclePhase {
@@ -245,6 +284,7 @@ struct CyclePhase {
   XT* out2 = nullptr;           // CY_FIRST: x
   const double* ainv = nullptr;  // CY_GEMV
   XT c2 = 0, beta = 0, rhoinv = 1;
+  CorrArgs corr;                // CY_CORRECT (FP64 levels)
 };
 
 // grid-barrier word: arrivals, zeroed before each launch

@@ -200,6 +200,12 @@ struct Level {
   DevMat<double> Pm, Rm;
   int64_t xfer_stored = 0;  // stored entries of P and R together
   int psplit = 1, rsplit = 1;
+  // M^{-1} A P of an FP64 aggregation level whose rows touch at most four
+  // aggregates (corr.val null: none)
+  CorrMat corr;
+  void* corr_mem = nullptr;
+  size_t corr_bytes = 0;
+  int wmax = 0;  // stored entries of the widest slice
   int split = 1;  // warps per slice of the generic step kernel (wide rows)
   void* dinv = nullptr;   // 1 / M_i
   // FP64 and FP32 levels: the row-scaled values a_ij / M_i in the layout and
@@ -346,6 +352,17 @@ T* dupload(amgps_ctx* c, const T* h, size_t count) {
   T* d = (T*)dalloc(c, count * sizeof(T));
   if (count) CK(cudaMemcpy(d, h, count * sizeof(T), cudaMemcpyHostToDevice));
   return d;
+}
+
+// Gives the arrays of a level's coarse correction back (no kernel that uses
+// them may be enqueued; a captured graph that does is stale afterwards).
+void drop_correct(amgps_ctx* c, Level& L) {
+  if (!L.corr_mem) return;
+  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), L.corr_mem));
+  cudaFree(L.corr_mem);
+  c->alloc_bytes -= L.corr_bytes;
+  L.corr_mem = nullptr;
+  L.corr = CorrMat{};
 }
 
 void free_hierarchy(amgps_ctx* c) {
@@ -659,7 +676,7 @@ struct Engine {
   // u_j alternate between zb and xb (u_j overwrites u_{j+2}, which only its
   // own row reads); r holds x_0 + h s_0 for the last step when k >= 3.
   static void smooth_ops(amgps_ctx* c, int l, const Coefs& cf, const XT* b, XT* x, bool xzero,
-                         bool c_ready) {
+                         bool c_ready, bool corrected) {
     Level& L = c->lv[l];
     cudaStream_t s = c->stream;
     OpStep st[kMaxDegree];
@@ -669,11 +686,11 @@ struct Engine {
     XT* U[2] = {(XT*)L.zb, (XT*)L.xb};
     XT* t = (XT*)L.r;
     const bool profl = (l == 0);
-    if (!c_ready)
+    if (!c_ready && !corrected)
       do_first(FAM_JAC, L.n, b, (const XT*)L.dinv, nullptr, nullptr, cv, XT(0), XT(0), XT(1),
                c->nvec, s);
     const DevMat<VT> A = devmat<VT>(L);
-    if (!xzero) {
+    if (!xzero && !corrected) {
       StepArgs<VT, XT> a;
       a.A = A;
       a.A.val = (const VT*)L.sval;
@@ -721,15 +738,77 @@ struct Engine {
     check_launch();
   }
 
+  // Whether the first post-smoothing step of level L runs with the coarse
+  // correction (see CorrArgs).
+  static bool use_correct(const Level& L) {
+    return std::is_same<VT, double>::value && std::is_same<XT, double>::value &&
+           L.corr.val != nullptr;
+  }
+
+  // The coarse correction x_0 = x + P e with the first step of the application
+  // `cf` on x_0, from the unscaled residual in the level's r buffer; `smooth`
+  // with corrected = true continues.  x0: also keeps x_0 (null: not).
+  static void correct(amgps_ctx* c, int l, const Coefs& cf, const XT* e, XT* x, XT* x0) {
+    if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
+      Level& L = c->lv[l];
+      CorrArgs a;
+      a.m = L.corr;
+      a.n = L.n;
+      a.nc = L.nc;
+      a.r = (const double*)L.r;
+      a.dinv = (const double*)L.dinv;
+      a.e = e;
+      a.x = x;
+      a.x0out = x0;
+      a.xout = x;
+      const int k = cf.k;
+      if (use_ops(c, L, cf)) {
+        a.sout = (double*)L.za;  // s_0; x_0 + h s_0 for the last step (k = 2: x_0 itself)
+        OpStep st[kMaxDegree];
+        const int ns = op_plan(cf, st);
+        if (k >= 3) {
+          a.xout = (double*)L.r;
+          a.beta = st[ns - 1].h;
+        }
+      } else if (cf.fam == FAM_JAC) {
+        a.beta = 1.0;
+      } else {
+        if (k > 1) a.sout = (double*)L.r;
+        a.zout = (double*)L.za;
+        a.c2 = cf.fam == FAM_CHEB4 ? cf.c2[1] : cf.c2[0] * cf.rhoinv;
+        a.beta = cf.fam == FAM_CHEB4 ? cf.beta[1] : 1.0;
+      }
+      if (auto* R = rec()) {
+        CyclePhase<VT, XT> p;
+        p.op = CY_CORRECT;
+        p.n = L.n;
+        p.corr = a;
+        R->push_back(p);
+        return;
+      }
+      // counted as the smoother step it takes the place of
+      const bool ops = use_ops(c, L, cf), wt = k >= 3;
+      ProfScope ps(c, l == 0, 0, (double)L.n * (36.0 + 4.0 + 8.0 * 5.0) + (double)L.nc * 8.0,
+                   ops ? op_flops(L, FAM_OPT, true, true, false, wt)
+                       : step_flops(L, cf.fam, false, true),
+                   ops ? op_inst(L, FAM_OPT, true, true, false, wt)
+                       : step_inst(L, cf.fam, false, true));
+      launch_correct(a, c->nvec, c->stream);
+      check_launch();
+      ps.done();
+    }
+  }
+
   // One smoother application on level l: x <- S(b, x) (x = 0 when xzero).
+  // corrected: its first step has run (`correct`).
   // Returns true when it ran in the stored-operator form (then, from zero,
   // the level's za holds M^{-1} b for a following application with x given:
   // pass c_ready there).
   static bool smooth(amgps_ctx* c, int l, const Coefs& cf, const XT* b, XT* x, bool xzero,
-                     bool c_ready = false) {
+                     bool c_ready = false, bool corrected = false) {
     Level& L = c->lv[l];
     if (use_ops(c, L, cf)) {
-      smooth_ops(c, l, cf, b, x, xzero, c_ready);
+      smooth_ops(c, l, cf, b, x, xzero, c_ready, corrected);
       return true;
     }
     cudaStream_t s = c->stream;
@@ -745,7 +824,9 @@ struct Engine {
       XT* cur = x;
       XT* oth = xb;
       int j0 = 0;
-      if (xzero) {
+      if (corrected) {
+        j0 = 1;
+      } else if (xzero) {
         do_first(FAM_JAC, L.n, b, md, nullptr, nullptr, cur, XT(0), XT(0), XT(1), c->nvec, s);
         j0 = 1;
       }
@@ -772,7 +853,9 @@ struct Engine {
     }
     const XT* rin_next;
     XT* xcur = x;
-    if (xzero) {
+    if (corrected) {
+      rin_next = r;
+    } else if (xzero) {
       double c2 = (cf.fam == FAM_CHEB4) ? cf.c2[1] : cf.c2[0];
       double rhoinv = cf.rhoinv;
       if (L.sval && cf.fam == FAM_CHEB1) {  // scaled 1st-kind form: r = rho r^(0)
@@ -915,11 +998,16 @@ struct Engine {
       }
       ps.done();
     }
-    if (L.xfer_general) launch_xfer<XT>(L.Pm, (const XT*)C.x, x, 1, L.psplit, s);
-    else do_prolong(L, (const XT*)C.x, x, c->nvec, s);
-    if (record)
-      CK(cudaMemcpyAsync(L.bx2, x, c->nvec * L.n * sizeof(XT), cudaMemcpyDeviceToDevice, s));
-    smooth(c, l, cf, b, x, false, c_kept);
+    const bool corr = use_correct(L);
+    if (corr) {
+      correct(c, l, cf, (const XT*)C.x, x, record ? (XT*)L.bx2 : nullptr);
+    } else {
+      if (L.xfer_general) launch_xfer<XT>(L.Pm, (const XT*)C.x, x, 1, L.psplit, s);
+      else do_prolong(L, (const XT*)C.x, x, c->nvec, s);
+      if (record)
+        CK(cudaMemcpyAsync(L.bx2, x, c->nvec * L.n * sizeof(XT), cudaMemcpyDeviceToDevice, s));
+    }
+    smooth(c, l, cf, b, x, false, c_kept, corr);
     check_launch();
   }
 
@@ -1291,6 +1379,59 @@ bool op_level(const amgps_ctx* c, const Level& L) {
   return c->prec == AMGPS_F64 && L.sval && !L.coarsest && L.split == 1 && L.n >= kOpMinRows;
 }
 
+// M^{-1} A P of every FP64 aggregation level with rows of at most eight stored
+// entries, for the coarse correction (36 B a row).  A level whose arrays do not
+// fit the device or the allocation limit, or with a row that touches more than
+// four aggregates, keeps the prolongation and the full first step.
+void prepare_correct(amgps_ctx* c) {
+  if (c->prec != AMGPS_F64) return;
+  struct Try {
+    Level* L;
+    int* bad;
+    CorrMat m;
+  };
+  std::vector<Try> built;
+  int32_t table[kCorrTable];
+  std::fill(table, table + kCorrTable, kCorrEmpty);
+  table[0] = 0;
+  for (auto& L : c->lv) {
+    if (L.coarsest || L.xfer_general || L.wmax > 8) continue;
+    const size_t vb = (size_t)L.nslices * kSlice * kCorrEntries * sizeof(double);
+    const size_t cb = ((size_t)L.n * sizeof(uint32_t) + 255) / 256 * 256;
+    const size_t tb = kCorrTable * sizeof(int32_t);
+    try {
+      L.corr_mem = dalloc(c, vb + cb + tb + 256);
+    } catch (const Fail& f) {
+      if (f.st != AMGPS_E_NOMEM) throw;
+      continue;
+    }
+    L.corr_bytes = vb + cb + tb + 256;
+    char* base = (char*)L.corr_mem;
+    int* bad = (int*)(base + vb + cb + tb);
+    CorrMat m;
+    m.val = (const double*)base;
+    m.code = (const uint32_t*)(base + vb);
+    m.delta = (const int32_t*)(base + vb + cb);
+    m.agg = L.agg;
+    CK(cudaMemcpyAsync(base + vb + cb, table, tb, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
+    DevMat<double> B = devmat<double>(L);
+    B.val = (const double*)L.sval;
+    launch_build_correct(B, L.agg, (double*)base, (uint32_t*)(base + vb),
+                         (int32_t*)(base + vb + cb), bad, c->stream);
+    check_launch();
+    built.push_back({&L, bad, m});
+  }
+  std::vector<int> flags(built.size(), 0);
+  for (size_t i = 0; i < built.size(); ++i)
+    CK(cudaMemcpyAsync(&flags[i], built[i].bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  for (size_t i = 0; i < built.size(); ++i) {
+    if (flags[i] == 0) built[i].L->corr = built[i].m;
+    else drop_correct(c, *built[i].L);
+  }
+}
+
 // Builds, on the library stream, the stored operators of every such level
 // for its current smoother (degree >= 2), unless they are
 // already built for it.  A level whose operators would not fit the device or
@@ -1307,13 +1448,22 @@ void prepare_ops(amgps_ctx* c) {
     if (c->step_form != 1 || cap != cudaStreamCaptureStatusNone || !op_level(c, L)) continue;
     if (cf.k < 2) continue;
     const int ns = cf.k - 1;
-    try {
-      while ((int)L.ops.size() < ns)
-        L.ops.push_back((double*)dalloc(c, (size_t)L.stored * sizeof(double)));
-    } catch (const Fail& f) {
-      if (f.st != AMGPS_E_NOMEM) throw;
-      continue;
+    bool fits = false;
+    for (int attempt = 0; attempt < 2 && !fits; ++attempt) {
+      if (attempt == 1) {  // the operators go before the coarse corrections
+        CK(cudaStreamSynchronize(c->stream));
+        for (auto& K : c->lv) drop_correct(c, K);
+        c->graph_ok = c->loop_ok = false;
+      }
+      try {
+        while ((int)L.ops.size() < ns)
+          L.ops.push_back((double*)dalloc(c, (size_t)L.stored * sizeof(double)));
+        fits = true;
+      } catch (const Fail& f) {
+        if (f.st != AMGPS_E_NOMEM) throw;
+      }
     }
+    if (!fits) continue;
     OpStep st[kMaxDegree];
     op_plan(cf, st);
     DevMat<double> B = devmat<double>(L);
@@ -2067,6 +2217,7 @@ amgps_status amgps_hierarchy_load(amgps_ctx* c, int n_levels, const amgps_csr* A
       load_levels(c, n_levels, A, P, prec);
       prepare_ops(c);
       prepare_coarse(c);
+      prepare_correct(c);
     } catch (...) {
       free_hierarchy(c);  // a failed load keeps no buffers
       leave(c);
@@ -2117,6 +2268,7 @@ void load_levels(amgps_ctx* c, int n_levels, const amgps_csr* A, const amgps_csr
     L.nslices = h.nslices;
     L.stored = h.stored;
     L.explicit_entries = h.explicit_entries;
+    for (const SliceDesc& d : h.sd) L.wmax = std::max(L.wmax, (int)d.w);
     L.sd = dupload(c, h.sd.data(), h.sd.size());
     if (h.off.empty()) h.off.push_back(0);  // every slice explicit: keep a valid pointer
     L.off = dupload(c, h.off.data(), h.off.size());

@@ -419,6 +419,42 @@ __device__ __forceinline__ void prolong_row(int64_t i, const int32_t* agg, const
   x[i] = xi + ldv<CG>(ec + c);
 }
 
+// Row i of the coarse correction (see CorrArgs).
+template <bool CG = false, bool WAIT = false>
+__device__ __forceinline__ void correct_row(const CorrArgs& a, int64_t i, int64_t v) {
+  const int64_t at = (i >> 5) * (kCorrEntries * kSlice) + (i & 31);
+  double w[kCorrEntries], e[kCorrEntries];
+  int32_t c[kCorrEntries];
+  const uint32_t code = __ldcs(a.m.code + i);
+  c[0] = __ldg(a.m.agg + i);
+#pragma unroll
+  for (int k = 0; k < kCorrEntries; ++k) w[k] = __ldcs(a.m.val + at + kSlice * k);
+  const double di = __ldg(a.dinv + i);
+#pragma unroll
+  for (int k = 1; k < kCorrEntries; ++k)
+    c[k] = c[0] + __ldg(a.m.delta + ((code >> (10 * (k - 1))) & (kCorrTable - 1)));
+  if constexpr (WAIT) {
+    pdl_wait();
+    pdl_go();
+  }
+  const int64_t j = v * a.n + i;
+  const double* ev = a.e + v * a.nc;
+  const double r = ldv<CG>(a.r + j), x = ldv<CG>(a.x + j);
+#pragma unroll
+  for (int k = 0; k < kCorrEntries; ++k) e[k] = ldv<CG>(ev + c[k]);
+  double s = r * di;
+#pragma unroll
+  for (int k = 0; k < kCorrEntries; ++k) s = fma(-w[k], e[k], s);
+  const double x0 = x + e[0];
+  if (a.x0out) a.x0out[j] = x0;
+  if (a.sout) a.sout[j] = s;
+  if (a.zout) {
+    s *= a.c2;
+    a.zout[j] = s;
+  }
+  a.xout[j] = fma(a.beta, s, x0);
+}
+
 // x_i = (A_c^{-1} b)_i for the coarsest level, one warp per row: lane l sums
 // columns l, l + 32, ... in order, then a fixed butterfly adds the lanes.  The
 // first 16 entries of a lane (512 columns) are loaded together, before the
