@@ -3109,7 +3109,7 @@ amgps_status amgps_galerkin(amgps_ctx* c, const amgps_csr* A, const amgps_csr* P
   return guard(c, [&] {
     REQ(c && A && P && Ac, AMGPS_E_ARG, "null argument");
     CK(cudaSetDevice(c->device));
-    galerkin_on_device(SetupEnv{c->stream, c->nsm}, *A, *P, Ac);
+    galerkin_on_device(SetupEnv{c->stream, c->nsm, pool_of(c->device)}, *A, *P, Ac);
   });
 }
 
@@ -3119,7 +3119,7 @@ amgps_status amgps_sa_level(amgps_ctx* c, const amgps_csr* A, const int32_t* agg
   return guard(c, [&] {
     REQ(c && A && agg && omega && P_out && Ac_out, AMGPS_E_ARG, "null argument");
     CK(cudaSetDevice(c->device));
-    sa_level_on_device(SetupEnv{c->stream, c->nsm}, *A, agg, n_coarse, omega, P_out, Ac_out);
+    sa_level_on_device(SetupEnv{c->stream, c->nsm, pool_of(c->device)}, *A, agg, n_coarse, omega, P_out, Ac_out);
   });
 }
 

@@ -17,15 +17,26 @@
 namespace amgps {
 namespace {
 
+// Device scratch of one call: from the library's stream-ordered pool (no
+// device-wide wait for each buffer), or plain allocations without one.
 struct DevScratch {
+  cudaMemPool_t pool;
+  cudaStream_t stream;
   std::vector<void*> ptrs;
+  explicit DevScratch(const SetupEnv& env) : pool(env.pool), stream(env.stream) {}
   ~DevScratch() {
-    for (void* p : ptrs) cudaFree(p);
+    for (void* p : ptrs) {
+      if (pool) cudaFreeAsync(p, stream);
+      else cudaFree(p);
+    }
   }
   template <class T>
   T* alloc(size_t count) {
     void* p = nullptr;
-    const cudaError_t e = cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T));
+    const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+    const cudaError_t e =
+        pool ? cudaMallocFromPoolAsync(&p, bytes, pool, stream) : cudaMalloc(&p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
     REQ(e == cudaSuccess, AMGPS_E_NOMEM, std::string("set-up scratch: ") + cudaGetErrorString(e));
     ptrs.push_back(p);
     return (T*)p;
@@ -71,33 +82,35 @@ void check_dev_err(int* derr, cudaStream_t s, const char* what) {
   REQ(!dev_err_set(derr, s), AMGPS_E_ARG, what);
 }
 
-// rowptr from per-row counts (prefix on the host); allocates col and val
+// rowptr from per-row counts; allocates col and val
 DevCsr from_counts(DevScratch& B, const int32_t* dcnt, int64_t rows, int64_t cols,
                    cudaStream_t s) {
-  std::vector<int32_t> h((size_t)rows);
-  if (rows) CK(cudaMemcpyAsync(h.data(), dcnt, rows * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  std::vector<int32_t> rp((size_t)rows + 1, 0);
-  int64_t acc = 0;
-  for (int64_t i = 0; i < rows; ++i) {
-    acc += h[i];
-    REQ(acc < (int64_t(1) << 31), AMGPS_E_ARG, "sparse product exceeds 2^31 entries");
-    rp[i + 1] = (int32_t)acc;
-  }
   DevCsr C;
   C.n_rows = rows;
   C.n_cols = cols;
-  C.nnz = acc;
-  C.rowptr = B.upload(rp.data(), rp.size(), s);
-  C.col = B.alloc<int32_t>(acc);
-  C.val = B.alloc<double>(acc);
+  C.rowptr = B.alloc<int32_t>((size_t)rows + 1);
+  const int64_t nb = scan_blocks(rows);
+  int64_t* sums = B.alloc<int64_t>((size_t)nb + 1);
+  launch_scan(rows, dcnt, C.rowptr, sums, s);
+  check_launch();
+  CK(cudaMemcpyAsync(&C.nnz, sums + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  REQ(C.nnz < (int64_t(1) << 31), AMGPS_E_ARG, "sparse product exceeds 2^31 entries");
+  C.col = B.alloc<int32_t>(C.nnz);
+  C.val = B.alloc<double>(C.nnz);
   return C;
 }
 
 DevCsr dev_spgemm(const SetupEnv& env, DevScratch& B, const DevCsr& X, const DevCsr& Y, int* derr) {
   cudaStream_t s = env.stream;
   int32_t* cnt = B.alloc<int32_t>(X.n_rows);
-  if (Y.n_cols <= kDenseMaxCols) {  // few columns: dense row accumulator
+  // the smallest table first, the next one when a row exceeds its limit
+  int form = Y.n_cols <= kDenseFirst ? kWide : kTiny;
+  for (; form < kWide; ++form) {
+    launch_spgemm(X, Y, cnt, DevCsr{}, derr, false, (GemmForm)form, env.nsm, s);
+    if (!dev_err_set(derr, s)) break;
+  }
+  if (form == kWide && Y.n_cols <= kDenseMaxCols) {  // few columns: dense row accumulator
     launch_spgemm_dense(X, Y, cnt, DevCsr{}, derr, false, env.nsm, s);
     check_dev_err(derr, s, "sparse product: symbolic pass failed");
     DevCsr C = from_counts(B, cnt, X.n_rows, Y.n_cols, s);
@@ -105,16 +118,12 @@ DevCsr dev_spgemm(const SetupEnv& env, DevScratch& B, const DevCsr& X, const Dev
     check_dev_err(derr, s, "sparse product: numeric pass failed");
     return C;
   }
-  // narrow form first; the wide form when some row exceeds its limit
-  bool wide = false;
-  launch_spgemm(X, Y, cnt, DevCsr{}, derr, false, false, env.nsm, s);
-  if (dev_err_set(derr, s)) {
-    wide = true;
-    launch_spgemm(X, Y, cnt, DevCsr{}, derr, false, true, env.nsm, s);
+  if (form == kWide) {
+    launch_spgemm(X, Y, cnt, DevCsr{}, derr, false, kWide, env.nsm, s);
     check_dev_err(derr, s, "sparse product: a row has more than 6144 distinct columns");
   }
   DevCsr C = from_counts(B, cnt, X.n_rows, Y.n_cols, s);
-  launch_spgemm(X, Y, nullptr, C, derr, true, wide, env.nsm, s);
+  launch_spgemm(X, Y, nullptr, C, derr, true, (GemmForm)form, env.nsm, s);
   check_dev_err(derr, s, "sparse product: numeric pass failed");
   return C;
 }
@@ -189,7 +198,7 @@ void galerkin_on_device(const SetupEnv& env, const amgps_csr& A, const amgps_csr
   REQ(P.n_rows == A.n_rows, AMGPS_E_ARG, "P rows must equal A rows");
   require_sorted_rows(P, "P");
   cudaStream_t s = env.stream;
-  DevScratch B;
+  DevScratch B(env);
   int* derr = B.alloc<int>(1);
   CK(cudaMemsetAsync(derr, 0, sizeof(int), s));
   const DevCsr dA = upload_csr(B, A, s), dP = upload_csr(B, P, s);
@@ -211,7 +220,7 @@ void sa_level_on_device(const SetupEnv& env, const amgps_csr& A, const int32_t* 
     REQ(used[I], AMGPS_E_ARG, "empty aggregate (coarse index without a fine point)");
   cudaStream_t s = env.stream;
   const int64_t n = A.n_rows;
-  DevScratch B;
+  DevScratch B(env);
   int* derr = B.alloc<int>(1);
   CK(cudaMemsetAsync(derr, 0, sizeof(int), s));
   const DevCsr dA = upload_csr(B, A, s);
@@ -229,16 +238,14 @@ void sa_level_on_device(const SetupEnv& env, const amgps_csr& A, const int32_t* 
   REQ(std::isfinite(lam) && lam > 0.0, AMGPS_E_NAN, "row-sum bound not finite");
   const double om = 4.0 / (3.0 * lam);
   // P_hat (one unit entry per row), A P_hat, then P in place
-  std::vector<int32_t> iota((size_t)n + 1);
-  for (int64_t i = 0; i <= n; ++i) iota[i] = (int32_t)i;
-  std::vector<double> ones((size_t)n, 1.0);
   DevCsr Ph;
   Ph.n_rows = n;
   Ph.n_cols = n_coarse;
   Ph.nnz = n;
-  Ph.rowptr = B.upload(iota.data(), iota.size(), s);
+  Ph.rowptr = B.alloc<int32_t>((size_t)n + 1);
   Ph.col = dagg;
-  Ph.val = B.upload(ones.data(), ones.size(), s);
+  Ph.val = B.alloc<double>((size_t)n);
+  launch_unit_rows(n, Ph.rowptr, Ph.val, s);
   const DevCsr P = dev_spgemm(env, B, dA, Ph, derr);
   launch_sa_combine(P, dagg, diag, om, s);
   check_launch();

@@ -14,6 +14,7 @@ namespace amgps {
 struct SetupEnv {
   cudaStream_t stream;
   int nsm;  // SMs of the device (grid sizes)
+  cudaMemPool_t pool;  // where scratch comes from (null: plain allocations)
 };
 
 // A_c = P^T A P (amgps_galerkin)
