@@ -235,12 +235,13 @@ void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, d
 // r -= alpha q ; r.r (S_RR).  The x update of the same iteration is deferred
 // to k_xpay_x, which reads p anyway.  WC: also c = M^{-1} r (the product the
 // stored-operator smoother of the next V-cycle starts from, same operation
-// as its own c pass).
-template <bool WC>
+// as its own c pass).  WF: also r rounded to FP32 (the right-hand side of an
+// FP32 or BF16 V-cycle).
+template <bool WC, bool WF>
 __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n, const double* q, double* r,
                                                      const RedWork w, double* scal,
                                                      const double* __restrict__ dinv, double* cout,
-                                                     cudaGraphConditionalHandle h) {
+                                                     float* fout, cudaGraphConditionalHandle h) {
   pdl_wait();
   pdl_go();
   const double alpha = ldv<false>(scal + S_ALPHA);
@@ -250,6 +251,7 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n,
     ri = fma(-alpha, qi, ri);
     r[i] = ri;
     if constexpr (WC) cout[i] = ri * __ldg(dinv + i);
+    if constexpr (WF) fout[i] = (float)ri;
     acc = fma(ri, ri, acc);
   };
   uint32_t i = blockIdx.x * kBlock + threadIdx.x;
@@ -267,14 +269,16 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n,
 }
 
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
-                     cudaStream_t s, const double* dinv, double* cout, const PcgLoop& loop) {
-  launch_dep(cout ? k_r_update<true> : k_r_update<false>, w.grid, kBlock, 0, s, n, q, r, w, scal,
-             dinv, cout, loop.handle);
+                     cudaStream_t s, const double* dinv, double* cout, float* fout,
+                     const PcgLoop& loop) {
+  auto* k = cout ? k_r_update<true, false> : fout ? k_r_update<false, true> : k_r_update<false, false>;
+  launch_dep(k, w.grid, kBlock, 0, s, n, q, r, w, scal, dinv, cout, fout, loop.handle);
 }
 
 // x += alpha p with the previous alpha, then p = z + beta p (x_beta = 1), or
 // only x += alpha p (x_beta = 0: the last iteration)
-__global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const double* z, double* p,
+template <class ZT>
+__global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const ZT* z, double* p,
                                                    double* x, const double* scal, int with_p,
                                                    double* const* xslot) {
   pdl_wait();
@@ -284,19 +288,26 @@ __global__ void __launch_bounds__(kBlock) k_xpay_x(int64_t n, const double* z, d
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (i >= n) return;
   const double pi = ldv<false>(p + i), xi = ldv<false>(x + i);
-  const double zi = with_p ? ldv<false>(z + i) : 0.0;
+  const double zi = with_p ? (double)ldv<false>(z + i) : 0.0;
   x[i] = fma(alpha, pi, xi);
   if (with_p) p[i] = fma(beta, pi, zi);
 }
 
-void launch_xpay_x(int64_t n, const double* z, double* p, double* x, const double* scal,
-                   int with_p, cudaStream_t s, const PcgLoop& loop) {
+template <class ZT>
+void launch_xpay_x(int64_t n, const ZT* z, double* p, double* x, const double* scal, int with_p,
+                   cudaStream_t s, const PcgLoop& loop) {
   if (n == 0) return;
-  launch_dep(k_xpay_x, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, z, p, x, scal,
+  launch_dep(k_xpay_x<ZT>, (unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, s, n, z, p, x, scal,
              with_p, loop.x);
 }
+template void launch_xpay_x<double>(int64_t, const double*, double*, double*, const double*, int,
+                                    cudaStream_t, const PcgLoop&);
+template void launch_xpay_x<float>(int64_t, const float*, double*, double*, const double*, int,
+                                   cudaStream_t, const PcgLoop&);
 
-__global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, const double* a, const double* b,
+template <class BT>
+__global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, const double* a,
+                                                                 const BT* b,
                                                 const RedWork w, double* scal, int slot,
                                                 int rz_shift) {
   pdl_wait();
@@ -304,7 +315,8 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, cons
   double acc = 0.0;
   const int64_t step = (int64_t)gridDim.x * kBlock;
   for (int64_t i0 = (int64_t)blockIdx.x * kBlock + threadIdx.x; i0 < n; i0 += kLoads * step) {
-    double av[kLoads], bv[kLoads];
+    double av[kLoads];
+    BT bv[kLoads];
 #pragma unroll
     for (int k = 0; k < kLoads; ++k) {
       const int64_t i = i0 + k * step;
@@ -315,7 +327,7 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, cons
     }
 #pragma unroll
     for (int k = 0; k < kLoads; ++k)
-      if (i0 + k * step < n) acc = fma(av[k], bv[k], acc);
+      if (i0 + k * step < n) acc = fma(av[k], (double)bv[k], acc);
   }
   grid_sum(acc, w, [&](double tot) {
     if (rz_shift) {
@@ -328,10 +340,15 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, cons
   });
 }
 
-void launch_dot(int64_t n, const double* a, const double* b, const RedWork& w, double* scal,
+template <class BT>
+void launch_dot(int64_t n, const double* a, const BT* b, const RedWork& w, double* scal,
                 int out_slot, int rz_mode, cudaStream_t s) {
-  launch_dep(k_dot, w.grid, kBlock, 0, s, n, a, b, w, scal, out_slot, rz_mode);
+  launch_dep(k_dot<BT>, w.grid, kBlock, 0, s, n, a, b, w, scal, out_slot, rz_mode);
 }
+template void launch_dot<double>(int64_t, const double*, const double*, const RedWork&, double*, int,
+                                 int, cudaStream_t);
+template void launch_dot<float>(int64_t, const double*, const float*, const RedWork&, double*, int,
+                                int, cudaStream_t);
 
 __global__ void __launch_bounds__(kBlock) k_sub(int64_t n, const double* x, const double* y,
                                                 double* out) {

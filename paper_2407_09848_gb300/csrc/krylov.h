@@ -53,17 +53,20 @@ void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, d
 // first direction is then z), no iterations done; the loop runs if b.b > 0
 void launch_pcg_begin(double* scal, cudaGraphConditionalHandle handle, cudaStream_t s);
 // standard PCG with the x update deferred: r -= alpha q and r.r (with cout:
-// also cout = dinv .* r); later x += alpha p together with p = z + beta p
+// also cout = dinv .* r, with fout: also r in FP32); later x += alpha p together with p = z + beta p
 // (with_p = 0: x only)
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
                      cudaStream_t s, const double* dinv = nullptr, double* cout = nullptr,
-                     const PcgLoop& loop = {});
-void launch_xpay_x(int64_t n, const double* z, double* p, double* x, const double* scal,
-                   int with_p, cudaStream_t s, const PcgLoop& loop = {});
+                     float* fout = nullptr, const PcgLoop& loop = {});
+template <class ZT>
+void launch_xpay_x(int64_t n, const ZT* z, double* p, double* x, const double* scal, int with_p,
+                   cudaStream_t s, const PcgLoop& loop = {});
 // rz_mode 0: scal[out_slot] = a.b.  1: scal[S_RZOLD] <- scal[S_RZ], scal[S_RZ] = a.b,
 // scal[S_BETA] = S_RZ / S_RZOLD.  2: as 1 with the flexible (Polak-Ribiere)
 // beta = (S_RZ - S_RZP) / S_RZOLD.
-void launch_dot(int64_t n, const double* a, const double* b, const RedWork& w, double* scal,
+// (b may be FP32: each entry is widened)
+template <class BT>
+void launch_dot(int64_t n, const double* a, const BT* b, const RedWork& w, double* scal,
                 int out_slot, int rz_mode, cudaStream_t s);
 template <class XT>
 void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, int nvec, cudaStream_t s);
