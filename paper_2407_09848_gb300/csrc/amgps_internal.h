@@ -221,6 +221,32 @@ void launch_sub(int64_t n, const double* x, const double* y, double* out, cudaSt
 void launch_scale_dev(int64_t n, const double* x, double* out, const double* s_dev, int stride,
                       double factor, int nvec, cudaStream_t s);
 
+// ---- residual, restriction and the next level's first step (kernels_smooth.cu) ----
+// r = b - A u, b_c[I] = sum of r over the children of I in list order, and (fam
+// >= 0) the first step from zero of the coarse level's smoother on b_c[I]
+// (first_row): what the FAM_RES step, the aggregation and k_first do one after
+// the other, with the same operations in the same order.
+template <class VT, class XT>
+struct RestrictArgs {
+  DevMat<VT> A;
+  const XT* b = nullptr;
+  const XT* u = nullptr;
+  XT* r = nullptr;
+  const int32_t* cptr = nullptr;
+  const int32_t* cidx = nullptr;
+  int64_t nc = 0;
+  XT* bc = nullptr;
+  int fam = -1;  // FAM_CHEB4, FAM_CHEB1 or FAM_JAC
+  const XT* dinv = nullptr;  // of the coarse level, as the rest
+  XT *rout = nullptr, *zout = nullptr, *xout = nullptr;
+  XT c2 = 0, beta = 0, rhoinv = 1;
+};
+template <class VT, class XT>
+void launch_restrict(const RestrictArgs<VT, XT>& a, int nvec, cudaStream_t s);
+// Levels of at most this many rows take it: there the three kernels are mostly
+// latency; on larger ones the children's rows are better read coalesced.
+constexpr int64_t kFuseRows = 1 << 16;
+
 // ---- coarse correction with the first post-smoothing step (kernels_smooth.cu) ----
 // After the coarse solve e, the post-smoother starts from x_0 = x + P e and
 // its residual.  With an aggregation P, M^{-1}(b - A x_0) = M^{-1} r - (M^{-1} A P) e

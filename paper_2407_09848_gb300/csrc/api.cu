@@ -714,9 +714,7 @@ struct Engine {
     XT* U[2] = {(XT*)L.zb, (XT*)L.xb};
     XT* t = (XT*)L.r;
     const bool profl = (l == 0);
-    if (!c_ready && !corrected)
-      do_first(FAM_JAC, L.n, b, (const XT*)L.dinv, nullptr, nullptr, cv, XT(0), XT(0), XT(1),
-               c->nvec, s);
+    if (!c_ready && !corrected) run_first(c, L, first_of(c, L, cf, x), b);
     const DevMat<VT> A = devmat<VT>(L);
     if (!xzero && !corrected) {
       StepArgs<VT, XT> a;
@@ -835,7 +833,42 @@ struct Engine {
     }
   }
 
+  // The first step from zero of application `cf` on level l (launch_first):
+  // in the stored-operator form c = M^{-1} b.
+  struct First {
+    int fam = FAM_JAC;
+    XT *r = nullptr, *z = nullptr, *x = nullptr;
+    XT c2 = 0, beta = 0, rhoinv = 1;
+  };
+  static First first_of(const amgps_ctx* c, const Level& L, const Coefs& cf, XT* x) {
+    First f;
+    if (use_ops(c, L, cf)) {
+      f.x = (XT*)L.za;
+      return f;
+    }
+    f.x = x;
+    if (cf.fam == FAM_JAC) return f;
+    f.fam = cf.fam;
+    f.r = (XT*)L.r;
+    f.z = (XT*)L.za;
+    double c2 = (cf.fam == FAM_CHEB4) ? cf.c2[1] : cf.c2[0];
+    double rhoinv = cf.rhoinv;
+    if (L.sval && cf.fam == FAM_CHEB1) {  // scaled 1st-kind form: r = rho r^(0)
+      c2 *= rhoinv;
+      rhoinv = 1.0;
+    }
+    f.c2 = XT(c2);
+    f.beta = XT(cf.beta[1]);
+    f.rhoinv = XT(rhoinv);
+    return f;
+  }
+  static void run_first(amgps_ctx* c, const Level& L, const First& f, const XT* b) {
+    do_first(f.fam, L.n, b, (const XT*)L.dinv, f.r, f.z, f.x, f.c2, f.beta, f.rhoinv, c->nvec,
+             c->stream);
+  }
+
   // One smoother application on level l: x <- S(b, x) (x = 0 when xzero).
+  // c_ready: from zero, its first step has run already (first_of).
   // corrected: its first step has run (`correct`).
   // Returns true when it ran in the stored-operator form (then, from zero,
   // the level's za holds M^{-1} b for a following application with x given:
@@ -863,7 +896,7 @@ struct Engine {
       if (corrected) {
         j0 = 1;
       } else if (xzero) {
-        do_first(FAM_JAC, L.n, b, md, nullptr, nullptr, cur, XT(0), XT(0), XT(1), c->nvec, s);
+        if (!c_ready) run_first(c, L, first_of(c, L, cf, x), b);
         j0 = 1;
       }
       for (int j = j0; j < k; ++j) {
@@ -892,13 +925,7 @@ struct Engine {
     if (corrected) {
       rin_next = r;
     } else if (xzero) {
-      double c2 = (cf.fam == FAM_CHEB4) ? cf.c2[1] : cf.c2[0];
-      double rhoinv = cf.rhoinv;
-      if (L.sval && cf.fam == FAM_CHEB1) {  // scaled 1st-kind form: r = rho r^(0)
-        c2 *= rhoinv;
-        rhoinv = 1.0;
-      }
-      do_first(cf.fam, L.n, b, md, r, zc, x, XT(c2), XT(cf.beta[1]), XT(rhoinv), c->nvec, s);
+      if (!c_ready) run_first(c, L, first_of(c, L, cf, x), b);
       rin_next = (cf.fam == FAM_CHEB4) ? b : r;
     } else {
       StepArgs<VT, XT> a;
@@ -984,8 +1011,16 @@ struct Engine {
     }
   }
 
+  // Whether the residual, the restriction and the next level's first step run
+  // as one kernel (see RestrictArgs).
+  static bool fuse_restrict(const amgps_ctx* c, const Level& L) {
+    return !rec() && !L.xfer_general && L.split == 1 && L.n <= kFuseRows &&
+           !(c->nvec == 1 && level_uses_tma(c, L));
+  }
+
   // record: keep each level's post-smoother input (for the reverse pass);
-  // c_ready: the level's za already holds M^{-1} b (written by the PCG update)
+  // c_ready: the level's first step from zero has run (written by the PCG
+  // update or by the restriction)
   static void vcycle_level(amgps_ctx* c, int l, const XT* b, XT* x, bool record = false,
                            bool c_ready = false) {
     Level& L = c->lv[l];
@@ -1003,6 +1038,8 @@ struct Engine {
     // stored-operator form: za = M^{-1} b afterwards, for the post-smoother
     const bool c_kept = smooth(c, l, cf, b, x, true, c_ready);
     Level& C = c->lv[l + 1];
+    const bool replay = l + 1 == 1 && c->nvec == 1 && c->graph_ok && !record && !capturing(c);
+    bool first_done = false;  // of the next level
     {
       // b_{l+1} = P^T (b - A x): the true residual (into the level's r buffer,
       // free between the smoothers), then the children sums of each aggregate
@@ -1010,27 +1047,53 @@ struct Engine {
                    (double)L.nnz * sizeof(VT) + (double)L.explicit_entries * 4.0 +
                        (double)L.n * sizeof(XT) * 4 + (double)L.n * 4 + (double)C.n * 12 +
                        (L.xfer_general ? (double)L.xfer_stored * 6.0 : 0.0));
-      StepArgs<VT, XT> a;
-      a.A = devmat<VT>(L);
-      a.u = x;
-      a.rin = b;
-      a.zout = (XT*)L.r;
-      a.fam = FAM_RES;
-      a.init = true;
-      a.go = false;
-      run_step(c, L, a, s);
-      if (L.xfer_general) launch_xfer<XT>(L.Rm, (const XT*)L.r, (XT*)C.b, 0, L.rsplit, s);
-      else do_aggregate(L, (const XT*)L.r, (XT*)C.b, c->nvec, s);
+      if (fuse_restrict(c, L)) {
+        RestrictArgs<VT, XT> a;
+        a.A = devmat<VT>(L);
+        a.b = b;
+        a.u = x;
+        a.r = (XT*)L.r;
+        a.cptr = L.cptr;
+        a.cidx = L.cidx;
+        a.nc = L.nc;
+        a.bc = (XT*)C.b;
+        if (!C.coarsest && !replay) {
+          const First f = first_of(
+              c, C, make_coefs(C.spec.kind, C.spec.k, C.spec.w, C.spec.rho), (XT*)C.x);
+          a.fam = f.fam;
+          a.dinv = (const XT*)C.dinv;
+          a.rout = f.r;
+          a.zout = f.z;
+          a.xout = f.x;
+          a.c2 = f.c2;
+          a.beta = f.beta;
+          a.rhoinv = f.rhoinv;
+          first_done = true;
+        }
+        launch_restrict<VT, XT>(a, c->nvec, s);
+      } else {
+        StepArgs<VT, XT> a;
+        a.A = devmat<VT>(L);
+        a.u = x;
+        a.rin = b;
+        a.zout = (XT*)L.r;
+        a.fam = FAM_RES;
+        a.init = true;
+        a.go = false;
+        run_step(c, L, a, s);
+        if (L.xfer_general) launch_xfer<XT>(L.Rm, (const XT*)L.r, (XT*)C.b, 0, L.rsplit, s);
+        else do_aggregate(L, (const XT*)L.r, (XT*)C.b, c->nvec, s);
+      }
       ps.done();
     }
     {
       // levels >= 1 of the cycle, timed as one class-4 interval from level 0
       ProfScope ps(c, l == 0, 4, 0.0);
-      if (l + 1 == 1 && c->nvec == 1 && c->graph_ok && !record && !capturing(c)) {
+      if (replay) {
         CK(cudaGraphLaunch(c->gexec, s));
         c->launch_adjust += c->graph_kernels;
       } else {
-        vcycle_level(c, l + 1, (const XT*)C.b, (XT*)C.x, record);
+        vcycle_level(c, l + 1, (const XT*)C.b, (XT*)C.x, record, first_done);
       }
       ps.done();
     }

@@ -361,10 +361,10 @@ __device__ __forceinline__ void step_slice_mv(const StepArgs<VT, XT>& a, int64_t
 //   4th kind: z_1 = c2 M^{-1} b, x = beta_1 z_1 (r_0 = b is not copied)
 //   1st kind: r^(0) = (1/rho) M^{-1} b, d^(0) = r^(0)/theta, x = d^(0)
 //   Jacobi:   x = M^{-1} b
-template <class XT, int FAM, bool CG = false>
-__device__ __forceinline__ void first_row(int64_t i, const XT* b, XT di, XT* rout, XT* zout,
-                                          XT* xout, XT c2, XT beta, XT rhoinv) {
-  const XT bm = ldv<CG>(b + i) * di;
+template <class XT, int FAM>
+__device__ __forceinline__ void first_value(int64_t i, XT bi, XT di, XT* rout, XT* zout, XT* xout,
+                                            XT c2, XT beta, XT rhoinv) {
+  const XT bm = bi * di;
   if constexpr (FAM == FAM_CHEB4) {
     const XT z = c2 * bm;
     zout[i] = z;
@@ -378,6 +378,11 @@ __device__ __forceinline__ void first_row(int64_t i, const XT* b, XT di, XT* rou
   } else {
     xout[i] = bm;
   }
+}
+template <class XT, int FAM, bool CG = false>
+__device__ __forceinline__ void first_row(int64_t i, const XT* b, XT di, XT* rout, XT* zout,
+                                          XT* xout, XT c2, XT beta, XT rhoinv) {
+  first_value<XT, FAM>(i, ldv<CG>(b + i), di, rout, zout, xout, c2, beta, rhoinv);
 }
 
 // b_c[I] = sum of res over the children of coarse row I, in list order.  The
@@ -488,20 +493,20 @@ __device__ __forceinline__ void coarse_gemv_row(int i, int nc, const double* ain
   }
 }
 
-// Sum over a block (any blockDim multiple of 32, <= 1024); result valid in thread 0.
+// Sum over a block of kBlock threads; result valid in warp 0.  One warp adds
+// the values (eight a lane in thread order, then a butterfly): 12 FP64 warp
+// instructions of 16 clocks on the SM's one narrow pipe, where a butterfly in
+// each of the eight warps takes 45.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
+  __syncthreads();
+  sh[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x >= 32) return 0.0;
+  v = sh[threadIdx.x];
+#pragma unroll
+  for (int k = 1; k < kWarpsPerBlock; ++k) v += sh[threadIdx.x + 32 * k];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sh[warp] = v;
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  v = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-  if (warp == 0) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  }
   return v;
 }
 
@@ -511,7 +516,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // function of the problem size, so the result is bitwise reproducible.
 template <class Fin>
 __device__ __forceinline__ void grid_sum(double v, const RedWork& w, Fin fin) {
-  __shared__ double sh[32];
+  __shared__ double sh[kBlock];
   __shared__ bool last;
   double b = block_sum(v, sh);
   if (threadIdx.x == 0) {
@@ -531,6 +536,20 @@ __device__ __forceinline__ void grid_sum(double v, const RedWork& w, Fin fin) {
       *w.counter = 0u;
     }
   }
+}
+
+// Threads per block of a kernel of `threads` one-row threads (or lanes): 256,
+// fewer on levels that would leave SMs without a block -- an SM issues one FP64
+// warp instruction in 16 clocks, so the eight warps of a block take eight
+// times one warp's time (4096-row level: 0.5 us of FP64 issue on 16 SMs, 0.06
+// on 128).
+constexpr int kSms = 152;
+inline int small_block(int64_t threads) {
+  const int64_t warps = (threads + 31) / 32, per = (warps + kSms - 1) / kSms;
+  return 32 * (int)(per < 1 ? 1 : per > kWarpsPerBlock ? kWarpsPerBlock : per);
+}
+inline unsigned blocks_of(int64_t threads, int block) {
+  return (unsigned)((threads + block - 1) / block);
 }
 
 // Launch of a kernel that calls pdl_wait() as the programmatic dependent of

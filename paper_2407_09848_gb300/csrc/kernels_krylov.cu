@@ -92,7 +92,7 @@ void launch_spmv_dot_mv(const DevMat<double>& A, const double* p, double* q, con
 template <class Fin>
 __device__ __forceinline__ void grid_sum3(double v0, double v1, double v2, const RedWork& w,
                                           Fin fin) {
-  __shared__ double sh[32];
+  __shared__ double sh[kBlock];
   __shared__ bool last;
   const double b0 = block_sum(v0, sh);
   const double b1 = block_sum(v1, sh);
@@ -387,7 +387,7 @@ template <class XT>
 __global__ void __launch_bounds__(kBlock) k_coarse_gemv(int nc, const double* __restrict__ ainv,
                                                         const XT* b, XT* x, int nvec) {
   const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (i >= nc) return;
   const int v0 = blockIdx.y * kGemvVecs;
   const size_t o = (size_t)v0 * nc;
@@ -398,8 +398,9 @@ template <class XT>
 void launch_coarse_gemv(int nc, const double* ainv, const XT* b, XT* x, int nvec,
                         cudaStream_t s) {
   if (nc == 0) return;
-  const dim3 g((nc + kWarpsPerBlock - 1) / kWarpsPerBlock, (nvec + kGemvVecs - 1) / kGemvVecs);
-  launch_dep(k_coarse_gemv<XT>, g, kBlock, 0, s, nc, ainv, b, x, nvec);
+  const int gy = (nvec + kGemvVecs - 1) / kGemvVecs, blk = small_block((int64_t)nc * 32 * gy);
+  const dim3 g(blocks_of((int64_t)nc * 32, blk), gy);
+  launch_dep(k_coarse_gemv<XT>, g, blk, 0, s, nc, ainv, b, x, nvec);
 }
 
 // Dense Cholesky A = L L^T (right-looking, one block, in place in `work`,
