@@ -54,8 +54,10 @@ __device__ bool grid_barrier(const CycleSync& sy, unsigned target) {
   return ok != 0;
 }
 
+// (a call, not inlined: the kernel holds some forty of these, and the compiler
+// hoists the loads of inlined ones together into thousands of spilled bytes)
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
-__device__ __forceinline__ void cy_slices(const StepArgs<VT, XT>& a, int64_t gw, int64_t nw,
+__device__ __noinline__ void cy_slices(const StepArgs<VT, XT>& a, int64_t gw, int64_t nw,
                                           int lane) {
   for (int64_t s = gw; s < a.A.nslices; s += nw)
     step_slice<VT, XT, FAM, INIT, WR, ZOWN, true>(a, s, lane);

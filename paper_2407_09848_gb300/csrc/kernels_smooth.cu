@@ -95,9 +95,91 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
   step_finish<VT, XT, FAM, INIT, WR, ZOWN>(a, ro, acc, rin, xin, di, zo);
 }
 
+// Split form of the FP64 levels with too few slices for the SMs: a slice's 32
+// rows are also shared out over E blocks (R = 32 / E rows each), E lanes of a
+// warp working on one row, so the split of the level is E x G.  With one block
+// per slice the 54 slices of a 1728-row level of 573 entries a row kept 54 SMs
+// busy, their FP64 pipes alone for 5 us; four steps there take 39.0 us instead of
+// 47.5 (call included).  Where one block per slice fills the SMs the shorter
+// runs of a row's values cost more than they give (432 slices: 56.3 us instead
+// of 51.3), so E is the smallest with two blocks an SM.  G warps of a block
+// share the rows' entries (G = 1: a block holds kWideUnits independent units).
+constexpr int kWideLanes = 8;  // the largest E
+constexpr int kWideUnits = 4;
+struct WideShape {
+  int E, G, units;  // lanes per row, warps per unit, units per block
+};
+inline WideShape wide_shape(int split, int64_t nslices) {
+  WideShape w;
+  w.E = 1;
+  while (w.E < kWideLanes && w.E < split && nslices * w.E < 2 * kSms) w.E *= 2;
+  w.G = split / w.E;
+  w.units = w.G == 1 ? kWideUnits : 1;
+  return w;
+}
+
+// The part of a row sum that unit `unit` (a slice's rows first .. first + R-1)
+// leaves to its warp 0: calls body(row, sum) for every row there.
+template <int SIGN, int E, class Init, class Body>
+__device__ __forceinline__ void wide_unit(const DevMat<double>& A, const double* u, int G, Init init,
+                                          Body body) {
+  constexpr int R = 32 / E;
+  __shared__ double part[kMaxSplit / 2][R];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = G > 1 ? warp : 0;
+  const int64_t nunits = A.nslices * E;
+  const int64_t unit = G > 1 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * kWideUnits + warp;
+  if (unit >= nunits) return;  // whole warps; G = 1 needs no block-wide meeting
+  const int64_t s = unit / E;
+  const int first = (int)(unit % E) * R;
+  const SliceDesc d = ld_desc(A.sd + s);
+  const int64_t row0 = s * kSlice + first, row = row0 + lane % R;
+  const int k0 = (int)((int64_t)d.w * g / G), k1 = (int)((int64_t)d.w * (g + 1) / G);
+  const bool own = g == 0 && lane < R && row < A.n;
+  double t = row_accumulate_wide<SIGN, E>(
+      A, d, first, row0, u, [&] { return own ? init(row) : 0.0; }, k0, k1);
+  if (G > 1) {
+    if (lane < R) part[g][lane] = t;
+    __syncthreads();
+    if (g == 0)
+      for (int q = 1; q < G; ++q) t += part[q][lane % R];
+  }
+  if (own) body(row, t);
+}
+
+template <int E, int FAM, bool INIT, bool WR, bool ZOWN>
+__global__ void __launch_bounds__(32 * (kMaxSplit / E)) k_step_wide(const StepArgs<double, double> a,
+                                                              int G) {
+  const int64_t o = (int64_t)blockIdx.y * a.A.n;  // vector of a batch
+  using F = StepForm<FAM, INIT>;
+  double rin = 0.0, xin = 0.0, zo = 0.0, di = 0.0;
+  wide_unit<F::kSign, E>(
+      a.A, a.u + o, G,
+      [&](int64_t row) {
+        if (step_needs_dinv<FAM>()) di = __ldg(a.dinv + row);
+        rin = ldv<false>(a.rin + o + row);
+        if (FAM != FAM_RES) xin = ldv<false>(a.xin + o + row);
+        if (ZOWN) zo = ldv<false>(a.zown + o + row);
+        return step_init<FAM, F::kResidual>(rin, di);
+      },
+      [&](int64_t row, double t) {
+        step_finish<double, double, FAM, INIT, WR, ZOWN>(a, o + row, t, rin, xin, di, zo);
+      });
+}
+
+template <int FAM, bool INIT, bool WR, bool ZOWN>
+static void go_wide(const StepArgs<double, double>& a, const WideShape& w, cudaStream_t s) {
+  const dim3 g((unsigned)((a.A.nslices * w.E + w.units - 1) / w.units), a.nvec);
+  auto* k = w.E == 2   ? k_step_wide<2, FAM, INIT, WR, ZOWN>
+            : w.E == 4 ? k_step_wide<4, FAM, INIT, WR, ZOWN>
+                       : k_step_wide<8, FAM, INIT, WR, ZOWN>;
+  launch_dep(k, g, 32 * w.G * w.units, 0, s, a, w.G);
+}
+
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
 static void go(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
-  if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
+  constexpr bool f64 = std::is_same<VT, double>::value && std::is_same<XT, double>::value;
+  if constexpr (f64) {
     if (a.nvec > 1 && a.split == 1) {  // batches run on all slices
       const int gy = (a.nvec + kVecs - 1) / kVecs, blk = small_block(work * kSlice * gy);
       launch_dep(k_step_mv<VT, XT, FAM, INIT, WR, ZOWN>, dim3(blocks_of(work * kSlice, blk), gy), blk,
@@ -105,10 +187,17 @@ static void go(const StepArgs<VT, XT>& a, int64_t work, cudaStream_t s) {
       return;
     }
   }
-  if (a.split > 1)
+  if constexpr (f64 && !is_op(FAM)) {  // FP32 rows keep their order of summation
+    const WideShape w = wide_shape(a.split, work);
+    if (w.E > 1) {
+      go_wide<FAM, INIT, WR, ZOWN>(a, w, s);
+      return;
+    }
+  }
+  if (a.split > 1) {
     launch_dep(k_step_split<VT, XT, FAM, INIT, WR, ZOWN>, dim3((unsigned)work, a.nvec),
                32 * a.split, 0, s, a);
-  else {
+  } else {
     const int blk = small_block(work * kSlice);
     launch_dep(k_step<VT, XT, FAM, INIT, WR, ZOWN>, blocks_of(work * kSlice, blk), blk, 0, s, a);
   }
@@ -567,9 +656,27 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_xfer_split(const DevMat<doub
   y[row] = t;
 }
 
+template <int E>
+__global__ void __launch_bounds__(32 * (kMaxSplit / E)) k_xfer_wide(const DevMat<double> M,
+                                                              const double* u, double* y, int add,
+                                                              int G) {
+  wide_unit<1, E>(
+      M, u, G, [&](int64_t row) { return add ? ldv<false>(y + row) : 0.0; },
+      [&](int64_t row, double t) { y[row] = t; });
+}
+
 template <class XT>
 void launch_xfer(const DevMat<double>& M, const XT* u, XT* y, int add, int split, cudaStream_t s) {
   if (M.nslices == 0) return;
+  if constexpr (std::is_same<XT, double>::value) {
+    const WideShape w = wide_shape(split, M.nslices);
+    if (w.E > 1) {
+      auto* k = w.E == 2 ? k_xfer_wide<2> : w.E == 4 ? k_xfer_wide<4> : k_xfer_wide<8>;
+      launch_dep(k, (unsigned)((M.nslices * w.E + w.units - 1) / w.units), 32 * w.G * w.units, 0, s,
+                 M, u, y, add, w.G);
+      return;
+    }
+  }
   if (split > 1)
     launch_dep(k_xfer_split<XT>, (unsigned)M.nslices, 32 * split, 0, s, M, u, y, add);
   else
