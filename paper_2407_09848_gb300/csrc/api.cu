@@ -1988,11 +1988,12 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
 // fewer launches and a 7-point row's values are read once for four vectors.
 // B x n_0 is kept near kBatchRows: measured on the 32 vectors of a 64^3
 // problem, one pass (6 pre-cycles, loss and gradient) takes 43.2 ms one by one
-// and 17.8 ms in two batches of 16 (its FP64 multiply-adds alone: 10.6 ms).
+// and 17.8 ms in two batches of 16 (its FP64 multiply-adds alone: 10.6 ms); with
+// the later kernels 16.8 in two batches and 15.5 in one of 32 (0.95 GB).
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int64_t kBatchRows = int64_t(1) << 22;
+constexpr int64_t kBatchRows = int64_t(1) << 23;
 
 // The batch buffers come from one stream-ordered pool per device, shared by
 // the contexts of the process (a training run holds hundreds of contexts and
