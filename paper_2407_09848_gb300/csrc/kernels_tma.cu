@@ -92,6 +92,16 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// The same with an L2 eviction policy.
+__device__ __forceinline__ void bulk_g2s_policy(void* dst, const void* src, uint32_t bytes,
+                                                uint64_t* bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], "
+      "%2, [%3], %4;" ::"r"(su32(dst)),
+      "l"(src), "r"(bytes), "r"(su32(bar)), "l"(policy)
+      : "memory");
+}
+
 template <class XT>
 __device__ __forceinline__ XT widen(double v) { return XT(v); }
 template <class XT>
@@ -138,12 +148,18 @@ __global__ void __launch_bounds__((tma_warps<XT>() + 1) * 32, TmaShape<XT>::kCta
     constexpr bool c0 = reads_slot0<FAM, INIT>(), c1 = reads_slot1<FAM, ZOWN>();
     constexpr int nvec = (c0 ? 1 : 0) + (c1 ? 1 : 0) + (wdi ? 1 : 0);
     const uint32_t stage_tx = (uint32_t)(p.vals_bytes + nvec * p.vec_bytes + p.win_bytes);
+    // Values are read once per step and come first for eviction, so that the
+    // step's vectors, which its neighbour tiles and the next step read, stay in
+    // L2: 256^3 solve 88.1 -> 84.6 ms, six steps on 173x151x129 374 -> 352 us, the
+    // FP32 128^3 level-0 step 26.3 -> 23.9 us, BF16 192^3 solve 75.4 -> 74.6 ms.
+    uint64_t evict_first;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(evict_first));
     // a tile's values (no kernel of the chain writes them) ...
     auto copy_vals = [&](int st, long long r0, long long vb) {
       stage_r0[st] = r0;
       mbar_expect_tx(&full[st], stage_tx);
-      bulk_g2s(stages + (size_t)st * p.stage_bytes, a.A.val + vb, (uint32_t)p.vals_bytes,
-               &full[st]);
+      bulk_g2s_policy(stages + (size_t)st * p.stage_bytes, a.A.val + vb, (uint32_t)p.vals_bytes,
+                      &full[st], evict_first);
     };
     // ... and its vectors, which the previous kernel may have written
     auto copy_vecs = [&](int st, long long r0) {
