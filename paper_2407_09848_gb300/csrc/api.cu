@@ -562,6 +562,8 @@ double op_inst(const Level& L, int fam, bool s0, bool s0add, bool s1, bool wt) {
 // ---------------------------------------------------------------------------
 template <class VT, class XT>
 struct Engine {
+  using Value = VT;
+  using Vector = XT;
   // While a phase list is being recorded (build_tail), the kernel calls below
   // append their arguments to it instead of launching.
   static std::vector<CyclePhase<VT, XT>>*& rec() {
@@ -1715,9 +1717,34 @@ void fcg1_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit,
 // the same.
 bool loop_fp32(const amgps_ctx* c) { return c->prec != AMGPS_F64 && c->flexible != 2; }
 
-// One iteration, from r (and, with fuse_c, c = M^{-1} r; with loop_fp32, r in
-// FP32) to the next r.
-void loop_body(amgps_ctx* c, const PcgLoop& lp, bool fuse_c) {
+// The first step of level 0's smoother as part of the r update (level 0 not
+// the coarsest, not the one-reduction form, and not where it would overwrite
+// the z that the flexible form still needs); r and x: the V-cycle's boundary
+// vectors.  BF16 192^3 solve 77.5 -> 75.4 ms, 32^3 778 -> 766 us.
+template <class VT, class XT>
+RFirst<XT> loop_first(amgps_ctx* c, XT* r, XT* x) {
+  RFirst<XT> f;
+  const Level& L = c->lv[0];
+  if constexpr (sizeof(XT) == 4) f.fout = r;
+  if (L.coarsest || c->flexible == 2) return f;
+  const Coefs cf = make_coefs(L.spec.kind, L.spec.k, L.spec.w, L.spec.rho);
+  const auto g = Engine<VT, XT>::first_of(c, L, cf, x);
+  if (c->flexible == 1 && g.x == x) return f;
+  f.fam = g.fam;
+  f.dinv = (const XT*)L.dinv;
+  f.rout = g.r;
+  f.zout = g.z;
+  f.xout = g.x;
+  f.c2 = g.c2;
+  f.beta = g.beta;
+  f.rhoinv = g.rhoinv;
+  return f;
+}
+
+// One iteration, from r (and its first smoother step; with loop_fp32 r in
+// FP32 too) to the next r.
+template <class VT, class XT>
+void loop_body(amgps_ctx* c, const PcgLoop& lp) {
   Level& L = c->lv[0];
   cudaStream_t s = c->stream;
   const int64_t n = L.n;
@@ -1725,42 +1752,32 @@ void loop_body(amgps_ctx* c, const PcgLoop& lp, bool fuse_c) {
   RedWork rw_dot = redwork(c, 0, n, kRedBlocksPerSm), rw_spmv = redwork(c, 1, n),
           rw_upd = redwork(c, 2, n, kRedBlocksPerSm);
   rw_spmv.grid = reduction_grid(L.nslices * kSlice, c->nsm);
-  double *z = c->pz, *p = c->pp, *q = c->pq, *r = c->pr;
-  // FP32 and BF16 hierarchies (cg, flexible): the V-cycle's boundary vectors
-  // stay FP32 -- the r update writes the right-hand side beside r, the dot and
-  // the direction update widen z as they read it -- instead of two conversion
-  // passes (28 B a row and two launches; the same values): BF16 192^3 solve
-  // 80.1 -> 77.6 ms, FP32 128^3 9757 -> 9680 us.
-  if (loop_fp32(c)) {
-    float *rf = (float*)L.b, *zf = (float*)L.x;
-    if (c->flexible == 1) launch_dot(n, r, zf, rw_dot, c->dscal, S_RZP, 0, s);
-    if (c->prec == AMGPS_F32) Engine<float, float>::vcycle_level(c, 0, rf, zf);
-    else Engine<__nv_bfloat16, float>::vcycle_level(c, 0, rf, zf);
-    launch_dot(n, r, zf, rw_dot, c->dscal, S_RZ, c->flexible == 1 ? 2 : 1, s);
-    launch_xpay_x(n, zf, p, nullptr, c->dscal, 1, s, lp);
-    launch_spmv_dot(A, p, q, rw_spmv, c->dscal, s);
-    launch_r_update(n, q, r, rw_upd, c->dscal, s, nullptr, nullptr, rf, lp);
-    return;
-  }
-  if (c->flexible == 1) launch_dot(n, r, z, rw_dot, c->dscal, S_RZP, 0, s);
-  with_engine(c, [&](auto eng) { decltype(eng)::vcycle_plain(c, r, z, fuse_c); });
+  double *p = c->pp, *q = c->pq, *r = c->pr;
+  using E = Engine<VT, XT>;
   if (c->flexible == 2) {
-    launch_spmv_dot3(A, z, c->pz2, r, q, 0, rw_spmv, c->dscal, s);
-    launch_fcg_update(n, z, c->pz2, p, q, nullptr, r, 0, rw_upd, c->dscal, s, lp);
+    E::vcycle_plain(c, r, c->pz, false);
+    launch_spmv_dot3(A, c->pz, c->pz2, r, q, 0, rw_spmv, c->dscal, s);
+    launch_fcg_update(n, c->pz, c->pz2, p, q, nullptr, r, 0, rw_upd, c->dscal, s, lp);
     return;
   }
+  // FP32 and BF16 hierarchies: the V-cycle's boundary vectors stay FP32 -- the
+  // r update writes the right-hand side beside r, the dot and the direction
+  // update widen z as they read it -- instead of two conversion passes (28 B a
+  // row and two launches; the same values): BF16 192^3 solve 80.1 -> 77.6 ms,
+  // FP32 128^3 9757 -> 9680 us.
+  constexpr bool f32 = sizeof(XT) == 4;
+  XT *rv = f32 ? (XT*)L.b : (XT*)r, *z = f32 ? (XT*)L.x : (XT*)c->pz;
+  const RFirst<XT> first = loop_first<VT, XT>(c, rv, z);
+  if (c->flexible == 1) launch_dot(n, r, z, rw_dot, c->dscal, S_RZP, 0, s);
+  E::vcycle_level(c, 0, rv, z, false, first.fam >= 0);
   launch_dot(n, r, z, rw_dot, c->dscal, S_RZ, c->flexible == 1 ? 2 : 1, s);
   launch_xpay_x(n, z, p, nullptr, c->dscal, 1, s, lp);
   launch_spmv_dot(A, p, q, rw_spmv, c->dscal, s);
-  if (fuse_c)
-    launch_r_update(n, q, r, rw_upd, c->dscal, s, (const double*)L.dinv, (double*)L.za, nullptr,
-                    lp);
-  else
-    launch_r_update(n, q, r, rw_upd, c->dscal, s, nullptr, nullptr, nullptr, lp);
+  launch_r_update(n, q, r, rw_upd, c->dscal, s, first, lp);
 }
 
 // Builds c->loop_exec; false (and c->loop_refused) if the runtime refuses it.
-bool build_loop(amgps_ctx* c, bool fuse_c) {
+bool build_loop(amgps_ctx* c) {
   if (c->loop_ok) return true;
   if (c->loop_refused) return false;
   if (c->loop_exec) {
@@ -1801,7 +1818,9 @@ bool build_loop(amgps_ctx* c, bool fuse_c) {
     if (e == cudaSuccess) body = np.conditional.phGraph_out[0];
   }
   if (e == cudaSuccess) e = capture(body, [&] {
-    loop_body(c, lp, fuse_c);
+    if (c->prec == AMGPS_F64) loop_body<double, double>(c, lp);
+    else if (c->prec == AMGPS_F32) loop_body<float, float>(c, lp);
+    else loop_body<__nv_bfloat16, float>(c, lp);
     check_launch();
   });
   const int64_t captured = launches_enqueued() - before;
@@ -1821,7 +1840,7 @@ bool build_loop(amgps_ctx* c, bool fuse_c) {
 
 // The solve through c->loop_exec; arguments and results as pcg_impl.
 void pcg_loop(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, int* iters,
-              double* relres, bool* converged, bool fuse_c) {
+              double* relres, bool* converged) {
   Level& L = c->lv[0];
   cudaStream_t s = c->stream;
   const int64_t n = L.n;
@@ -1843,9 +1862,15 @@ void pcg_loop(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
   CK(cudaMemcpyAsync(c->dscal + S_RTOL, c->hscal + S_RTOL, 2 * sizeof(double),
                      cudaMemcpyHostToDevice, s));
   launch_dot(n, b, b, redwork(c, 0, n, kRedBlocksPerSm), c->dscal, S_BB, 0, s);
-  if (fuse_c)
-    launch_first<double>(FAM_JAC, n, c->pr, (const double*)L.dinv, nullptr, nullptr, (double*)L.za,
-                         0.0, 0.0, 1.0, 1, s);
+  with_engine(c, [&](auto eng) {  // what the r update does later
+    using E = decltype(eng);
+    using VT = typename E::Value;
+    using XT = typename E::Vector;
+    XT *rv = sizeof(XT) == 4 ? (XT*)L.b : (XT*)c->pr, *z = sizeof(XT) == 4 ? (XT*)L.x : (XT*)c->pz;
+    if (loop_first<VT, XT>(c, rv, z).fam >= 0)
+      E::run_first(
+          c, L, E::first_of(c, L, make_coefs(L.spec.kind, L.spec.k, L.spec.w, L.spec.rho), z), rv);
+  });
   CK(cudaGraphLaunch(c->loop_exec, s));
   check_launch();
   CK(cudaMemcpyAsync(c->hscal, c->dscal, S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1896,10 +1921,9 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
   // The loop on the device, unless the kernels are being timed (events between
   // them), the caller captures the stream, or the coarse levels run as a
   // cooperative kernel; a caller's preconditioner keeps the host loop.
-  const bool fuse_loop = fuse_c && c->flexible != 2;
   if (!precond && !c->prof && !c->use_cycle && !Engine<double, double>::capturing(c) &&
-      build_loop(c, fuse_loop)) {
-    pcg_loop(c, b, x, rtol, maxit, iters, relres, converged, fuse_loop);
+      build_loop(c)) {
+    pcg_loop(c, b, x, rtol, maxit, iters, relres, converged);
     return;
   }
   if (c->flexible == 2) {
@@ -1941,10 +1965,9 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
       ps.done();
     }
     // r -= alpha q now; x += alpha p is deferred to the direction update
-    if (fuse_c)
-      launch_r_update(n, c->pq, c->pr, rw_upd, c->dscal, s, (const double*)L.dinv, (double*)L.za);
-    else
-      launch_r_update(n, c->pq, c->pr, rw_upd, c->dscal, s);
+    RFirst<double> first;
+    if (fuse_c) first = loop_first<double, double>(c, c->pr, nullptr);
+    launch_r_update(n, c->pq, c->pr, rw_upd, c->dscal, s, first);
     check_launch();
     CK(cudaMemcpyAsync(c->hscal, c->dscal, S_COUNT * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaEventRecord(c->ev_sync, s));

@@ -233,15 +233,16 @@ void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, d
 }
 
 // r -= alpha q ; r.r (S_RR).  The x update of the same iteration is deferred
-// to k_xpay_x, which reads p anyway.  WC: also c = M^{-1} r (the product the
-// stored-operator smoother of the next V-cycle starts from, same operation
-// as its own c pass).  WF: also r rounded to FP32 (the right-hand side of an
-// FP32 or BF16 V-cycle).
-template <bool WC, bool WF>
-__global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n, const double* q, double* r,
-                                                     const RedWork w, double* scal,
-                                                     const double* __restrict__ dinv, double* cout,
-                                                     float* fout, cudaGraphConditionalHandle h) {
+// to k_xpay_x, which reads p anyway.  FAM >= 0: also the first step from zero
+// of the next V-cycle's smoother (the same operations as its own launch; in the
+// stored-operator form that is c = M^{-1} r), which saves that launch and its
+// read of r.
+template <class FT, int FAM>
+__global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n, const double* q,
+                                                                      double* r, const RedWork w,
+                                                                      double* scal,
+                                                                      const RFirst<FT> f,
+                                                                      cudaGraphConditionalHandle h) {
   pdl_wait();
   pdl_go();
   const double alpha = ldv<false>(scal + S_ALPHA);
@@ -250,8 +251,11 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n,
   auto one = [&](uint32_t i, double qi, double ri) {
     ri = fma(-alpha, qi, ri);
     r[i] = ri;
-    if constexpr (WC) cout[i] = ri * __ldg(dinv + i);
-    if constexpr (WF) fout[i] = (float)ri;
+    const FT bi = (FT)ri;
+    if constexpr (sizeof(FT) == 4) f.fout[i] = bi;
+    if constexpr (FAM >= 0) {
+      first_value<FT, FAM>(i, bi, __ldg(f.dinv + i), f.rout, f.zout, f.xout, f.c2, f.beta, f.rhoinv);
+    }
     acc = fma(ri, ri, acc);
   };
   uint32_t i = blockIdx.x * kBlock + threadIdx.x;
@@ -268,12 +272,19 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n,
   });
 }
 
+template <class FT>
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
-                     cudaStream_t s, const double* dinv, double* cout, float* fout,
-                     const PcgLoop& loop) {
-  auto* k = cout ? k_r_update<true, false> : fout ? k_r_update<false, true> : k_r_update<false, false>;
-  launch_dep(k, w.grid, kBlock, 0, s, n, q, r, w, scal, dinv, cout, fout, loop.handle);
+                     cudaStream_t s, const RFirst<FT>& f, const PcgLoop& loop) {
+  auto* k = f.fam < 0              ? k_r_update<FT, -1>
+            : f.fam == FAM_CHEB4   ? k_r_update<FT, FAM_CHEB4>
+            : f.fam == FAM_CHEB1   ? k_r_update<FT, FAM_CHEB1>
+                                   : k_r_update<FT, FAM_JAC>;
+  launch_dep(k, w.grid, kBlock, 0, s, n, q, r, w, scal, f, loop.handle);
 }
+template void launch_r_update<double>(int64_t, const double*, double*, const RedWork&, double*,
+                                      cudaStream_t, const RFirst<double>&, const PcgLoop&);
+template void launch_r_update<float>(int64_t, const double*, double*, const RedWork&, double*,
+                                     cudaStream_t, const RFirst<float>&, const PcgLoop&);
 
 // x += alpha p with the previous alpha, then p = z + beta p (x_beta = 1), or
 // only x += alpha p (x_beta = 0: the last iteration)

@@ -52,12 +52,21 @@ void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, d
 // start of a solve in a loop: alpha = beta = 0 and r_old.z_old infinite (the
 // first direction is then z), no iterations done; the loop runs if b.b > 0
 void launch_pcg_begin(double* scal, cudaGraphConditionalHandle handle, cudaStream_t s);
-// standard PCG with the x update deferred: r -= alpha q and r.r (with cout:
-// also cout = dinv .* r, with fout: also r in FP32); later x += alpha p together with p = z + beta p
+// What the r update also does for the V-cycle that follows: the first step from
+// zero of level 0's smoother on r (fam >= 0; first_value in
+// kernels_common.cuh), in FP32 for FT = float, with r itself in fout
+template <class FT>
+struct RFirst {
+  int fam = -1;
+  const FT* dinv = nullptr;
+  FT *rout = nullptr, *zout = nullptr, *xout = nullptr, *fout = nullptr;
+  FT c2 = 0, beta = 0, rhoinv = 1;
+};
+// standard PCG with the x update deferred: r -= alpha q and r.r; later x += alpha p together with p = z + beta p
 // (with_p = 0: x only)
+template <class FT = double>
 void launch_r_update(int64_t n, const double* q, double* r, const RedWork& w, double* scal,
-                     cudaStream_t s, const double* dinv = nullptr, double* cout = nullptr,
-                     float* fout = nullptr, const PcgLoop& loop = {});
+                     cudaStream_t s, const RFirst<FT>& first = {}, const PcgLoop& loop = {});
 template <class ZT>
 void launch_xpay_x(int64_t n, const ZT* z, double* p, double* x, const double* scal, int with_p,
                    cudaStream_t s, const PcgLoop& loop = {});
