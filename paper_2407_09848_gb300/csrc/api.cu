@@ -2241,7 +2241,7 @@ void load_general_transfer(amgps_ctx* c, Level& L, const amgps_csr& P) {
   const amgps_csr R{nc, n, P.nnz, rptr.data(), rcol.data(), rval.data()};
   auto put = [&](const amgps_csr& M, DevMat<double>& d, int& split) {
     HostSell h = build_sell(M, false);
-    split = split_for(h.stored, h.nslices);
+    split = split_for(h.stored, h.nslices, c->prec == AMGPS_F64);
     d.n = M.n_rows;
     d.nslices = h.nslices;
     d.sd = dupload(c, h.sd.data(), h.sd.size());
@@ -2416,7 +2416,7 @@ void load_levels(amgps_ctx* c, int n_levels, const amgps_csr* A, const amgps_csr
       // SpMV of a single-level hierarchy and for l1-Jacobi coarse sweeps
     }
     HostSell h = build_sell(A[l]);
-    L.split = split_for(h.stored, h.nslices);
+    L.split = split_for(h.stored, h.nslices, prec == AMGPS_F64);
     L.nslices = h.nslices;
     L.stored = h.stored;
     L.explicit_entries = h.explicit_entries;

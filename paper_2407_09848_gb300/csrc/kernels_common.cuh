@@ -143,6 +143,57 @@ __device__ __forceinline__ XT row_accumulate(const DevMat<VT>& A, const SliceDes
   return t;
 }
 
+// The same sum with the entries of a row shared by E lanes of a warp: lane
+// q R + r (R = 32 / E) takes entries k0 + q, k0 + q + E, ... of row r0 + r of the
+// slice (r0 = `first`), the E partial sums are then added over the lanes, and
+// every lane of a row ends with its sum.  init() counts in lanes q = 0 only.
+template <int SIGN, int E, class Init>
+__device__ __forceinline__ double row_accumulate_wide(const DevMat<double>& A, const SliceDesc d,
+                                                      int first, int64_t row0, const double* u,
+                                                      Init init, int k0, int k1) {
+  constexpr int R = 32 / E, NB = 4;
+  const int lane = threadIdx.x & 31, r = lane % R, q = lane / R;
+  const int64_t nm1 = A.n - 1, row = row0 + r;
+  const double* val = A.val + d.vbase + first + r;
+  double a[NB];
+  int32_t c[NB];
+  auto fetch = [&](int kb) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      const int k = kb + j * E;
+      if (k < k1) {
+        a[j] = ldval(val + (int64_t)k * kSlice);
+        if (d.cref >= 0) {
+          const int64_t cc = row + (int64_t)__ldg(A.off + d.cref + k);
+          c[j] = (int32_t)(cc < 0 ? 0 : (cc > nm1 ? nm1 : cc));
+        } else {
+          c[j] = __ldg(A.col + d.vbase + first + r + (int64_t)k * kSlice);
+        }
+      }
+    }
+  };
+  fetch(k0 + q);
+  pdl_wait();
+  pdl_go();
+  double t = init();
+  for (int kb = k0 + q; kb < k1; kb += NB * E) {
+    double av[NB], uv[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      if (kb + j * E < k1) uv[j] = ldv<false>(u + c[j]);
+      av[j] = a[j];
+    }
+    fetch(kb + NB * E);
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+      if (kb + j * E < k1) t = fma(SIGN > 0 ? av[j] : -av[j], uv[j], t);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = R; o < 32; o *= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
 // The whole row: entries 0 .. w-1 of the slice.
 template <int SIGN, class VT, class XT>
 __device__ __forceinline__ XT row_spmv(const DevMat<VT>& A, int64_t s, int lane, int64_t row,
@@ -248,7 +299,7 @@ __device__ __forceinline__ void step_slice(const StepArgs<VT, XT>& a, int64_t s,
   constexpr int kSign = StepForm<FAM, INIT>::kSign;
   if constexpr (is_op(FAM)) {
     XT uc = XT(0);
-    const XT acc = row_accumulate<kSign, VT, XT, CG, WAIT, sizeof(XT) == 8 ? 4 : 8, false>(
+    const XT acc = row_accumulate<kSign, VT, XT, CG, WAIT, sizeof(XT) == 8 ? 4 : 8, WAIT && sizeof(XT) == 8>(
         a.A, d, lane, row, a.u,
         [&] {
           XT s0 = XT(0), s1 = XT(0);
@@ -265,7 +316,7 @@ __device__ __forceinline__ void step_slice(const StepArgs<VT, XT>& a, int64_t s,
   }
   XT rin = XT(0), xin = XT(0), zo = XT(0), di = XT(0);
   if (live && step_needs_dinv<FAM>()) di = __ldg(a.dinv + row);  // formed at set-up
-  const XT acc = row_accumulate<kSign, VT, XT, CG, WAIT, sizeof(XT) == 8 ? 4 : 8, false>(
+  const XT acc = row_accumulate<kSign, VT, XT, CG, WAIT, sizeof(XT) == 8 ? 4 : 8, WAIT && sizeof(XT) == 8>(
       a.A, d, lane, row, a.u,
       [&] {
         if (live) {

@@ -80,23 +80,30 @@ void require_positive_diagonal(const amgps_csr& A) {
   });
 }
 
-// Warps per slice for the split kernels (measured on the 256^3
-// smoothed-aggregation levels): 1 while rows average under 24 stored entries;
-// otherwise the larger of a width term (the power of two nearest avg / 32 once
-// avg >= 48) and a parallelism term (the power of two at or below
-// 24576 / slices, so small levels still field ~24k warps), capped at avg / 8
-// entries per warp and kMaxSplit.
-int split_for(int64_t stored, int64_t nslices) {
+// Warps per slice for the split kernels: 1 while rows average under 24 stored
+// entries, at least 8 entries a warp, at most kMaxSplit.
+// FP64 rows: the largest power of two that keeps the level in one resident wave
+// (kWaveWarps: 32 warps of 64 registers on each SM).  The kernels fetch ahead,
+// so a wave of long rows is bound by FP64 issue, and every further wave pays
+// its first three loads again (four steps and the call, 96^3 smoothed
+// aggregation: 3456 slices of 32 entries 60.4 us with 4 warps a slice, 53.4
+// with 1; 432 of 165 entries 49.6 with 16, 42.5 with 8).
+// FP32 rows keep the rule their order of summation was fixed by (measured on the
+// 256^3 levels, kernels that did not fetch ahead): the larger of a width term
+// (the power of two nearest avg / 32 once avg >= 48) and a parallelism term (the
+// power of two at or below 24576 / slices).
+int split_for(int64_t stored, int64_t nslices, bool f64) {
+  constexpr double kWaveWarps = 32 * 152;
   if (nslices == 0) return 1;
   const double avg = (double)stored / ((double)nslices * kSlice);
   if (avg < 24.0) return 1;
-  int g1 = 1;
-  if (avg >= 48.0)
-    while (g1 < kMaxSplit && 2.0 * g1 <= avg / 32.0 * 1.41421356) g1 *= 2;
-  int g2 = 1;
-  while (g2 < kMaxSplit && 2.0 * g2 <= 24576.0 / (double)nslices) g2 *= 2;
   int cap = 1;
   while (cap < kMaxSplit && 2.0 * cap <= avg / 8.0) cap *= 2;
+  const double most = f64 ? kWaveWarps : 24576.0;
+  int g1 = 1, g2 = 1;
+  if (!f64 && avg >= 48.0)
+    while (g1 < kMaxSplit && 2.0 * g1 <= avg / 32.0 * 1.41421356) g1 *= 2;
+  while (g2 < kMaxSplit && 2.0 * g2 <= most / (double)nslices) g2 *= 2;
   return std::max(1, std::min(std::max(g1, g2), cap));
 }
 

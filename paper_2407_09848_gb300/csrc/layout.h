@@ -44,7 +44,8 @@ void validate_csr(const amgps_csr& A, const char* what, bool square);
 // validated square CSR)
 void require_positive_diagonal(const amgps_csr& A);
 // Warps per slice for the split kernels of a level (1: no split)
-int split_for(int64_t stored, int64_t nslices);
+// (f64: FP64 vectors)
+int split_for(int64_t stored, int64_t nslices, bool f64);
 // SELL-32 form of A; allow_uniform = false keeps every slice explicit
 HostSell build_sell(const amgps_csr& A, bool allow_uniform = true);
 // FP64 -> BF16 bits, round to nearest even directly from the double
