@@ -663,10 +663,6 @@ struct Engine {
       a.fam = a.init ? FAM_CHEB1SR : FAM_CHEB1S;
       a.c2 = a.c2 * a.rhoinv;
     }
-    // TMA option 1 (auto): only where the level has at least 4 tiles per SM
-    // (two per CTA for FP32 vectors, four per CTA for FP64); below that the
-    // persistent pipeline cannot fill and the direct kernel (more, smaller
-    // blocks) is faster.  Option 2 takes it wherever planned.
     if (auto* R = rec()) {  // the persistent kernel runs the direct form
       CyclePhase<VT, XT> p;
       p.op = CY_STEP;
@@ -687,8 +683,18 @@ struct Engine {
     launch_step<VT, XT>(a, s);
   }
 
+  // TMA option 1 (auto): only where the level has enough tiles per SM to fill
+  // the persistent pipeline; below that the direct kernel (more, smaller blocks,
+  // matrix data fetched under the previous kernel) is faster.  Option 2 takes it
+  // wherever planned.  Measured, four steps and the call, direct / TMA-fed us:
+  //   FP64, 22 tiles of 512 rows: 96^3 70.7 / 79.0, 112^3 (2744 tiles) 105.0 /
+  //     108.5, 128^3 (4096) 156.1 / 150.7, 192^3 532.6 / 453.3
+  //   FP32, 3 tiles of 1024 rows: 72^3 (364 tiles) 31.1 / 33.4, 84^3 (578) 41.7 /
+  //     40.0, 128^3 129.0 / 102.6; BF16 32.7 / 36.5, 43.1 / 40.3, 137.2 / 93.5
+  static constexpr int kTmaTilesPerSm = sizeof(XT) == 8 ? 22 : 3;
   static bool level_uses_tma(const amgps_ctx* c, const Level& L) {
-    return L.ntma > 0 && (c->use_tma == 2 || (c->use_tma == 1 && L.ntma >= 4 * c->nsm));
+    return L.ntma > 0 &&
+           (c->use_tma == 2 || (c->use_tma == 1 && L.ntma >= kTmaTilesPerSm * c->nsm));
   }
 
   // Whether this application on level L runs in the stored-operator form.
