@@ -265,8 +265,10 @@ amgps_status amgps_vcycle(amgps_ctx* ctx, const double* r_dev, double* z_dev);
 /* Preconditioned CG on A_0 x = b with one V-cycle as preconditioner, x_0 = 0,
  * stopping when ||r_k||_2 <= rtol ||b||_2 (recurrence residual) or after maxit
  * iterations.  *iters = products with A_0 performed, *relres = final
- * ||r_k||/||b||.  b_dev, x_dev: n_0 FP64 device vectors.  Synchronous (one
- * host read of ||r||^2 per iteration).  Returns AMGPS_E_NOCONV at maxit. */
+ * ||r_k||/||b||.  b_dev, x_dev: n_0 FP64 device vectors.  Synchronous (the
+ * iterations run as one CUDA graph with the loop on the device; with timed
+ * kernels, AMGPS_OPT_COARSE_KERNEL or a caller's preconditioner the host reads
+ * ||r||^2 every iteration).  Returns AMGPS_E_NOCONV at maxit. */
 amgps_status amgps_pcg(amgps_ctx* ctx, const double* b_dev, double* x_dev, double rtol,
                        int maxit, int* iters, double* relres);
 
@@ -309,7 +311,10 @@ amgps_status amgps_synchronize(amgps_ctx* ctx);
  * AMGPS_OPT_COARSE_SWEEPS (default 0): the coarsest level of the V-cycle is
  * solved with the dense FP64 inverse (0), or by m = 1..1000 l1-Jacobi sweeps
  * from zero, x <- x + M^{-1}(b - A_c x), the coarse solver of the paper's
- * experiments (Sec. 4 uses 30); the V-cycle stays symmetric either way.
+ * experiments (Sec. 4 uses 30); the V-cycle stays symmetric either way.  On
+ * FP64 hierarchies four or more sweeps run as one product with their matrix,
+ * formed when the option is set or a hierarchy is loaded (counted against
+ * AMGPS_OPT_ALLOC_LIMIT; without room the sweeps run one by one).
  * AMGPS_OPT_COARSE_KERNEL (default 0): 1 runs the levels below the last one
  * that runs the TMA-fed step, down to the coarsest, as one persistent kernel
  * (one co-resident grid with a bounded grid-wide barrier between dependent

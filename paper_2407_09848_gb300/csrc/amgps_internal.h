@@ -98,7 +98,8 @@ struct StepArgs {
   const int32_t* slices = nullptr;  // optional list of slices to process (null: all)
   int64_t nlist = 0;                // entries in `slices`
   int split = 1;  // > 1: one block of `split` warps per slice, entries split among them
-  // host hint for the scaled form: rin is still unscaled (b)
+  // rin is still unscaled (b): picks the family of a scaled recurrence step; a
+  // FAM_OPT step then multiplies it by 1/M
   bool rin_raw = false;
   // TMA-fed kernel: whether the next kernel's blocks may start while this one
   // runs.  Only another TMA-fed step gains by it: a kernel that works through

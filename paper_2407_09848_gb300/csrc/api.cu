@@ -722,14 +722,17 @@ struct Engine {
     XT* U[2] = {(XT*)L.zb, (XT*)L.xb};
     XT* t = (XT*)L.r;
     const bool profl = (l == 0);
-    if (!c_ready && !corrected) run_first(c, L, first_of(c, L, cf, x), b);
+    // (from a given x_0 the s_0 step forms c on the way)
+    if (xzero && !c_ready && !corrected) run_first(c, L, first_of(c, L, cf, x), b);
     const DevMat<VT> A = devmat<VT>(L);
     if (!xzero && !corrected) {
       StepArgs<VT, XT> a;
       a.A = A;
       a.A.val = (const VT*)L.sval;
       a.u = x;
-      a.rin = cv;
+      a.rin = c_ready ? cv : b;
+      a.rin_raw = !c_ready;
+      a.dinv = (const XT*)L.dinv;
       a.zout = cv;
       a.fam = FAM_OPT;
       a.write_r = k >= 3;

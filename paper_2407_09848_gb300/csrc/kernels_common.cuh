@@ -223,12 +223,14 @@ __device__ __forceinline__ constexpr bool step_needs_dinv() {
 }
 
 // Stored-operator steps: the vector terms the accumulation starts from
-// (s0 = slot-0 entry of the row, s1 = slot-1 entry), then the stores.
+// (s0 = slot-0 entry of the row, s1 = slot-1 entry), then the stores.  A
+// FAM_OPT step whose slot 0 is still the unscaled right-hand side (rin_raw)
+// scales it itself: c = M^{-1} b needs no pass of its own.
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
-__device__ __forceinline__ XT op_init(const StepArgs<VT, XT>& a, XT s0, XT s1) {
+__device__ __forceinline__ XT op_init(const StepArgs<VT, XT>& a, int64_t row, XT s0, XT s1) {
   XT acc = XT(0);
   if constexpr (FAM == FAM_OPT) {
-    acc = s0;
+    acc = a.rin_raw ? s0 * __ldg(a.dinv + row) : s0;
   } else {
     if constexpr (INIT) acc = WR ? s0 : a.c2 * s0;
     if constexpr (ZOWN) acc = INIT ? fma(a.c1, s1, acc) : a.c1 * s1;
@@ -308,7 +310,7 @@ __device__ __forceinline__ void step_slice(const StepArgs<VT, XT>& a, int64_t s,
             if (reads_slot1<FAM, ZOWN>()) s1 = ldv<CG>(a.xin + row);
             if (FAM == FAM_OPT && WR) uc = ldv<CG>(a.u + row);
           }
-          return op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, s0, s1);
+          return op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, live ? row : 0, s0, s1);
         },
         0, d.w);
     if (live) op_finish<VT, XT, FAM, WR>(a, row, acc, uc);
@@ -377,7 +379,7 @@ __device__ __forceinline__ void step_slice_mv(const StepArgs<VT, XT>& a, int64_t
       const XT* u = a.u + o;
 #pragma unroll
       for (int k = 0; k < 7; ++k) uv[k] = ldv<false>(u + cv[k]);
-      if constexpr (is_op(FAM)) t = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, rin, xin);
+      if constexpr (is_op(FAM)) t = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, lr, rin, xin);
       else t = step_init<FAM, StepForm<FAM, INIT>::kResidual>(rin, di);
 #pragma unroll
       for (int k = 0; k < 7; ++k) t = fma(kSign > 0 ? av[k] : -av[k], uv[k], t);

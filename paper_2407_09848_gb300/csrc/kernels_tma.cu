@@ -273,11 +273,11 @@ __global__ void __launch_bounds__((tma_warps<XT>() + 1) * 32, TmaShape<XT>::kCta
         const VT* v1 = reinterpret_cast<const VT*>(base) + (size_t)cs * p.w * kSlice + lane;
         const VT* v2 =
             reinterpret_cast<const VT*>(base) + (size_t)(two ? cs2 : cs) * p.w * kSlice + lane;
-        XT acc1 = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, c0 ? sv[r1] : XT(0),
+        XT acc1 = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, r0 + r1, c0 ? sv[r1] : XT(0),
                                                        c1 ? sv[p.rows + r1] : XT(0));
         XT uc1 = XT(0), uc2 = XT(0);
         if constexpr (W > 0) {
-          XT acc2 = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, c0 ? sv[r2] : XT(0),
+          XT acc2 = op_init<VT, XT, FAM, INIT, WR, ZOWN>(a, r0 + r2, c0 ? sv[r2] : XT(0),
                                                          c1 ? sv[p.rows + r2] : XT(0));
 #pragma unroll
           for (int k = 0; k < W; ++k) {
