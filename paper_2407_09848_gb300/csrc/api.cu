@@ -2021,7 +2021,7 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
 // B x n_0 is kept near kBatchRows: measured on the 32 vectors of a 64^3
 // problem, one pass (6 pre-cycles, loss and gradient) takes 43.2 ms one by one
 // and 17.8 ms in two batches of 16 (its FP64 multiply-adds alone: 10.6 ms); with
-// the later kernels 16.8 in two batches and 15.5 in one of 32 (0.95 GB).
+// the later kernels 16.8 in two batches, 14.5 in one of 32 (0.95 GB).
 // ---------------------------------------------------------------------------
 namespace {
 

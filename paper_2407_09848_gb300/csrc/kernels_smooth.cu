@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_step(const StepArgs<VT, XT> a) {
 // vectors, and the step is bound by FP64 issue alone.
 constexpr int kVecs = 4;
 template <class VT, class XT, int FAM, bool INIT, bool WR, bool ZOWN>
-__global__ void __launch_bounds__(kBlock, 3) k_step_mv(const StepArgs<VT, XT> a) {
+__global__ void __launch_bounds__(kBlock, 4) k_step_mv(const StepArgs<VT, XT> a) {
   const int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (s >= a.A.nslices) return;
   const int v0 = blockIdx.y * kVecs;
