@@ -299,22 +299,40 @@ def _csr_struct(A, keep):
     return CSR(A.shape[0], A.shape[1], A.nnz, rowptr.ctypes.data, col.ctypes.data, val.ctypes.data)
 
 
+class _BufOwner:
+    """Keeps the arrays of a library-allocated CSR until the last view of one is gone."""
+
+    def __init__(self, buf):
+        self._buf = buf
+        self._free = lib().amgps_csr_buf_free
+
+    def view(self, ptr, ctype, count):
+        if count == 0:
+            return np.zeros(0, dtype=ctype)
+        raw = (ctype * count).from_address(C.addressof(ptr.contents))
+        raw._owner = self  # the array's buffer holds `raw`, which holds this
+        return np.frombuffer(raw, dtype=ctype)
+
+    def __del__(self):
+        self._free(C.byref(self._buf))
+
+
 def _from_buf(b):
-    """Copy a library-allocated CSR into scipy and release it."""
+    """A library-allocated CSR as scipy CSR on the library's own arrays (no
+    copy; they are released with the last array that uses them)."""
     import scipy.sparse as sp
     n, nnz, ncol = b.n_rows, b.nnz, b.n_cols
-    try:
-        rp = np.ctypeslib.as_array(b.rowptr, shape=(n + 1,)).copy()
-        col = np.ctypeslib.as_array(b.col, shape=(max(nnz, 1),))[:nnz].copy()
-        val = np.ctypeslib.as_array(b.val, shape=(max(nnz, 1),))[:nnz].copy()
-    finally:
-        lib().amgps_csr_buf_free(C.byref(b))
-    return sp.csr_matrix((val, col, rp), shape=(n, ncol))
+    own = _BufOwner(b)
+    A = sp.csr_matrix((own.view(b.val, C.c_double, nnz), own.view(b.col, C.c_int32, nnz),
+                       own.view(b.rowptr, C.c_int32, n + 1)), shape=(n, ncol), copy=False)
+    A.has_sorted_indices = True  # the library's rows are sorted by column
+    return A
 
 
 def _sorted_csr(A):
     import scipy.sparse as sp
-    A = sp.csr_matrix(A)
+    if not (isinstance(A, sp.csr_matrix) and A.has_sorted_indices):
+        A = sp.csr_matrix(A)
     return A if A.has_sorted_indices else A.sorted_indices()
 
 

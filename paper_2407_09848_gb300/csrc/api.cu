@@ -299,8 +299,6 @@ struct amgps_ctx {
   bool loop_ok = false;        // built for the current smoothers and options
   bool loop_refused = false;   // the runtime would not build one: the host loop runs
   int64_t loop_kernels = 0;    // kernel nodes of the iteration
-  double** dx = nullptr;       // device slot: the solution vector of the running solve
-  void** hx = nullptr;         // pinned copy of the slot
   int use_tma = 1;             // AMGPS_OPT_TMA: TMA-fed step kernels 0 off, 1 auto, 2 always
   int flexible = 0;            // AMGPS_OPT_FLEXIBLE: 0 standard, 1 Polak-Ribiere, 2 one-reduction
   int coarse_sweeps = 0;       // AMGPS_OPT_COARSE_SWEEPS: 0 dense Cholesky, m l1-Jacobi sweeps
@@ -1810,7 +1808,7 @@ bool build_loop(amgps_ctx* c) {
     return e != cudaSuccess ? e : ee;
   };
   PcgLoop lp;
-  lp.x = c->dx;
+  lp.x = (double* const*)(c->dscal + S_X);
   cudaGraphNode_t begin = nullptr, loop = nullptr;
   size_t nb = 1;
   cudaError_t e = cudaGraphCreate(&g, 0);
@@ -1864,11 +1862,10 @@ void pcg_loop(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
     CK(cudaMemsetAsync(c->pz, 0, bytes, s));
   }
   if (c->flexible == 2) CK(cudaMemsetAsync(c->pq, 0, bytes, s));
-  *c->hx = x;
-  CK(cudaMemcpyAsync(c->dx, c->hx, sizeof(double*), cudaMemcpyHostToDevice, s));
   c->hscal[S_RTOL] = rtol;
   c->hscal[S_MAXIT] = maxit;
-  CK(cudaMemcpyAsync(c->dscal + S_RTOL, c->hscal + S_RTOL, 2 * sizeof(double),
+  std::memcpy(&c->hscal[S_X], &x, sizeof(x));
+  CK(cudaMemcpyAsync(c->dscal + S_RTOL, c->hscal + S_RTOL, 3 * sizeof(double),
                      cudaMemcpyHostToDevice, s));
   launch_dot(n, b, b, redwork(c, 0, n, kRedBlocksPerSm), c->dscal, S_BB, 0, s);
   with_engine(c, [&](auto eng) {  // what the r update does later
@@ -2307,8 +2304,6 @@ amgps_status amgps_create(amgps_ctx** out, int device, void* user_stream) {
     CK(cudaMalloc(&u->dscal, S_COUNT * sizeof(double)));
     CK(cudaMemset(u->dscal, 0, S_COUNT * sizeof(double)));
     CK(cudaMallocHost(&u->hscal, S_COUNT * sizeof(double)));
-    CK(cudaMalloc((void**)&u->dx, sizeof(double*)));
-    CK(cudaMallocHost((void**)&u->hx, sizeof(double*)));
     CK(cudaMalloc(&u->ddots, kDotSlots * sizeof(double)));
     CK(cudaMallocHost(&u->hdots, kDotSlots * sizeof(double)));
     const int maxgrid = u->nsm * kRedBlocksPerSm;
@@ -2335,8 +2330,6 @@ amgps_status amgps_destroy(amgps_ctx* c) {
   if (c->hscal) cudaFreeHost(c->hscal);
   if (c->hdots) cudaFreeHost(c->hdots);
   if (c->ddots) cudaFree(c->ddots);
-  if (c->dx) cudaFree(c->dx);
-  if (c->hx) cudaFreeHost(c->hx);
   if (c->dscal) cudaFree(c->dscal);
   if (c->part) cudaFree(c->part);
   if (c->counters) cudaFree(c->counters);
@@ -2483,7 +2476,7 @@ void load_levels(amgps_ctx* c, int n_levels, const amgps_csr* A, const amgps_csr
             const int64_t e = d.vbase + (int64_t)k * kSlice + ln;
             if (row < L.n) sv[e] = h.val[e] / m[row];
           }
-      });
+      }, kSlice);
       if (prec == AMGPS_F64) {
         L.sval = dupload(c, sv.data(), sv.size());
       } else {

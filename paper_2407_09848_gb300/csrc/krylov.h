@@ -15,6 +15,7 @@ enum Scalar {
   S_DELTA = 11,  // z . A z (one-reduction flexible CG)
   // the solve loop on the device (PcgLoop): iterations done, rtol, maxit
   S_IT = 12, S_RTOL = 13, S_MAXIT = 14,
+  S_X = 15,  // (a pointer) its solution vector
   S_COUNT = 16
 };
 

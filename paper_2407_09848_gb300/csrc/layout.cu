@@ -20,14 +20,15 @@ int64_t ceil_to(int64_t x, int64_t a) { return -floor_to(-x, a); }
 
 }  // namespace
 
-int parallel_threads(int64_t count) {
+int parallel_threads(int64_t count, int weight) {
   if (count < 4096) return 1;
-  const unsigned hw = std::thread::hardware_concurrency();
-  return (int)std::max(1u, std::min(hw == 0 ? 1u : hw, 32u));
+  const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
+  const int want = (int)std::lround(std::sqrt((double)count * weight / 8000.0));
+  return std::max(1, std::min({want, hw, 32}));
 }
 
-void parallel_for(int64_t count, const std::function<void(int64_t, int)>& f) {
-  const int nt = parallel_threads(count);
+void parallel_for(int64_t count, const std::function<void(int64_t, int)>& f, int weight) {
+  const int nt = parallel_threads(count, weight);
   if (nt == 1) {
     for (int64_t i = 0; i < count; ++i) f(i, 0);
     return;
@@ -57,10 +58,10 @@ void validate_csr(const amgps_csr& A, const char* what, bool square) {
   REQ(!square || A.n_rows == A.n_cols, AMGPS_E_ARG, w + ": not square");
   REQ(A.rowptr[0] == 0 && A.rowptr[A.n_rows] == A.nnz, AMGPS_E_ARG, w + ": bad rowptr ends");
   parallel_for(A.n_rows, [&](int64_t i, int) {
-    REQ(A.rowptr[i + 1] >= A.rowptr[i], AMGPS_E_ARG, w + ": rowptr not monotone");
-  });
-  // rowptr is monotone from 0 to nnz, so the rows cover every entry once
-  parallel_for(A.n_rows, [&](int64_t i, int) {
+    // (a row inside [0, nnz) may be read whatever the other rows say; monotone
+    // from 0 to nnz, the rows cover every entry once)
+    REQ(A.rowptr[i + 1] >= A.rowptr[i] && A.rowptr[i] >= 0 && A.rowptr[i + 1] <= A.nnz, AMGPS_E_ARG,
+        w + ": rowptr not monotone");
     for (int e = A.rowptr[i]; e < A.rowptr[i + 1]; ++e) {
       REQ(A.col[e] >= 0 && A.col[e] < A.n_cols, AMGPS_E_ARG, w + ": column index out of range");
       REQ(std::isfinite(A.val[e]), AMGPS_E_ARG, w + ": non-finite value");
@@ -139,7 +140,7 @@ HostSell build_sell(const amgps_csr& A, bool allow_uniform) {
         o.push_back((int32_t)((int64_t)A.col[e] - r));
     std::sort(o.begin(), o.end());
     o.erase(std::unique(o.begin(), o.end()), o.end());
-  });
+  }, kSlice);
   std::map<std::vector<int32_t>, int32_t> pats;
   const std::vector<int32_t>* prev = nullptr;
   int32_t prev_ref = -1;
@@ -180,7 +181,7 @@ HostSell build_sell(const amgps_csr& A, bool allow_uniform) {
   h.stored = vbase;
   h.val.assign(vbase, 0.0);
   if (h.any_explicit) h.col.assign(vbase, 0);
-  const int nt = parallel_threads(h.nslices);
+  const int nt = parallel_threads(h.nslices, kSlice);
   std::vector<std::vector<std::pair<int32_t, double>>> rowbufs(nt);
   std::vector<std::vector<uint8_t>> filleds(nt);
   parallel_for(h.nslices, [&](int64_t s, int t) {
@@ -215,7 +216,7 @@ HostSell build_sell(const amgps_csr& A, bool allow_uniform) {
           h.col[d.vbase + (int64_t)k * kSlice + lane] = (int32_t)std::min<int64_t>(r, A.n_cols - 1);
       }
     }
-  });
+  }, kSlice);
   return h;
 }
 

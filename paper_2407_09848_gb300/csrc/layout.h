@@ -32,11 +32,13 @@ struct HostPlan {
   std::vector<int32_t> gen;  // slices the TMA kernel does not cover
 };
 
-// Host threads for `count` independent items (1 below 4096 items, else the
-// hardware concurrency, at most 32); parallel_for calls f(i, thread) for
-// i in [0, count) in contiguous chunks and rethrows the first failure.
-int parallel_threads(int64_t count);
-void parallel_for(int64_t count, const std::function<void(int64_t, int)>& f);
+// Host threads for `count` independent items of about `weight` matrix rows each:
+// 1 below 4096 items, else about sqrt(work / cost of a thread) -- starting one
+// takes as long as looking through some 8000 rows -- at most the hardware
+// concurrency and 32; parallel_for calls f(i, thread) for i in [0, count) in
+// contiguous chunks and rethrows the first failure.
+int parallel_threads(int64_t count, int weight = 1);
+void parallel_for(int64_t count, const std::function<void(int64_t, int)>& f, int weight = 1);
 
 // AMGPS_E_ARG (through Fail) unless A is a well-formed CSR (square if asked)
 void validate_csr(const amgps_csr& A, const char* what, bool square);
