@@ -564,31 +564,37 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 }
 
 // Deterministic grid-wide sum: each block writes its partial, the last block to
-// arrive adds the partials in index order with a fixed tree and calls
-// fin(total) from thread 0, then re-arms the counter.  The grid size is a pure
-// function of the problem size, so the result is bitwise reproducible.
-template <class Fin>
-__device__ __forceinline__ void grid_sum(double v, const RedWork& w, Fin fin) {
+// arrive adds the partials in index order with a fixed tree and thread 0 calls
+// fin(total, pre()), with pre() -- the scalars fin needs -- loaded beside the
+// partials; then the counter is re-armed.  The grid size is a pure function of
+// the problem size, so the result is bitwise reproducible.  (The whole block
+// adds the partials: one warp alone, without block barriers, was slower, 32^3
+// solve 736 against 721 us.)
+template <class Pre, class Fin>
+__device__ __forceinline__ void grid_sum(double v, const RedWork& w, Pre pre, Fin fin) {
   __shared__ double sh[kBlock];
   __shared__ bool last;
-  double b = block_sum(v, sh);
+  const double b = block_sum(v, sh);
   if (threadIdx.x == 0) {
     w.part[blockIdx.x] = b;
     __threadfence();
-    const unsigned t = atomicAdd(w.counter, 1u);
-    last = (t == gridDim.x - 1);
+    last = atomicAdd(w.counter, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (last) {
-    __threadfence();
-    double s = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(w.part + i);
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) {
-      fin(s);
-      *w.counter = 0u;
-    }
+  if (!last) return;
+  __threadfence();
+  const auto pr = pre();
+  double s = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += kBlock) s += __ldcg(w.part + i);
+  s = block_sum(s, sh);
+  if (threadIdx.x == 0) {
+    fin(s, pr);
+    *w.counter = 0u;
   }
+}
+template <class Fin>
+__device__ __forceinline__ void grid_sum(double v, const RedWork& w, Fin fin) {
+  grid_sum(v, w, [] { return 0; }, [&](double s, int) { fin(s); });
 }
 
 // Threads per block of a kernel of `threads` one-row threads (or lanes): 256,

@@ -44,10 +44,12 @@ __global__ void __launch_bounds__(kBlock, 4) k_spmv_dot(const DevMat<double> A,
       acc = fma(ldv<false>(p + row), t, acc);
     }
   }
-  grid_sum(acc, w, [&](double tot) {
-    scal[S_PQ] = tot;
-    scal[S_ALPHA] = scal[S_RZ] / tot;  // once per iteration, not once per thread
-  });
+  grid_sum(
+      acc, w, [&] { return __ldcg(scal + S_RZ); },
+      [&](double tot, double rz) {
+        scal[S_PQ] = tot;
+        scal[S_ALPHA] = rz / tot;  // once per iteration, not once per thread
+      });
 }
 
 void launch_spmv_dot(const DevMat<double>& A, const double* p, double* q, const RedWork& w,
@@ -168,18 +170,30 @@ void launch_spmv_dot3(const DevMat<double>& A, const double* z, double* w, const
 }
 
 // Ends an iteration of a solve in a loop (thread 0 of the last block; rr is
-// its r.r): the tests of the host loop in api.cu, in the same order of
-// operations, so both take the same number of iterations.  The one-reduction
-// form (FCG) also needs a finite alpha.
+// its r.r, p the scalars): the tests of the host loop in api.cu, with the same
+// operations, so both take the same number of iterations.  Far from the
+// tolerance the square roots and the division (some 1.5 us of dependent FP64
+// instructions) are left out: rr > rtol^2 b.b with a margin no rounding spans.
+// The one-reduction form (FCG) also needs a finite alpha.
+struct LoopScalars {
+  double it, pq, err, bb, rtol, maxit, alpha;
+};
+__device__ __forceinline__ LoopScalars loop_scalars(const double* scal) {
+  return LoopScalars{__ldcg(scal + S_IT), __ldcg(scal + S_PQ),    __ldcg(scal + S_ERR),
+                     __ldcg(scal + S_BB), __ldcg(scal + S_RTOL),  __ldcg(scal + S_MAXIT),
+                     __ldcg(scal + S_ALPHA)};
+}
 template <bool FCG>
-__device__ __forceinline__ void pcg_continue(cudaGraphConditionalHandle h, double* scal, double rr) {
+__device__ __forceinline__ void pcg_continue(cudaGraphConditionalHandle h, double* scal, double rr,
+                                             const LoopScalars& p) {
   if (!h) return;
-  const double it = scal[S_IT] + 1.0, pq = scal[S_PQ];
+  const double it = p.it + 1.0;
   scal[S_IT] = it;
-  const bool ok = scal[S_ERR] == 0.0 && isfinite(pq) && isfinite(rr) && pq > 0.0 &&
-                  (!FCG || isfinite(scal[S_ALPHA]));
-  const bool more = !(sqrt(rr) / sqrt(scal[S_BB]) <= scal[S_RTOL]) && it < scal[S_MAXIT];
-  cudaGraphSetConditional(h, ok && more ? 1u : 0u);
+  const bool ok = p.err == 0.0 && isfinite(p.pq) && isfinite(rr) && p.pq > 0.0 &&
+                  (!FCG || isfinite(p.alpha));
+  bool above = rr > 1.0001 * (p.rtol * p.rtol) * p.bb;
+  if (!above) above = !(sqrt(rr) / sqrt(p.bb) <= p.rtol);
+  cudaGraphSetConditional(h, ok && above && it < p.maxit ? 1u : 0u);
 }
 
 __global__ void k_pcg_begin(double* scal, cudaGraphConditionalHandle h) {
@@ -220,10 +234,12 @@ __global__ void __launch_bounds__(kBlock) k_fcg_update(int64_t n, const double* 
     r[i] = ri;
     acc = fma(ri, ri, acc);
   }
-  grid_sum(acc, rw, [&](double tot) {
-    scal[S_RR] = tot;
-    pcg_continue<true>(loop.handle, scal, tot);
-  });
+  grid_sum(
+      acc, rw, [&] { return loop_scalars(scal); },
+      [&](double tot, const LoopScalars& ls) {
+        scal[S_RR] = tot;
+        pcg_continue<true>(loop.handle, scal, tot, ls);
+      });
 }
 
 void launch_fcg_update(int64_t n, const double* z, const double* w, double* p, double* q,
@@ -266,10 +282,12 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_r_update(int64_t n,
     one(i + step, q1, r1);
   }
   if (i < m) one(i, ldv<false>(q + i), ldv<false>(r + i));
-  grid_sum(acc, w, [&](double tot) {
-    scal[S_RR] = tot;
-    pcg_continue<false>(h, scal, tot);
-  });
+  grid_sum(
+      acc, w, [&] { return loop_scalars(scal); },
+      [&](double tot, const LoopScalars& ls) {
+        scal[S_RR] = tot;
+        pcg_continue<false>(h, scal, tot, ls);
+      });
 }
 
 template <class FT>
@@ -340,15 +358,20 @@ __global__ void __launch_bounds__(kBlock, kRedBlocksPerSm) k_dot(int64_t n, cons
     for (int k = 0; k < kLoads; ++k)
       if (i0 + k * step < n) acc = fma(av[k], (double)bv[k], acc);
   }
-  grid_sum(acc, w, [&](double tot) {
-    if (rz_shift) {
-      scal[S_RZOLD] = scal[S_RZ];
-      scal[S_RZ] = tot;
-      scal[S_BETA] = (rz_shift == 2 ? tot - scal[S_RZP] : tot) / scal[S_RZOLD];
-    } else {
-      scal[slot] = tot;
-    }
-  });
+  struct Old {
+    double rz, rzp;
+  };
+  grid_sum(
+      acc, w, [&] { return Old{__ldcg(scal + S_RZ), __ldcg(scal + S_RZP)}; },
+      [&](double tot, const Old& old) {
+        if (rz_shift) {
+          scal[S_RZOLD] = old.rz;
+          scal[S_RZ] = tot;
+          scal[S_BETA] = (rz_shift == 2 ? tot - old.rzp : tot) / old.rz;
+        } else {
+          scal[slot] = tot;
+        }
+      });
 }
 
 template <class BT>
