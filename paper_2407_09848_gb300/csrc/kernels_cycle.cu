@@ -154,7 +154,10 @@ __global__ void __launch_bounds__(kCycleThreads, kCycleMaxBlocksPerSm)
           coarse_gemv_row<XT, true>((int)i, (int)P.n, P.ainv, P.in0, P.out0, lane);
         break;
       case CY_CORRECT:
-        for (int64_t i = gt; i < P.n; i += nt) correct_row<true>(P.corr, i, 0);
+        for (int64_t i = gt; i < P.n; i += nt) {
+          if (P.corr.zout) correct_row<true, true>(P.corr, i, 0);
+          else correct_row<false, true>(P.corr, i, 0);
+        }
         break;
       default:  // CY_COPY
         for (int64_t i = gt; i < P.n; i += nt) P.out0[i] = __ldcg(P.in0 + i);

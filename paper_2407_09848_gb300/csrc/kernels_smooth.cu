@@ -452,15 +452,16 @@ void launch_l1diag(const DevMat<VT>& A, XT* dinv, cudaStream_t s) {
 // vectors out) where the prolongation and the step with the full row moved
 // 117; the gathered e is an eighth of the level and stays in L2.  256^3 solve
 // 93.8 -> 90.0 ms, one V-cycle on 61x53x47 101.6 -> 95.8 us.
+template <bool Z>
 __global__ void __launch_bounds__(kBlock) k_correct(const CorrArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < a.n) correct_row<false, true>(a, i, blockIdx.y);
+  if (i < a.n) correct_row<Z, false, true>(a, i, blockIdx.y);
 }
 
 void launch_correct(const CorrArgs& a, int nvec, cudaStream_t s) {
   if (a.n == 0) return;
   const int blk = small_block(a.n * nvec);
-  launch_dep(k_correct, dim3(blocks_of(a.n, blk), nvec), blk, 0, s, a);
+  launch_dep(a.zout ? k_correct<true> : k_correct<false>, dim3(blocks_of(a.n, blk), nvec), blk, 0, s, a);
 }
 
 // Set-up of M^{-1} A P, one row per lane of a slice: the row's entries are
