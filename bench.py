@@ -677,16 +677,19 @@ def run_ours(a):
         # nonzero for the products), averaged per launch.  In the
         # stored-operator form a k = 4 cycle's seven level-0 steps total
         # 14 nnz + 7 n (2 nnz + n per launch); the recurrence form's are
-        # 2 nnz + 5 n per launch.  Peak: 304 FP64 FMA thread-instructions per
+        # 2 nnz + 5 n per launch.  These are the plain steps of the method: the
+        # scaled steps and the first post-smoothing step (which runs with the
+        # coarse correction, four products a row) need up to a tenth fewer
+        # instructions than they count for.  Peak: 304 FP64 FMA thread-instructions per
         # clock (152 SMs x 2, ncu peak_sustained) x 2 flops x the SM clock
         # sampled during the profiled pass.
         fl = prof["step_flops"] / n_step
         mhz = clk_prof.get("sm_mhz") or 2070.0
         fpeak = 304 * 2 * mhz * 1e6 / 1e12
         fach = fl / (1e-3 * ms_step / n_step) / 1e12
-        # FP64 issue: thread instructions per launch (one per stored entry and
-        # per vector term) against 304 per clock; a lone multiply is one flop
-        # but a whole issue slot, so this is the pipe's utilisation
+        # FP64 issue: thread instructions of the plain steps (one per stored
+        # entry and per vector term) against 304 per clock; a lone multiply is
+        # one flop but a whole issue slot
         inst = prof["step_fp64_inst"] / n_step
         issue = inst / (1e-3 * ms_step / n_step) / (304 * mhz * 1e6)
         roof = {"bound": "alu", "achieved": fach, "peak": fpeak, "unit": "TFLOP/s",

@@ -7,7 +7,8 @@
 // one V-cycle (Eq. amg) and the outer PCG (Sec. 4).  The V-cycle below the
 // finest level is captured once into a CUDA graph and replayed, since those
 // levels are launch-bound; the finest level is launched eagerly so that its
-// kernels can be timed with plain CUDA events.
+// kernels can be timed with plain CUDA events.  A PCG solve whose kernels are
+// not being timed is one graph with the loop on the device (PcgLoop).
 #include <algorithm>
 #include <cstdlib>
 #include <chrono>
