@@ -288,7 +288,8 @@ struct amgps_ctx {
   double* dloss = nullptr;      // per error vector: <e0, A e0>, <e1, A e1>
   double* hdots = nullptr;
   bool bwd_ready = false;
-  int nvec = 1;                 // vectors the engine's kernels work on (> 1 inside a Batch)
+  int nvec = 1;                 // vectors the engine's kernels work on
+  bool batched = false;         // a Batch's buffers stand in the place of the levels' own
   double* part = nullptr;
   unsigned* counters = nullptr;
   int red_grid = 0;
@@ -1035,8 +1036,9 @@ struct Engine {
                            bool c_ready = false) {
     Level& L = c->lv[l];
     cudaStream_t s = c->stream;
-    if (!record && !rec() && c->nvec == 1 && c->tail_ok && l == c->tail_level && b == (const XT*)L.b &&
-        x == (XT*)L.x) {
+    // (the recorded phases and the captured graph work on the levels' own buffers)
+    if (!record && !rec() && !c->batched && c->tail_ok && l == c->tail_level &&
+        b == (const XT*)L.b && x == (XT*)L.x) {
       launch_tail(c);
       return;
     }
@@ -1048,7 +1050,7 @@ struct Engine {
     // stored-operator form: za = M^{-1} b afterwards, for the post-smoother
     const bool c_kept = smooth(c, l, cf, b, x, true, c_ready);
     Level& C = c->lv[l + 1];
-    const bool replay = l + 1 == 1 && c->nvec == 1 && c->graph_ok && !record && !capturing(c);
+    const bool replay = l + 1 == 1 && !c->batched && c->graph_ok && !record && !capturing(c);
     bool first_done = false;  // of the next level
     {
       // b_{l+1} = P^T (b - A x): the true residual (into the level's r buffer,
@@ -2095,6 +2097,7 @@ class Batch {
       return;
     }
     saved_ = c->lv;
+    c->batched = true;
     c->nvec = B;
     layout(c, B, bwd, (char*)base_);
   }
@@ -2105,13 +2108,14 @@ class Batch {
       L.b = S.b, L.x = S.x, L.r = S.r, L.za = S.za, L.zb = S.zb, L.xb = S.xb;
       L.bx2 = S.bx2, L.bgx = S.bgx, L.bgb = S.bgb, L.bt1 = S.bt1, L.bt2 = S.bt2, L.bt3 = S.bt3;
     }
+    c_->batched = false;
     c_->nvec = 1;
     cudaFreeAsync(base_, c_->stream);
   }
   Batch(const Batch&) = delete;
   Batch& operator=(const Batch&) = delete;
   bool ok() const { return base_ != nullptr; }
-  // a smaller last batch: the buffers keep their places
+  // a smaller last batch, of one vector perhaps: the buffers keep their places
   void size(int B) { c_->nvec = B; }
   double *r = nullptr, *z = nullptr, *e1 = nullptr, *dots = nullptr;
   RedWork rw;
