@@ -2026,6 +2026,8 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
 namespace {
 
 constexpr int64_t kBatchRows = int64_t(1) << 23;
+// the vectors of a batch are blocks in y
+constexpr int64_t kBatchVectors = 65535;
 
 // The batch buffers come from one stream-ordered pool per device, shared by
 // the contexts of the process (a training run holds hundreds of contexts and
@@ -2179,7 +2181,7 @@ int batch_size(amgps_ctx* c, int m, bool bwd) {
   if (cap != cudaStreamCaptureStatusNone) return 1;
   for (const Level& L : c->lv)
     if (L.xfer_general) return 1;
-  int64_t B = std::min<int64_t>(m, kBatchRows / c->lv[0].n);
+  int64_t B = std::min({(int64_t)m, kBatchRows / c->lv[0].n, kBatchVectors});
   if (B < 2) return 1;
   const int64_t parts = (m + B - 1) / B;  // of equal size
   B = (m + parts - 1) / parts;

@@ -1,6 +1,7 @@
 """Error cycles in several batches, the last of one vector: the graph of the
 coarse levels (and the persistent coarse kernel) that an earlier V-cycle has
-built belongs to the context's own buffers, not to a batch's."""
+built belongs to the context's own buffers, not to a batch's; and more vectors
+than a grid has blocks in y."""
 import pytest
 
 from paper_2407_09848_gb300 import problems as pr
@@ -65,4 +66,19 @@ def test_last_batch_of_one_vector(shape, coarse_kernel):
     n5 = _launches(S, lambda: S.error_cycles(E, 2))     # 2 + 2 + 1
     assert 2 * n5 == 3 * n4
     assert torch.equal(four, one[:4]) and torch.equal(E, one)
+    S.close()
+
+
+def test_more_vectors_than_blocks_in_y():
+    import torch
+    from paper_2407_09848_gb300.amgps import Solver
+    H = _hierarchy((3, 3, 3), 8)
+    S = Solver().load(H.A, H.P)
+    m = 70000
+    E = torch.from_numpy(pr.vec_normal(27, seed=1, count=m)).cuda()
+    parts = E.clone()
+    S.error_cycles(E, 1)
+    for i in range(0, m, 30000):
+        S.error_cycles(parts[i:i + 30000], 1)
+    assert torch.equal(E, parts)
     S.close()
