@@ -393,6 +393,11 @@ void drop_correct(amgps_ctx* c, Level& L) {
   L.corr = CorrMat{};
 }
 
+// After a change of smoothers, operators or options: the captured graphs and
+// the coarse kernel's recorded phases hold the old ones.  (The phases too: a
+// solve's graph captures the V-cycle without going through build_graph.)
+void drop_recorded(amgps_ctx* c) { c->graph_ok = c->loop_ok = c->tail_ok = false; }
+
 void free_hierarchy(amgps_ctx* c) {
   if (c->gexec) {
     cudaGraphExecDestroy(c->gexec);
@@ -402,8 +407,8 @@ void free_hierarchy(amgps_ctx* c) {
     cudaGraphExecDestroy(c->loop_exec);
     c->loop_exec = nullptr;
   }
-  c->graph_ok = c->loop_ok = c->loop_refused = false;
-  c->tail_ok = false;
+  drop_recorded(c);
+  c->loop_refused = false;
   if (!c->allocs.empty()) cudaStreamSynchronize(c->stream);
   for (void* p : c->allocs) cudaFree(p);
   c->allocs.clear();
@@ -1567,7 +1572,7 @@ bool prepare_ops(amgps_ctx* c) {
       if (attempt == 1) {  // the operators go before the coarse corrections
         CK(cudaStreamSynchronize(c->stream));
         for (auto& K : c->lv) drop_correct(c, K);
-        c->graph_ok = c->loop_ok = false;
+        drop_recorded(c);
       }
       try {
         while ((int)L.ops.size() < ns)
@@ -2581,9 +2586,9 @@ amgps_status amgps_set_smoother(amgps_ctx* c, int level, amgps_kind kind, int de
                 !std::equal(s.w, s.w + kMaxDegree, o.w);
       o = s;
     }
-    if (changed) c->graph_ok = c->loop_ok = false;
+    if (changed) drop_recorded(c);
     enter(c);
-    if (prepare_ops(c)) c->graph_ok = c->loop_ok = false;
+    if (prepare_ops(c)) drop_recorded(c);
     leave(c);
   });
 }
@@ -3005,7 +3010,7 @@ amgps_status amgps_set_option(amgps_ctx* c, int option, int64_t value) {
     if (option == AMGPS_OPT_STEP_FORM) {
       REQ(value == 0 || value == 1, AMGPS_E_ARG, "AMGPS_OPT_STEP_FORM takes 0 or 1");
       c->step_form = (int)value;
-      c->graph_ok = c->loop_ok = false;
+      drop_recorded(c);
       if (c->loaded) {
         enter(c);
         prepare_ops(c);
@@ -3014,7 +3019,7 @@ amgps_status amgps_set_option(amgps_ctx* c, int option, int64_t value) {
     } else if (option == AMGPS_OPT_TMA) {
       REQ(value >= 0 && value <= 2, AMGPS_E_ARG, "AMGPS_OPT_TMA takes 0, 1 or 2");
       c->use_tma = (int)value;
-      c->graph_ok = c->loop_ok = false;
+      drop_recorded(c);
     } else if (option == AMGPS_OPT_FLEXIBLE) {
       REQ(value >= 0 && value <= 2, AMGPS_E_ARG, "AMGPS_OPT_FLEXIBLE takes 0, 1 or 2");
       c->flexible = (int)value;
@@ -3025,7 +3030,7 @@ amgps_status amgps_set_option(amgps_ctx* c, int option, int64_t value) {
     } else if (option == AMGPS_OPT_COARSE_KERNEL) {
       REQ(value == 0 || value == 1, AMGPS_E_ARG, "AMGPS_OPT_COARSE_KERNEL takes 0 or 1");
       c->use_cycle = (int)value;
-      c->graph_ok = c->loop_ok = false;
+      drop_recorded(c);
     } else {
       REQ(value >= 0 && value <= 1000, AMGPS_E_ARG, "AMGPS_OPT_COARSE_SWEEPS takes 0..1000");
       c->coarse_sweeps = (int)value;
@@ -3034,7 +3039,7 @@ amgps_status amgps_set_option(amgps_ctx* c, int option, int64_t value) {
         prepare_coarse(c);
         leave(c);
       }
-      c->graph_ok = c->loop_ok = false;  // the coarse-level graph holds the coarse solve
+      drop_recorded(c);  // the coarse-level graph holds the coarse solve
     }
   });
 }

@@ -1,0 +1,32 @@
+"""The solve loop on the device after the context's state has changed."""
+import pytest
+
+from paper_2407_09848_gb300 import problems as pr
+
+pytestmark = pytest.mark.gpu
+
+
+def _solver(shape, coarse_max=64):
+    from paper_2407_09848_gb300.amgps import Solver
+    H = pr.build_hierarchy(pr.varcoef(shape[0], 1.0, 4.0, seed=4, ny=shape[1], nz=shape[2]),
+                           coarse_max)
+    return Solver().load(H.A, H.P), H.A[0].shape[0]
+
+
+def test_solve_after_the_coarse_kernel_was_switched_off():
+    """The phases that the coarse kernel recorded for the old weights are not used again."""
+    import torch
+    out = []
+    for recorded in (True, False):
+        S, n = _solver((31, 26, 22))
+        assert S.n_levels >= 3
+        b = torch.from_numpy(pr.rhs_uniform(n, seed=1)).cuda()
+        x, z = torch.empty_like(b), torch.empty_like(b)
+        if recorded:
+            S.set_coarse_kernel(True)
+            S.vcycle(b, z)
+            S.set_coarse_kernel(False)
+        S.set_smoother(-1, "l1jacobi", 1)
+        out.append((S.pcg(b, x, rtol=1e-8), x))
+        S.close()
+    assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1])
