@@ -173,7 +173,8 @@ void launch_spmv_dot3(const DevMat<double>& A, const double* z, double* w, const
 // its r.r, p the scalars): the tests of the host loop in api.cu, with the same
 // operations, so both take the same number of iterations.  Far from the
 // tolerance the square roots and the division (some 1.5 us of dependent FP64
-// instructions) are left out: rr > rtol^2 b.b with a margin no rounding spans.
+// instructions) are left out: rr > rtol^2 b.b with a margin no rounding spans
+// while rtol^2 is a normal number (below, it loses bits or is 0).
 // The one-reduction form (FCG) also needs a finite alpha.
 struct LoopScalars {
   double it, pq, err, bb, rtol, maxit, alpha;
@@ -191,7 +192,7 @@ __device__ __forceinline__ void pcg_continue(cudaGraphConditionalHandle h, doubl
   scal[S_IT] = it;
   const bool ok = p.err == 0.0 && isfinite(p.pq) && isfinite(rr) && p.pq > 0.0 &&
                   (!FCG || isfinite(p.alpha));
-  bool above = rr > 1.0001 * (p.rtol * p.rtol) * p.bb;
+  bool above = p.rtol >= 1e-150 && rr > 1.0001 * (p.rtol * p.rtol) * p.bb;
   if (!above) above = !(sqrt(rr) / sqrt(p.bb) <= p.rtol);
   cudaGraphSetConditional(h, ok && above && it < p.maxit ? 1u : 0u);
 }

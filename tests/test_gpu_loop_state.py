@@ -1,4 +1,5 @@
-"""The solve loop on the device after the context's state has changed."""
+"""The solve loop on the device after the context's state has changed, and at
+tolerances whose square is not a normal number."""
 import pytest
 
 from paper_2407_09848_gb300 import problems as pr
@@ -30,3 +31,19 @@ def test_solve_after_the_coarse_kernel_was_switched_off():
         out.append((S.pcg(b, x, rtol=1e-8), x))
         S.close()
     assert out[0][0] == out[1][0] and torch.equal(out[0][1], out[1][1])
+
+
+# squares: 1e-320 and 1e-324 are not normal (the latter rounds to 0), 1e-300 is
+@pytest.mark.parametrize("rtol", [1e-150, 1e-160, 1e-162])
+@pytest.mark.parametrize("outer", ["cg", "flexible", "fcg1"])
+def test_tolerances_whose_square_underflows(rtol, outer):
+    import torch
+    S, n = _solver((19, 17, 13), 512)
+    S.set_flexible(outer)
+    b = torch.from_numpy(pr.rhs_uniform(n, seed=1) * 1e100).cuda()
+    x, y = torch.empty_like(b), torch.empty_like(b)
+    got = S.pcg(b, x, rtol=rtol, maxit=600, raise_on_noconv=False)
+    S.profile(True)  # the host loop
+    ref = S.pcg(b, y, rtol=rtol, maxit=600, raise_on_noconv=False)
+    assert got == ref and torch.equal(x, y)
+    S.close()
