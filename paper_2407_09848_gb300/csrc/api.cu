@@ -1487,12 +1487,18 @@ void check_kind_degree(int kind, int degree) {
 }
 
 // Levels that take the stored-operator form: FP64 values with the row-scaled
-// copy, one warp per slice, and at least kOpMinRows rows (whichever step
-// kernel runs them; the smaller levels are launch-bound, and their operators
-// would only take memory).
+// copy, at least kOpMinRows rows (whichever step kernel runs them; the smaller
+// levels are launch-bound, and their operators would only take memory), and
+// rows that split_for's rule for FP32 leaves to one warp a slice: under 24
+// entries on average, or wider on the largest levels.  (The FP64 rule splits
+// fewer levels, but a row of 170 entries saves two or three instructions by its
+// operators, which are three more copies of the matrix.  256^3 smoothed
+// aggregation, level 2 of 262,144 rows of 169 entries: with operators 1.08 GB
+// more and 53.88 ms a solve, without 53.91.)
 constexpr int64_t kOpMinRows = 1 << 17;
 bool op_level(const amgps_ctx* c, const Level& L) {
-  return c->prec == AMGPS_F64 && L.sval && !L.coarsest && L.split == 1 && L.n >= kOpMinRows;
+  return c->prec == AMGPS_F64 && L.sval && !L.coarsest && L.split == 1 &&
+         split_for(L.stored, L.nslices, false) == 1 && L.n >= kOpMinRows;
 }
 
 // M^{-1} A P of every FP64 aggregation level with rows of at most eight stored
