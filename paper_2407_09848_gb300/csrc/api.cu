@@ -319,6 +319,9 @@ struct amgps_ctx {
   void* noalloc = nullptr;        // device address of the allocation-free scratch array
   size_t alloc_limit = 0;         // AMGPS_OPT_ALLOC_LIMIT: hierarchy bytes allowed (0: no limit)
   size_t alloc_bytes = 0;         // hierarchy bytes allocated
+  // the caller has captured a call on this hierarchy: a graph of the caller's may
+  // read any of its arrays from now on, so none is given back or formed anew in place
+  bool captured = false;
   // persistent kernel for the coarse levels (option AMGPS_OPT_COARSE_KERNEL)
   int use_cycle = 0;
   bool tail_ok = false;
@@ -383,7 +386,7 @@ T* dupload(amgps_ctx* c, const T* h, size_t count) {
 }
 
 // Gives the arrays of a level's coarse correction back (no kernel that uses
-// them may be enqueued; a captured graph that does is stale afterwards).
+// them may be enqueued, and no graph of the caller's hold one).
 void drop_correct(amgps_ctx* c, Level& L) {
   if (!L.corr_mem) return;
   c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), L.corr_mem));
@@ -408,7 +411,7 @@ void free_hierarchy(amgps_ctx* c) {
     c->loop_exec = nullptr;
   }
   drop_recorded(c);
-  c->loop_refused = false;
+  c->loop_refused = c->captured = false;
   if (!c->allocs.empty()) cudaStreamSynchronize(c->stream);
   for (void* p : c->allocs) cudaFree(p);
   c->allocs.clear();
@@ -424,6 +427,9 @@ void enter(amgps_ctx* c) {
   CK(cudaSetDevice(c->device));
   CK(cudaEventRecord(c->ev_in, c->ustream));
   CK(cudaStreamWaitEvent(c->stream, c->ev_in, 0));
+  cudaStreamCaptureStatus cap;
+  CK(cudaStreamIsCapturing(c->stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) c->captured = true;
 }
 
 void leave(amgps_ctx* c) {
@@ -1576,6 +1582,7 @@ bool prepare_ops(amgps_ctx* c) {
     bool fits = false;
     for (int attempt = 0; attempt < 2 && !fits; ++attempt) {
       if (attempt == 1) {  // the operators go before the coarse corrections
+        if (c->captured) break;
         CK(cudaStreamSynchronize(c->stream));
         for (auto& K : c->lv) drop_correct(c, K);
         drop_recorded(c);
@@ -1615,7 +1622,7 @@ constexpr int kSweepMin = 4;
 void prepare_coarse(amgps_ctx* c) {
   Level& L = c->lv.back();
   const int m = c->coarse_sweeps;
-  if (L.qsweeps == m) return;
+  if (L.qsweeps == m || (L.qsweeps != 0 && c->captured)) return;
   L.qsweeps = 0;
   if (c->prec != AMGPS_F64 || m < kSweepMin || (double)m * L.n * L.stored > kSweepWork) return;
   if (Engine<double, double>::capturing(c)) return;
