@@ -234,6 +234,7 @@ struct Level {
   CorrMat corr;
   void* corr_mem = nullptr;
   size_t corr_bytes = 0;
+  bool corr_given = false;  // given back for something else's sake
   int wmax = 0;  // stored entries of the widest slice
   int split = 1;  // warps per slice of the generic step kernel (wide rows)
   void* dinv = nullptr;   // 1 / M_i
@@ -385,13 +386,17 @@ T* dupload(amgps_ctx* c, const T* h, size_t count) {
   return d;
 }
 
+void dfree(amgps_ctx* c, void* p, size_t bytes) {
+  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
+  cudaFree(p);
+  c->alloc_bytes -= bytes;
+}
+
 // Gives the arrays of a level's coarse correction back (no kernel that uses
 // them may be enqueued, and no graph of the caller's hold one).
 void drop_correct(amgps_ctx* c, Level& L) {
   if (!L.corr_mem) return;
-  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), L.corr_mem));
-  cudaFree(L.corr_mem);
-  c->alloc_bytes -= L.corr_bytes;
+  dfree(c, L.corr_mem, L.corr_bytes);
   L.corr_mem = nullptr;
   L.corr = CorrMat{};
 }
@@ -400,6 +405,33 @@ void drop_correct(amgps_ctx* c, Level& L) {
 // the coarse kernel's recorded phases hold the old ones.  (The phases too: a
 // solve's graph captures the V-cycle without going through build_graph.)
 void drop_recorded(amgps_ctx* c) { c->graph_ok = c->loop_ok = c->tail_ok = false; }
+
+// After an allocation has failed: room for `count` arrays of `bytes` together,
+// by giving coarse corrections back, the coarsest level's first.  False, and
+// nothing given back, where all of them would not be enough.
+bool make_room(amgps_ctx* c, size_t bytes, size_t count) {
+  cudaStreamCaptureStatus cap;
+  CK(cudaStreamIsCapturing(c->stream, &cap));
+  if (c->captured || cap != cudaStreamCaptureStatusNone) return false;
+  constexpr size_t kGrain = size_t(2) << 20;  // what the device hands out
+  auto fits = [&](size_t more) {
+    size_t dev = 0, total = 0;
+    CK(cudaMemGetInfo(&dev, &total));
+    if (c->alloc_limit && c->alloc_bytes + bytes > c->alloc_limit + more) return false;
+    return bytes + count * kGrain <= dev + more;
+  };
+  size_t all = 0;
+  for (const Level& L : c->lv) all += L.corr_bytes * (L.corr_mem != nullptr);
+  if (!fits(all)) return false;
+  CK(cudaStreamSynchronize(c->stream));
+  for (size_t l = c->lv.size(); l-- > 0 && !fits(0);) {
+    if (!c->lv[l].corr_mem) continue;
+    drop_correct(c, c->lv[l]);
+    c->lv[l].corr_given = true;
+    drop_recorded(c);
+  }
+  return true;
+}
 
 void free_hierarchy(amgps_ctx* c) {
   if (c->gexec) {
@@ -1511,8 +1543,9 @@ bool op_level(const amgps_ctx* c, const Level& L) {
 // entries, for the coarse correction (36 B a row).  A level whose arrays do not
 // fit the device or the allocation limit, or with a row that touches more than
 // four aggregates, keeps the prolongation and the full first step.
-void prepare_correct(amgps_ctx* c) {
-  if (c->prec != AMGPS_F64) return;
+// again: only the levels that have given theirs back.  True if any was built.
+bool prepare_correct(amgps_ctx* c, bool again = false) {
+  if (c->prec != AMGPS_F64) return false;
   struct Try {
     Level* L;
     int* bad;
@@ -1523,7 +1556,7 @@ void prepare_correct(amgps_ctx* c) {
   std::fill(table, table + kCorrTable, kCorrEmpty);
   table[0] = 0;
   for (auto& L : c->lv) {
-    if (L.coarsest || L.xfer_general || L.wmax > 8) continue;
+    if (L.coarsest || L.xfer_general || L.wmax > 8 || L.corr_mem || (again && !L.corr_given)) continue;
     const size_t vb = (size_t)L.nslices * kSlice * kCorrEntries * sizeof(double);
     const size_t cb = ((size_t)L.n * sizeof(uint32_t) + 255) / 256 * 256;
     const size_t tb = kCorrTable * sizeof(int32_t);
@@ -1549,7 +1582,9 @@ void prepare_correct(amgps_ctx* c) {
                          (int32_t*)(base + vb + cb), bad, c->stream);
     check_launch();
     built.push_back({&L, bad, m});
+    L.corr_given = false;
   }
+  if (built.empty()) return false;
   std::vector<int> flags(built.size(), 0);
   for (size_t i = 0; i < built.size(); ++i)
     CK(cudaMemcpyAsync(&flags[i], built[i].bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -1558,6 +1593,20 @@ void prepare_correct(amgps_ctx* c) {
     if (flags[i] == 0) built[i].L->corr = built[i].m;
     else drop_correct(c, *built[i].L);
   }
+  return true;
+}
+
+// Corrections that were given back return where there is room again: operator
+// arrays that the level's present smoother does not use make some.
+bool restore_correct(amgps_ctx* c) {
+  bool any = false;
+  for (const Level& L : c->lv) any = any || L.corr_given;
+  if (!any || c->captured || Engine<double, double>::capturing(c)) return false;
+  CK(cudaStreamSynchronize(c->stream));
+  for (Level& L : c->lv)
+    for (size_t used = L.ops_ok ? L.ops_cf.k - 1 : 0; L.ops.size() > used; L.ops.pop_back())
+      dfree(c, L.ops.back(), (size_t)L.stored * sizeof(double));
+  return prepare_correct(c, true);
 }
 
 // Builds, on the library stream, the stored operators of every such level
@@ -1579,17 +1628,12 @@ bool prepare_ops(amgps_ctx* c) {
     if (c->step_form != 1 || cap != cudaStreamCaptureStatusNone || !op_level(c, L)) continue;
     if (cf.k < 2) continue;
     const int ns = cf.k - 1;
-    bool fits = false;
+    bool fits = false;  // the operators go before the coarse corrections
     for (int attempt = 0; attempt < 2 && !fits; ++attempt) {
-      if (attempt == 1) {  // the operators go before the coarse corrections
-        if (c->captured) break;
-        CK(cudaStreamSynchronize(c->stream));
-        for (auto& K : c->lv) drop_correct(c, K);
-        drop_recorded(c);
-      }
+      const size_t one = (size_t)L.stored * sizeof(double), left = ns - std::min<size_t>(ns, L.ops.size());
+      if (attempt == 1 && !make_room(c, left * one, left)) break;
       try {
-        while ((int)L.ops.size() < ns)
-          L.ops.push_back((double*)dalloc(c, (size_t)L.stored * sizeof(double)));
+        while ((int)L.ops.size() < ns) L.ops.push_back((double*)dalloc(c, one));
         fits = true;
       } catch (const Fail& f) {
         if (f.st != AMGPS_E_NOMEM) throw;
@@ -1605,7 +1649,7 @@ bool prepare_ops(amgps_ctx* c) {
     L.ops_cf = cf;
     L.ops_ok = built = true;
   }
-  return built;
+  return restore_correct(c) || built;
 }
 
 // m l1-Jacobi sweeps from zero on the coarsest level are one fixed symmetric

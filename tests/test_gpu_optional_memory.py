@@ -43,6 +43,45 @@ def _reverse_bytes(H):
     return 8 * (6 * sum(n[:-1]) + 2 * n[-1]) + 8 * (32 * 32 + 2 * 4096) + 4096
 
 
+def test_corrections_stay_when_they_would_not_make_enough_room():
+    """Operators of degree 8 do not fit even without the corrections: those are kept."""
+    import torch
+    H = _hierarchy((57, 51, 48))
+    n = H.A[0].shape[0]
+    r = torch.from_numpy(pr.rhs_uniform(n, seed=1)).cuda()
+    z = [torch.empty_like(r) for _ in range(2)]
+    S = _solver(H)
+    S.vcycle(r, z[0])
+    S.set_alloc_limit(1)
+    S.set_smoother(0, "cheb4_opt", 8)
+    S.set_smoother(0, "cheb4_opt", 4)
+    S.vcycle(r, z[1])
+    assert torch.equal(z[0], z[1])
+    S.close()
+
+
+def test_corrections_come_back_with_a_smaller_degree():
+    import torch
+    H = _hierarchy((57, 51, 48))
+    n = H.A[0].shape[0]
+    r = torch.from_numpy(pr.rhs_uniform(n, seed=1)).cuda()
+    z = [torch.empty_like(r) for _ in range(3)]
+    S = _solver(H)
+    stored = S.level_info(0)[2]
+    S.set_smoother(0, "cheb4_opt", 2)
+    S.vcycle(r, z[0])
+    S.close()
+    # three operators at load (degree 4) and the corrections (36 B a row); one more
+    # operator (56 B a row) fits only without level 0's correction
+    S = _solver(H, _least(H) + 3 * 8 * stored + 60 * n)
+    S.set_smoother(0, "cheb4_opt", 5)
+    S.vcycle(r, z[1])
+    S.set_smoother(0, "cheb4_opt", 2)
+    S.vcycle(r, z[2])
+    assert torch.equal(z[0], z[2]) and not torch.equal(z[0], z[1])
+    S.close()
+
+
 @pytest.mark.parametrize("what", ["operators", "reverse", "sweeps"])
 def test_a_captured_cycle_keeps_its_arrays(what):
     """The caller's graph gives the same bits after a call that would like their place."""
