@@ -407,8 +407,9 @@ void drop_correct(amgps_ctx* c, Level& L) {
 void drop_recorded(amgps_ctx* c) { c->graph_ok = c->loop_ok = c->tail_ok = false; }
 
 // After an allocation has failed: room for `count` arrays of `bytes` together,
-// by giving coarse corrections back, the coarsest level's first.  False, and
-// nothing given back, where all of them would not be enough.
+// by giving back what only makes a hierarchy faster: coarse corrections, the
+// coarsest level's first, then the matrix of the coarse sweeps.  False, and
+// nothing given back, where all of it would not be enough.
 bool make_room(amgps_ctx* c, size_t bytes, size_t count) {
   cudaStreamCaptureStatus cap;
   CK(cudaStreamIsCapturing(c->stream, &cap));
@@ -422,7 +423,9 @@ bool make_room(amgps_ctx* c, size_t bytes, size_t count) {
   };
   size_t all = 0;
   for (const Level& L : c->lv) all += L.corr_bytes * (L.corr_mem != nullptr);
-  if (!fits(all)) return false;
+  Level& C = c->lv.back();
+  const size_t q = (size_t)C.n * C.n * sizeof(double) * (C.qinv != nullptr);
+  if (!fits(all + q)) return false;
   CK(cudaStreamSynchronize(c->stream));
   for (size_t l = c->lv.size(); l-- > 0 && !fits(0);) {
     if (!c->lv[l].corr_mem) continue;
@@ -430,7 +433,33 @@ bool make_room(amgps_ctx* c, size_t bytes, size_t count) {
     c->lv[l].corr_given = true;
     drop_recorded(c);
   }
+  if (C.qinv && !fits(0)) {
+    dfree(c, C.qinv, q);
+    C.qinv = nullptr;
+    C.qsweeps = 0;
+    drop_recorded(c);
+  }
   return true;
+}
+
+// Allocates every array of `want` that is not there yet.
+struct Want {
+  void** p;
+  size_t bytes;
+};
+void dalloc_all(amgps_ctx* c, const std::vector<Want>& want) {
+  for (int attempt = 0;; ++attempt) {
+    try {
+      for (const Want& w : want)
+        if (!*w.p) *w.p = dalloc(c, w.bytes);
+      return;
+    } catch (const Fail& f) {
+      size_t bytes = 0, count = 0;
+      for (const Want& w : want)
+        if (!*w.p) bytes += w.bytes, ++count;
+      if (f.st != AMGPS_E_NOMEM || attempt == 1 || !make_room(c, bytes, count)) throw;
+    }
+  }
 }
 
 void free_hierarchy(amgps_ctx* c) {
@@ -1299,22 +1328,20 @@ struct Engine {
   }
 
   static void ensure_loss(amgps_ctx* c) {
-    if (!c->dacc) c->dacc = (double*)dalloc(c, kDotSlots * sizeof(double));
-    if (!c->dloss) c->dloss = (double*)dalloc(c, 2 * kMaxLossVectors * sizeof(double));
+    dalloc_all(c, {{(void**)&c->dacc, kDotSlots * sizeof(double)},
+                   {(void**)&c->dloss, 2 * kMaxLossVectors * sizeof(double)}});
   }
 
   static void ensure_bwd(amgps_ctx* c) {
     if (c->bwd_ready) return;
+    std::vector<Want> want;
     for (auto& L : c->lv) {
       const size_t bytes = L.n * sizeof(XT);
-      L.bgx = dalloc(c, bytes);
-      L.bgb = dalloc(c, bytes);
+      for (void** p : {&L.bgx, &L.bgb}) want.push_back({p, bytes});
       if (L.coarsest) continue;
-      L.bx2 = dalloc(c, bytes);
-      L.bt1 = dalloc(c, bytes);
-      L.bt2 = dalloc(c, bytes);
-      L.bt3 = dalloc(c, bytes);
+      for (void** p : {&L.bx2, &L.bt1, &L.bt2, &L.bt3}) want.push_back({p, bytes});
     }
+    dalloc_all(c, want);
     c->bwd_ready = true;
   }
 

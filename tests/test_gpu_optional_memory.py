@@ -43,6 +43,39 @@ def _reverse_bytes(H):
     return 8 * (6 * sum(n[:-1]) + 2 * n[-1]) + 8 * (32 * 32 + 2 * 4096) + 4096
 
 
+@pytest.mark.parametrize("sweeps", [0, 30])
+@pytest.mark.parametrize("call", ["loss", "smooth", "vcycle"])
+def test_reverse_mode_fits_where_the_load_and_its_buffers_do(call, sweeps):
+    import torch
+    H = _hierarchy((31, 26, 22))
+    n = H.A[0].shape[0]
+    limit = _least(H) + _reverse_bytes(H)
+    r, g = (torch.from_numpy(pr.rhs_uniform(n, seed=i)).cuda() for i in (1, 2))
+    E = torch.from_numpy(pr.vec_normal(n, seed=1, count=3)).cuda()
+    z = torch.empty_like(r)
+
+    def run(S):
+        S.vcycle(r, z)  # builds the graphs, with whatever is optional
+        if call == "loss":
+            out = S.loss_grad(E)
+        elif call == "smooth":
+            gb, gx, gw = S.smooth_backward(0, "cheb4_opt", 4, r, None, g)
+            out = (gb.cpu().numpy(), gw)
+        else:
+            gr, gw = S.vcycle_backward(r, g)
+            out = (gr.cpu().numpy(), gw)
+        S.vcycle(r, z)
+        x = torch.empty_like(r)
+        it = S.pcg(r, x)[0]
+        S.close()
+        return [np.asarray(o) for o in out] + [z.cpu().numpy(), x.cpu().numpy(), it]
+    lim, free = run(_solver(H, limit, sweeps)), run(_solver(H, 0, sweeps))
+    assert lim[-1] == free[-1]
+    for a, b in zip(lim[:-1], free[:-1]):
+        # the correction in another form, sums over vectors in another order
+        assert np.linalg.norm(a - b) <= 1e-11 * np.linalg.norm(b)
+
+
 def test_corrections_stay_when_they_would_not_make_enough_room():
     """Operators of degree 8 do not fit even without the corrections: those are kept."""
     import torch
