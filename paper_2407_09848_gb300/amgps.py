@@ -323,16 +323,16 @@ def _from_buf(b):
     import scipy.sparse as sp
     n, nnz, ncol = b.n_rows, b.nnz, b.n_cols
     own = _BufOwner(b)
-    A = sp.csr_matrix((own.view(b.val, C.c_double, nnz), own.view(b.col, C.c_int32, nnz),
-                       own.view(b.rowptr, C.c_int32, n + 1)), shape=(n, ncol), copy=False)
-    A.has_sorted_indices = True  # the library's rows are sorted by column
-    return A
+    # (scipy's flag of sorted rows is left unset: it would outlive a renumbering in place)
+    return sp.csr_matrix((own.view(b.val, C.c_double, nnz), own.view(b.col, C.c_int32, nnz),
+                          own.view(b.rowptr, C.c_int32, n + 1)), shape=(n, ncol), copy=False)
 
 
 def _sorted_csr(A):
+    """A with sorted rows, looked at here: a flag that scipy keeps on the
+    caller's object may be older than its arrays."""
     import scipy.sparse as sp
-    if not (isinstance(A, sp.csr_matrix) and A.has_sorted_indices):
-        A = sp.csr_matrix(A)
+    A = sp.csr_matrix(A)
     return A if A.has_sorted_indices else A.sorted_indices()
 
 
@@ -397,8 +397,11 @@ class Solver:
     def sa_level(self, A, agg, n_coarse):
         """Smoothed-aggregation level on the device (amgps_sa_level):
         returns (P, A_c, omega) with P, A_c scipy CSR."""
+        return self._sa_level(_sorted_csr(A), agg, n_coarse)
+
+    def _sa_level(self, A, agg, n_coarse):
         keep = []
-        a = _csr_struct(_sorted_csr(A), keep)
+        a = _csr_struct(A, keep)
         g = np.ascontiguousarray(agg, dtype=np.int32)
         if g.size != a.n_rows:
             raise ValueError("agg needs one entry per row of A")
@@ -413,8 +416,8 @@ class Solver:
         aggregate maps [(agg, n_coarse, ...), ...] of each level; returns
         (A_list, P_list, omegas) ready for load()."""
         As, Ps, oms = [_sorted_csr(A0)], [], []
-        for lv in levels:
-            P, Ac, om = self.sa_level(As[-1], lv[0], lv[1])
+        for lv in levels:  # (the library's rows come sorted)
+            P, Ac, om = self._sa_level(As[-1], lv[0], lv[1])
             Ps.append(P)
             As.append(Ac)
             oms.append(om)
