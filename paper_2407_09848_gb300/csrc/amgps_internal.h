@@ -247,6 +247,13 @@ void launch_restrict(const RestrictArgs<VT, XT>& a, int nvec, cudaStream_t s);
 // Levels of at most this many rows take it: there the three kernels are mostly
 // latency; on larger ones the children's rows are better read coalesced.
 constexpr int64_t kFuseRows = 1 << 16;
+// And with at most this many children a coarse row, two rounds of its eight
+// lanes: each further round is one more chain of dependent loads, on fewer lanes
+// than the level has rows.  V-cycle on two levels, separate / fused us, FP64: 8
+// children (12^3) 29.4 / 29.0, 16 (20^3) 32.4 / 31.8, 24 (24^3) 35.2 / 37.2, 27
+// (20^3) 34.6 / 35.8, 125 (32^3) 44.7 / 55.2, 512 (32^3) 80.4 / 116, 4096 (32^3)
+// 325 / 676; FP32 the same within 1 us up to 64, 512 64.5 / 93.1.
+constexpr int kFuseChildren = 16;
 
 // ---- coarse correction with the first post-smoothing step (kernels_smooth.cu) ----
 // After the coarse solve e, the post-smoother starts from x_0 = x + P e and

@@ -223,6 +223,7 @@ struct Level {
   int32_t* cptr = nullptr;
   int32_t* cidx = nullptr;
   int64_t nc = 0;
+  int cmax = 0;  // rows of the largest aggregate
   // general prolongator (not one unit entry per row): P (n x nc) and R = P^T
   // (nc x n), FP64 values, explicit SELL-32 slices
   bool xfer_general = false;
@@ -1097,7 +1098,7 @@ struct Engine {
   // Whether the residual, the restriction and the next level's first step run
   // as one kernel (see RestrictArgs).
   static bool fuse_restrict(const amgps_ctx* c, const Level& L) {
-    return !rec() && !L.xfer_general && L.split == 1 && L.n <= kFuseRows &&
+    return !rec() && !L.xfer_general && L.split == 1 && L.n <= kFuseRows && L.cmax <= kFuseChildren &&
            !(c->nvec == 1 && level_uses_tma(c, L));
   }
 
@@ -2609,6 +2610,7 @@ void load_levels(amgps_ctx* c, int n_levels, const amgps_csr* A, const amgps_csr
     }
     for (int64_t I = 0; I < nc; ++I) {
       REQ(cptr[I + 1] > 0, AMGPS_E_ARG, "P has an empty aggregate (zero column)");
+      L.cmax = std::max(L.cmax, cptr[I + 1]);
       cptr[I + 1] += cptr[I];
     }
     std::vector<int32_t> fill(cptr.begin(), cptr.end() - 1);
