@@ -34,6 +34,14 @@ __device__ __forceinline__ void pdl_wait() {
 __device__ __forceinline__ void pdl_go() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// For kernels that only stream vectors, one row a thread: of one resident wave
+// (eight blocks on each SM) or less.  The instruction costs 0.37 ns a block, one
+// block after another, and beyond a wave that is more than a start under such a
+// kernel's tail gives: 2.1 million rows (8192 blocks) 9.1 us with it, 5.3
+// without, 8.2 as an ordinary launch; one FP32 step on 128^3 30.3 / 19.5 / 24.9 us.
+__device__ __forceinline__ void pdl_go_one_wave() {
+  if (gridDim.x * gridDim.y <= 8 * 152) pdl_go();
+}
 
 // Load of a vector entry.  CG = false: a plain cached load, issued where it
 // stands (volatile: neither the compiler nor the read-only path may move it

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kBlock) k_first(int64_t n, const XT* b,
   if (i >= n) return;
   const XT di = dinv[i];
   pdl_wait();
-  pdl_go();
+  pdl_go_one_wave();
   const int64_t o = (int64_t)blockIdx.y * n;  // vector of a batch
   first_row<XT, FAM>(i, b + o, di, rout + o, zout + o, xout + o, c2, beta, rhoinv);
 }
@@ -583,7 +583,7 @@ template <class A, class B>
 __global__ void __launch_bounds__(kBlock) k_convert(int64_t n, const A* in, B* out) {
   const int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   pdl_wait();
-  pdl_go();
+  pdl_go_one_wave();
   if (i < n) out[i] = B(in[i]);
 }
 
