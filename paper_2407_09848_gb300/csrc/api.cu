@@ -1817,8 +1817,8 @@ void fcg1_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit,
 // the same.
 bool loop_fp32(const amgps_ctx* c) { return c->prec != AMGPS_F64 && c->flexible != 2; }
 
-// The first step of level 0's smoother as part of the r update (level 0 not
-// the coarsest, not the one-reduction form, and not where it would overwrite
+// The first step of level 0's smoother as part of the r update (not in the
+// one-reduction form, and not where it would overwrite
 // the z that the flexible form still needs); r and x: the V-cycle's boundary
 // vectors.  BF16 192^3 solve 77.5 -> 75.4 ms, 32^3 778 -> 766 us.
 template <class VT, class XT>
@@ -1826,7 +1826,7 @@ RFirst<XT> loop_first(amgps_ctx* c, XT* r, XT* x) {
   RFirst<XT> f;
   const Level& L = c->lv[0];
   if constexpr (sizeof(XT) == 4) f.fout = r;
-  if (L.coarsest || c->flexible == 2) return f;
+  if (c->flexible == 2) return f;
   const Coefs cf = make_coefs(L.spec.kind, L.spec.k, L.spec.w, L.spec.rho);
   const auto g = Engine<VT, XT>::first_of(c, L, cf, x);
   if (c->flexible == 1 && g.x == x) return f;
@@ -2019,8 +2019,11 @@ void pcg_impl(amgps_ctx* c, const double* b, double* x, double rtol, int maxit, 
                       same_coefs(L.ops_cf, make_coefs(L.spec.kind, L.spec.k, L.spec.w, L.spec.rho));
   // The loop on the device, unless the kernels are being timed (events between
   // them), the caller captures the stream, or the coarse levels run as a
-  // cooperative kernel; a caller's preconditioner keeps the host loop.
-  if (!precond && !c->prof && !c->use_cycle && !Engine<double, double>::capturing(c) &&
+  // cooperative kernel; a caller's preconditioner keeps the host loop.  So does a
+  // single level: its dense solve leaves an iteration or two, which cost less
+  // than the loop's start (216 rows: 65 us, flexible 64, against 75 and 85).
+  if (!precond && !c->prof && !c->use_cycle && !L.coarsest &&
+      !Engine<double, double>::capturing(c) &&
       build_loop(c)) {
     pcg_loop(c, b, x, rtol, maxit, iters, relres, converged);
     return;
