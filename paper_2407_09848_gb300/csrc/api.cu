@@ -1564,7 +1564,7 @@ void check_kind_degree(int kind, int degree) {
 constexpr int64_t kOpMinRows = 1 << 17;
 bool op_level(const amgps_ctx* c, const Level& L) {
   return c->prec == AMGPS_F64 && L.sval && !L.coarsest && L.split == 1 &&
-         split_for(L.stored, L.nslices, false) == 1 && L.n >= kOpMinRows;
+         split_for(L.stored, L.nslices, false, L.wmax) == 1 && L.n >= kOpMinRows;
 }
 
 // M^{-1} A P of every FP64 aggregation level with rows of at most eight stored
@@ -2347,7 +2347,7 @@ void load_general_transfer(amgps_ctx* c, Level& L, const amgps_csr& P) {
   const amgps_csr R{nc, n, P.nnz, rptr.data(), rcol.data(), rval.data()};
   auto put = [&](const amgps_csr& M, DevMat<double>& d, int& split) {
     HostSell h = build_sell(M, false);
-    split = split_for(h.stored, h.nslices, c->prec == AMGPS_F64);
+    split = split_for(h.stored, h.nslices, c->prec == AMGPS_F64, widest(h));
     d.n = M.n_rows;
     d.nslices = h.nslices;
     d.sd = dupload(c, h.sd.data(), h.sd.size());
@@ -2518,11 +2518,11 @@ void load_levels(amgps_ctx* c, int n_levels, const amgps_csr* A, const amgps_csr
       // SpMV of a single-level hierarchy and for l1-Jacobi coarse sweeps
     }
     HostSell h = build_sell(A[l]);
-    L.split = split_for(h.stored, h.nslices, prec == AMGPS_F64);
+    L.wmax = widest(h);
+    L.split = split_for(h.stored, h.nslices, prec == AMGPS_F64, L.wmax);
     L.nslices = h.nslices;
     L.stored = h.stored;
     L.explicit_entries = h.explicit_entries;
-    for (const SliceDesc& d : h.sd) L.wmax = std::max(L.wmax, (int)d.w);
     L.sd = dupload(c, h.sd.data(), h.sd.size());
     if (h.off.empty()) h.off.push_back(0);  // every slice explicit: keep a valid pointer
     L.off = dupload(c, h.off.data(), h.off.size());

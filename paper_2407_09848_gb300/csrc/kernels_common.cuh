@@ -88,8 +88,11 @@ __device__ __forceinline__ SliceDesc ld_desc(const SliceDesc* p) {
 // few thousand rows, where a kernel is three dependent loads long, that is
 // most of its time.  Rows of other lengths go NB entries at a time; PIPE (the
 // kernels of wide rows): the next NB values and columns are fetched while the
-// current products are formed.
-template <int SIGN, class VT, class XT, bool CG, bool WAIT, int NB, bool PIPE, class Init>
+// current products are formed.  U8 (the split step): rows of a uniform slice,
+// which load no columns, go eight at a time instead (FP64, 100,000 rows of 251
+// in a band, 4 warps a slice, four steps and the call: 258 -> 226 us).
+template <int SIGN, class VT, class XT, bool CG, bool WAIT, int NB, bool PIPE, bool U8 = false,
+          class Init>
 __device__ __forceinline__ XT row_accumulate(const DevMat<VT>& A, const SliceDesc d, int lane,
                                              int64_t row, const XT* u, Init init, int k0, int k1) {
   const int64_t nm1 = A.n - 1;
@@ -122,33 +125,41 @@ __device__ __forceinline__ XT row_accumulate(const DevMat<VT>& A, const SliceDes
     for (int kk = 0; kk < 7; ++kk) t = fma(SIGN > 0 ? a[kk] : -a[kk], uv[kk], t);
     return t;
   }
-  XT a[NB];
-  int32_t c[NB];
-  auto fetch_batch = [&](int kb) {
+  auto batches = [&](auto nb, auto pipe) {
+    constexpr int N = decltype(nb)::value;
+    constexpr bool kAhead = decltype(pipe)::value;
+    XT a[N];
+    int32_t c[N];
+    auto fetch_batch = [&](int kb) {
 #pragma unroll
-    for (int kk = 0; kk < NB; ++kk)
-      if (kb + kk < k1) fetch(kb + kk, a[kk], c[kk]);
-  };
-  fetch_batch(k0);
-  if constexpr (WAIT) {
-    pdl_wait();
-    pdl_go();
-  }
-  XT t = init();
-  for (int kb = k0; kb < k1; kb += NB) {
-    XT av[NB], uv[NB];
-#pragma unroll
-    for (int kk = 0; kk < NB; ++kk) {
-      if (kb + kk < k1) uv[kk] = ldv<CG>(u + c[kk]);
-      av[kk] = a[kk];
+      for (int kk = 0; kk < N; ++kk)
+        if (kb + kk < k1) fetch(kb + kk, a[kk], c[kk]);
+    };
+    fetch_batch(k0);
+    if constexpr (WAIT) {
+      pdl_wait();
+      pdl_go();
     }
-    if (PIPE && kb + NB < k1) fetch_batch(kb + NB);
+    XT t = init();
+    for (int kb = k0; kb < k1; kb += N) {
+      XT av[N], uv[N];
 #pragma unroll
-    for (int kk = 0; kk < NB; ++kk)
-      if (kb + kk < k1) t = fma(SIGN > 0 ? av[kk] : -av[kk], uv[kk], t);
-    if (!PIPE && kb + NB < k1) fetch_batch(kb + NB);
+      for (int kk = 0; kk < N; ++kk) {
+        if (kb + kk < k1) uv[kk] = ldv<CG>(u + c[kk]);
+        av[kk] = a[kk];
+      }
+      if (kAhead && kb + N < k1) fetch_batch(kb + N);
+#pragma unroll
+      for (int kk = 0; kk < N; ++kk)
+        if (kb + kk < k1) t = fma(SIGN > 0 ? av[kk] : -av[kk], uv[kk], t);
+      if (!kAhead && kb + N < k1) fetch_batch(kb + N);
+    }
+    return t;
+  };
+  if constexpr (U8) {
+    if (d.cref >= 0) return batches(std::integral_constant<int, 8>{}, std::false_type{});
   }
-  return t;
+  return batches(std::integral_constant<int, NB>{}, std::integral_constant<bool, PIPE>{});
 }
 
 // The same sum with the entries of a row shared by E lanes of a warp: lane

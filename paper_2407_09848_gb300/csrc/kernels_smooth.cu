@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_step_split(const StepArgs<VT
   const XT di = (own && step_needs_dinv<FAM>()) ? __ldg(a.dinv + row) : XT(0);
   const SliceDesc d = ld_desc(a.A.sd + s);
   const int k0 = (int)((int64_t)d.w * g / G), k1 = (int)((int64_t)d.w * (g + 1) / G);
-  part[g][lane] = row_accumulate<F::kSign, VT, XT, false, true, 4, true>(
+  part[g][lane] = row_accumulate<F::kSign, VT, XT, false, true, 4, true, sizeof(VT) == 8>(
       a.A, d, lane, row, a.u + o,
       [&] {
         if (!own) return XT(0);

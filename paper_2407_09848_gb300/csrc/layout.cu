@@ -81,31 +81,57 @@ void require_positive_diagonal(const amgps_csr& A) {
   });
 }
 
+int widest(const HostSell& h) {
+  int w = 0;
+  for (const SliceDesc& d : h.sd) w = std::max(w, (int)d.w);
+  return w;
+}
+
 // Warps per slice for the split kernels: 1 while rows average under 24 stored
 // entries, at least 8 entries a warp, at most kMaxSplit.
 // FP64 rows: the largest power of two that keeps the level in one resident wave
-// (kWaveWarps: 32 warps of 64 registers on each SM).  The kernels fetch ahead,
+// (kWaveWarps: 32 warps of 64 registers on each SM; a fixed number, so that the
+// order of summation does not depend on the device).  The kernels fetch ahead,
 // so a wave of long rows is bound by FP64 issue, and every further wave pays
 // its first three loads again (four steps and the call, 96^3 smoothed
 // aggregation: 3456 slices of 32 entries 60.4 us with 4 warps a slice, 53.4
-// with 1; 432 of 165 entries 49.6 with 16, 42.5 with 8).
+// with 1; 432 of 165 entries 49.6 with 16, 42.5 with 8).  Two exceptions:
+// - waves that are less than three quarters full, with rows long enough for it
+//   (30 entries a warp): the most warps within 2.6 waves (bands, four steps and
+//   the call: 3125 slices of 251 entries 286 us with 1 warp, 226 with 4; 1563 of
+//   500 294 with 2, 231 with 8; 6250 of 125 262 with 1, 225 with 2);
+// - a slice much wider than the rest (a dense row), whose warps would run on
+//   alone: one entry of a chain takes as long as 50,000 entries of the level
+//   (20,000 rows of 251 on average, irregular: 198 us with 4 warps, 144 with 8).
 // FP32 rows keep the rule their order of summation was fixed by (measured on the
 // 256^3 levels, kernels that did not fetch ahead): the larger of a width term
 // (the power of two nearest avg / 32 once avg >= 48) and a parallelism term (the
 // power of two at or below 24576 / slices).
-int split_for(int64_t stored, int64_t nslices, bool f64) {
-  constexpr double kWaveWarps = 32 * 152;
+int split_for(int64_t stored, int64_t nslices, bool f64, int wmax) {
+  constexpr double kWaveWarps = 32 * 152, kMostWarps = 24576.0;
   if (nslices == 0) return 1;
-  const double avg = (double)stored / ((double)nslices * kSlice);
+  const double avg = (double)stored / ((double)nslices * kSlice), n = (double)nslices;
   if (avg < 24.0) return 1;
+  auto within = [&](double warps) {  // the largest power of two
+    int g = 1;
+    while (g < kMaxSplit && 2.0 * g * n <= warps) g *= 2;
+    return g;
+  };
   int cap = 1;
   while (cap < kMaxSplit && 2.0 * cap <= avg / 8.0) cap *= 2;
-  const double most = f64 ? kWaveWarps : 24576.0;
-  int g1 = 1, g2 = 1;
-  if (!f64 && avg >= 48.0)
-    while (g1 < kMaxSplit && 2.0 * g1 <= avg / 32.0 * 1.41421356) g1 *= 2;
-  while (g2 < kMaxSplit && 2.0 * g2 <= most / (double)nslices) g2 *= 2;
-  return std::max(1, std::min(std::max(g1, g2), cap));
+  if (!f64) {
+    int g = 1;
+    if (avg >= 48.0)
+      while (g < kMaxSplit && 2.0 * g <= avg / 32.0 * 1.41421356) g *= 2;
+    return std::min(std::max(g, within(kMostWarps)), cap);
+  }
+  int g = within(kWaveWarps);
+  const double waves = g * n / kWaveWarps;
+  const int more = within(2.63 * kWaveWarps);
+  if (waves < 0.75 * std::ceil(waves) && avg >= 30.0 * more) g = more;
+  while (2 * g <= cap && 2.0 * g * n <= kMostWarps && (double)wmax / g > (double)stored / 50000.0)
+    g *= 2;
+  return std::min(g, cap);
 }
 
 

@@ -46,8 +46,10 @@ void validate_csr(const amgps_csr& A, const char* what, bool square);
 // validated square CSR)
 void require_positive_diagonal(const amgps_csr& A);
 // Warps per slice for the split kernels of a level (1: no split)
-// (f64: FP64 vectors)
-int split_for(int64_t stored, int64_t nslices, bool f64);
+// (f64: FP64 vectors, which also look at wmax, the entries of the widest slice)
+int split_for(int64_t stored, int64_t nslices, bool f64, int wmax);
+// stored entries of the widest slice
+int widest(const HostSell& h);
 // SELL-32 form of A; allow_uniform = false keeps every slice explicit
 HostSell build_sell(const amgps_csr& A, bool allow_uniform = true);
 // FP64 -> BF16 bits, round to nearest even directly from the double
