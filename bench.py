@@ -597,6 +597,27 @@ def step_hbm_roofline(n_step, ms_step, by_step, traffic=None, kernel=None):
             "bytes_per_launch": by_step / max(n_step, 1), "peak_source": peak_src}
 
 
+def issued_work(k, form, launches, flops, inst, n, nnz, stored, h, g):
+    """(flops, FP64 thread instructions) that the level-0 step launches of FP64
+    V-cycles (4th kind, degree k, 2 k - 1 launches a cycle) do, from the counts of
+    the method's plain steps.  h, g: vector-term coefficients of the stored-operator
+    steps (amgps_op_coefs).
+    - The first post-smoothing step runs with the coarse correction: (1/M) r, four
+      products, x + e and the x update, 7 instructions and 12 flops a row; the
+      recurrence form also scales z.
+    - Stored-operator steps are scaled so that a vector term of coefficient 1 starts
+      the sum: the s_0 term of the middle steps, and for k = 4 the u_3 term of the
+      last step from zero, one multiply less each."""
+    cycles = launches / (2 * k - 1)
+    if form == 1 and k >= 2:
+        fine = [1e-3 <= abs(v) <= 1e3 for v in h]
+        saved = 2 * sum(fine[1:k - 2]) + (1 if k == 4 and 1e-3 <= abs(g[2]) <= 1e3 else 0)
+        wt = 1 if k >= 3 else 0
+        return (flops - cycles * (saved * n + 2 * nnz + 2 * wt * n - 12 * n),
+                inst - cycles * (saved * n + stored + wt * n - 7 * n))
+    return (flops - cycles * (2 * nnz + 4 * n - 13 * n), inst - cycles * (stored + 3 * n - 8 * n))
+
+
 def committed_traffic(workload, prec, step_form=1):
     """ncu DRAM bytes per launch of the level-0 step from the committed capture,
     when it was taken on the current sources of the step kernels in the same
@@ -671,31 +692,28 @@ def run_ours(a):
     hbm["share_of_solve_time"] = (ms_step / nprof) / ms_per if ms_per else None
     roof = hbm
     if a.prec == "f64" and a.kind in ("cheb4", "cheb4_opt", "weights") and n_step:
-        # FP64 path: the step is bound by the FP64 pipe.  Flops per launch: the
-        # library's algorithmic count over the profiled level-0 steps
-        # (amgps_profile_flops: a multiply-add 2, a lone multiply 1, 2 per
-        # nonzero for the products), averaged per launch.  In the
-        # stored-operator form a k = 4 cycle's seven level-0 steps total
-        # 14 nnz + 7 n (2 nnz + n per launch); the recurrence form's are
-        # 2 nnz + 5 n per launch.  These are the plain steps of the method: the
-        # scaled steps and the first post-smoothing step (which runs with the
-        # coarse correction, four products a row) need up to a tenth fewer
-        # instructions than they count for.  Peak: 304 FP64 FMA thread-instructions per
-        # clock (152 SMs x 2, ncu peak_sustained) x 2 flops x the SM clock
-        # sampled during the profiled pass.
-        fl = prof["step_flops"] / n_step
+        # FP64 path: the step is bound by the FP64 pipe.  Rate and fractions are
+        # of the work that the launches do (issued_work); the method's plain
+        # steps (amgps_profile_flops) and their rate stand beside them.  Peak: 304
+        # FP64 FMA thread-instructions per clock (152 SMs x 2, ncu peak_sustained)
+        # x 2 flops x the SM clock sampled during the profiled pass.
+        from paper_2407_09848_gb300.amgps import op_coefs, opt4_weights
+        nnz, stored = S.level_info(0)[1:]
+        w = opt4_weights(a.degree) if a.kind == "cheb4_opt" else None
+        h, g = op_coefs(a.kind, a.degree, w)[2:] if a.degree >= 2 else ([], [])
+        fl, inst = issued_work(a.degree, a.step_form, n_step, prof["step_flops"],
+                               prof["step_fp64_inst"], n, nnz, stored, h, g)
+        fl, inst, plain = fl / n_step, inst / n_step, prof["step_flops"] / n_step
         mhz = clk_prof.get("sm_mhz") or 2070.0
         fpeak = 304 * 2 * mhz * 1e6 / 1e12
-        fach = fl / (1e-3 * ms_step / n_step) / 1e12
-        # FP64 issue: thread instructions of the plain steps (one per stored
-        # entry and per vector term) against 304 per clock; a lone multiply is
-        # one flop but a whole issue slot
-        inst = prof["step_fp64_inst"] / n_step
-        issue = inst / (1e-3 * ms_step / n_step) / (304 * mhz * 1e6)
-        roof = {"bound": "alu", "achieved": fach, "peak": fpeak, "unit": "TFLOP/s",
-                "frac": fach / fpeak, "traffic": traffic, "kernel": hbm["kernel"],
+        sec = 1e-3 * ms_step / n_step
+        # FP64 issue: thread instructions against 304 per clock; a lone multiply
+        # is one flop but a whole issue slot
+        roof = {"bound": "alu", "achieved": fl / sec / 1e12, "peak": fpeak, "unit": "TFLOP/s",
+                "frac": fl / sec / 1e12 / fpeak, "traffic": traffic, "kernel": hbm["kernel"],
                 "flops_per_launch": fl, "fp64_inst_per_launch": inst,
-                "fp64_issue_frac": issue,
+                "fp64_issue_frac": inst / sec / (304 * mhz * 1e6),
+                "method_flops_per_launch": plain, "method_tflops": plain / sec / 1e12,
                 "peak_source": "derived: 2 FP64 FMA/clk/SM x 152 SMs x 2 flops x sampled SM clock",
                 "launches": n_step, "avg_launch_us": hbm["avg_launch_us"],
                 "share_of_solve_time": hbm["share_of_solve_time"], "hbm": hbm}

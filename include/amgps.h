@@ -155,7 +155,10 @@ amgps_status amgps_level_info(amgps_ctx* ctx, int level, int64_t* n, int64_t* nn
  * level).  degree in 1..16.  `weights` (host, `degree` doubles) is read only for
  * AMGPS_WEIGHTS and copied.  `rho` scales the spectral interval: the smoother
  * uses rho in place of rho(M^{-1}A) (CHEB1, CHEB4, WEIGHTS, CHEB4_OPT);
- * rho <= 0 means 1.  Synchronous host bookkeeping only. */
+ * rho <= 0 means 1.  Host bookkeeping, and on levels that AMGPS_OPT_STEP_FORM
+ * names the operators, formed on the device.  Graphs that the library keeps of
+ * the V-cycle and of a solve are built again by the next such call if the
+ * smoother changed. */
 amgps_status amgps_set_smoother(amgps_ctx* ctx, int level, amgps_kind kind, int degree,
                                 const double* weights, double rho);
 
@@ -329,6 +332,20 @@ amgps_status amgps_synchronize(amgps_ctx* ctx);
  * allocator, so a caller can reject a problem that would not fit its memory
  * share.  Any failed amgps_hierarchy_load leaves no hierarchy loaded and
  * keeps none of its buffers.
+ * Within the limit a load also forms what only makes a hierarchy faster: on
+ * FP64 hierarchies the matrices of the coarse corrections (36 bytes a row of
+ * the levels that have one) and of the coarse sweeps (up to 8 MB).  Where a
+ * later call finds no room for its own buffers or for the operators of
+ * AMGPS_OPT_STEP_FORM, they are given back if that is enough, and formed again
+ * with a later amgps_set_smoother (corrections) or AMGPS_OPT_COARSE_SWEEPS.
+ * Once the caller has captured a call on a hierarchy into a CUDA graph of its
+ * own they stay, since that graph reads them, and the later call fails or does
+ * without.  (A caller's graph holds the smoothers' scalars of its capture but
+ * reads the operators that amgps_set_smoother writes: capture again after it.)
+ * Outside the limit: scratch of the set-up calls and of batches of vectors
+ * (amgps_vcycle_loss_grad, amgps_error_cycles), from a pool per device that
+ * the contexts of the process share.  It keeps at most 1 GiB between calls, to
+ * which other allocations come first, and nothing after the last context.
  * AMGPS_OPT_STEP_FORM (default 1): how the smoothers of degree >= 2 (every
  * kind) run on FP64 levels of at least 131,072 rows that the step kernel
  * evaluates one warp per 32-row slice (every level whose rows average fewer

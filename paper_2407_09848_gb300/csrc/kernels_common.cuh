@@ -637,6 +637,8 @@ __device__ __forceinline__ void grid_sum(double v, const RedWork& w, Fin fin) {
 // warp instruction in 16 clocks, so the eight warps of a block take eight
 // times one warp's time (4096-row level: 0.5 us of FP64 issue on 16 SMs, 0.06
 // on 128).
+// (GB300's SMs as a fixed number: it also decides how many lanes share a wide
+// row, and with that an order of summation, which is not the device's affair.)
 constexpr int kSms = 152;
 inline int small_block(int64_t threads) {
   const int64_t warps = (threads + 31) / 32, per = (warps + kSms - 1) / kSms;
