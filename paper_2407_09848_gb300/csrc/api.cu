@@ -2925,8 +2925,8 @@ amgps_status amgps_error_cycles(amgps_ctx* c, double* E, int m, int cycles) {
     }
     if (bt) {
       CK(cudaMemsetAsync(bt->rw.counter, 0, B * sizeof(unsigned), s));
-      for (int i = 0; i < m; i += B) {
-        const int nv = std::min(B, m - i);
+      for (int64_t i = 0; i < m; i += B) {
+        const int nv = (int)std::min<int64_t>(B, m - i);
         bt->size(nv);
         double* e = E + (size_t)i * n;
         for (int q = 0; q < cycles; ++q) {
